@@ -95,9 +95,12 @@ const char* alp_status_string(alp_status s);
  * Native FP64 GEMM, Eq. 1 (Sect. 2, Fig. 2): TMA-staged A and B tiles in a
  * multi-stage mbarrier ring, FP64 DMMA tensor-core MMAs into per-thread
  * register tiles, alpha/beta epilogue.  cfg == NULL selects the config from the
- * tuned cache, else the loaded cost model, else the built-in default.
- * Operands whose base address is not 16-byte aligned, or whose lda/ldb is odd,
- * run through a non-TMA variant of the same kernel.
+ * tuned cache, else the loaded cost model; without either the call runs the
+ * register-direct kernels, which cut the work evenly over the SMs for any
+ * shape, alignment and leading dimension (a k range may be shared by a
+ * cluster's blocks, its partial sums added in a fixed order).
+ * With a config, operands whose base address is not 16-byte aligned, or whose
+ * lda/ldb is odd, run through a non-TMA variant of the same kernel.
  * Returns ALP_ERR_INVALID_ARG for negative sizes, ld < row width, NULL
  * operands that would be read, or an invalid cfg.
  */
@@ -107,11 +110,13 @@ alp_status alp_gemm_f64(int64_t M, int64_t N, int64_t K, double alpha,
                         const alp_config* cfg, void* stream);
 /* Transposed operands for the native GEMM: C = alpha op(A) op(B) + beta C with
  * op(X) = X (trans 0) or X^T (trans 1), storage as for alp_gemm_f64_emul_ex.
- * A transposed operand is first packed row-major into `workspace` (one read
- * and one write of it, small against the 2 M N K FP64 flops), then the product
- * runs as alp_gemm_f64 with `cfg`; results are bit-identical to alp_gemm_f64
- * on the transposed matrices.  workspace >= alp_gemm_f64_ex_workspace(...),
- * 256-byte aligned (none needed, and none read, when neither is transposed). */
+ * With a config (as alp_gemm_f64 selects it) a transposed operand is first
+ * packed row-major into `workspace` (one read and one write of it, small
+ * against the 2 M N K FP64 flops), then the product runs as alp_gemm_f64 with
+ * it; without one the operands are read where they are.  Results are
+ * bit-identical to alp_gemm_f64 on the transposed matrices either way.
+ * workspace >= alp_gemm_f64_ex_workspace(...), 256-byte aligned (none needed,
+ * and none read, when neither is transposed). */
 alp_status alp_gemm_f64_ex(int trans_a, int trans_b, int64_t M, int64_t N, int64_t K,
                            double alpha, const double* A, int64_t lda, const double* B,
                            int64_t ldb, double beta, double* C, int64_t ldc,

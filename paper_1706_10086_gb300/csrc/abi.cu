@@ -22,9 +22,12 @@ alp_status native_transpose(const double* X, int64_t R, int64_t Cn, int64_t ldx,
                             int64_t ldo, cudaStream_t stream);
 alp_status native_scale(int64_t M, int64_t N, double beta, double* C, int64_t ldc,
                         cudaStream_t stream);
-// tune.cu: tuned cache, then cost model, then default.
-bool select_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
-                   cudaStream_t stream);
+alp_status native_direct(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
+                         const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
+                         double* C, int64_t ldc, cudaStream_t stream);
+// tune.cu: tuned cache, then cost model; false when neither has a config.
+bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
+                  cudaStream_t stream);
 
 // ----------------------------------------------------------------------------
 // Per-device state.
@@ -142,6 +145,8 @@ alp_status make_tmap_3d_bf16(CUtensorMap* map, const void* base, uint64_t d0, ui
 }
 
 // The autotuner's pick for 8192^3 on GB300 (0.997 of the measured DMMA peak).
+// A call without a config takes it only while the fault-injection hook is on:
+// the kernel it otherwise runs (native_direct.cu) has no device-side waits.
 static bool default_native_config(alp_config* out) {
     *out = alp_config{64, 128, 64, 4, 4, 0};
     return true;
@@ -195,6 +200,18 @@ const char* alp_status_string(alp_status s) {
     return "unknown alp_status";
 }
 
+// The tile config of a native call: the caller's, a tuned one, or the default
+// while the fault-injection hook is on.  False: none, native_direct runs.
+static bool pick_config(int64_t M, int64_t N, int64_t K, const alp_config* cfg, alp_config* c,
+                        cudaStream_t s) {
+    if (cfg) {
+        *c = *cfg;
+        return true;
+    }
+    if (tuned_config(M, N, K, ALP_PATH_NATIVE, c, s)) return true;
+    return inject_skip_kt() >= 0 && default_config(ALP_PATH_NATIVE, c);
+}
+
 alp_status alp_gemm_f64(int64_t M, int64_t N, int64_t K, double alpha, const double* A,
                         int64_t lda, const double* B, int64_t ldb, double beta, double* C,
                         int64_t ldc, const alp_config* cfg, void* stream) {
@@ -203,13 +220,11 @@ alp_status alp_gemm_f64(int64_t M, int64_t N, int64_t K, double alpha, const dou
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (alpha == 0.0 || K == 0) return native_scale(M, N, beta, C, ldc, s);
     alp_config c;
-    if (cfg) {
-        c = *cfg;
-        if (!native_config_valid(c.bm, c.bn, c.bk, c.tm, c.tn, c.stages)) return ALP_ERR_INVALID_ARG;
-    } else if (!select_config(M, N, K, ALP_PATH_NATIVE, &c, s)) {
-        default_config(ALP_PATH_NATIVE, &c);
-    }
+    const bool have = pick_config(M, N, K, cfg, &c, s);
+    if (cfg && !native_config_valid(c.bm, c.bn, c.bk, c.tm, c.tn, c.stages))
+        return ALP_ERR_INVALID_ARG;
     if (M > 0x7fffffffLL || N > 0x7fffffffLL || K > 0x7fffffffLL) return ALP_ERR_UNSUPPORTED;
+    if (!have) return native_direct(0, 0, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
     // TMA wants 16-byte aligned bases and row strides that are multiples of 16 bytes.
     const bool tma_ok = (((uintptr_t)A & 15) == 0) && (((uintptr_t)B & 15) == 0) &&
                         (lda % 2 == 0) && (ldb % 2 == 0);
@@ -268,9 +283,20 @@ alp_status alp_gemm_f64_ex(int trans_a, int trans_b, int64_t M, int64_t N, int64
     if (!workspace || workspace_bytes < ba + bb || ((uintptr_t)workspace & 255))
         return ALP_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // the transposed operands are packed row-major into the workspace (one
-    // read and one write of 8 bytes per element, against 2 M N K flops of
-    // FP64 DMMA work), then the product runs as alp_gemm_f64
+    // a pack's grid has at most 65535 x 32 rows of each transposed operand
+    if ((trans_a && K > 65535LL * 32) || (trans_b && N > 65535LL * 32)) return ALP_ERR_UNSUPPORTED;
+    alp_config c;
+    if (!pick_config(M, N, K, cfg, &c, s)) {
+        // without a tile config nothing is packed: the operands are read
+        // where they are (1021 x 771 x 1333 with A transposed, odd leading
+        // dimensions: 3150 us with the pack and the shared-memory kernel,
+        // 1960 this way)
+        if (M > 0x7fffffffLL || N > 0x7fffffffLL || K > 0x7fffffffLL) return ALP_ERR_UNSUPPORTED;
+        return native_direct(trans_a, trans_b, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
+    }
+    // with one, the transposed operands are packed row-major into the
+    // workspace (one read and one write of 8 bytes per element, against 2 M N K
+    // flops of FP64 DMMA work), then the product runs as alp_gemm_f64
     char* ws = static_cast<char*>(workspace);
     const double* Aop = A;
     const double* Bop = B;

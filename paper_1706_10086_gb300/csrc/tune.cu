@@ -241,9 +241,9 @@ void cache_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_conf
 
 // Config of a GEMM issued with cfg == NULL: the tuned cache, else the cost
 // model's prediction (made once per shape and then cached; skipped while
-// `stream` is being captured, since the prediction synchronises), else the
-// default.
-bool select_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
+// `stream` is being captured, since the prediction synchronises).  False when
+// neither has one.
+bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                    cudaStream_t stream) {
     {
         std::lock_guard<std::mutex> lk(g_tmu);
@@ -260,7 +260,13 @@ bool select_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* o
         return true;
     }
     cudaGetLastError();
-    return default_config(path, out);
+    return false;
+}
+
+// The same, with the path's default config where there is no tuned one.
+bool select_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
+                   cudaStream_t stream) {
+    return tuned_config(M, N, K, path, out, stream) || default_config(path, out);
 }
 
 }  // namespace alp
