@@ -115,11 +115,14 @@ alp_status alp_tune_unload_model(void);
  * r = 0, 1, 2 for M <= 32, <= 64, larger and c likewise from N. */
 int alp_batched_class_of(int64_t M, int64_t N);
 
-/* Tile (bm x bn, K step bk) used for the problems of class `cls` (0..8):
- * bm, bn in {32, 64, 128}, bk in {16, 32, 64}; each tile runs on 8 warps with
- * a (bm/16) x (bn/16) register tile per thread.  Defaults: bm, bn = 32, 64,
- * 128 by class, bk = 32 for classes with a 32-wide side, else 16.  Process-wide
- * setting, read when a batched call is issued (or captured). */
+/* Tile (bm x bn, K step bk) of the problems of class `cls` (0..8): bm, bn in
+ * {32, 64, 128}, bk in {16, 32, 64}.  The persistent kernel's warps take 16 x 16
+ * units of a problem's C over its whole k, walking bm rows before the next 16
+ * columns; bn and bk do not change what it runs.  A problem's results are those
+ * of alp_gemm_f64 with any valid config, bit for bit (same order over k).
+ * Defaults: bm, bn = 32, 64, 128 by class, bk = 32 for classes with a 32-wide
+ * side, else 16.  Process-wide setting, read when a batched call is issued (or
+ * captured). */
 alp_status alp_batched_set_class_config(int cls, int bm, int bn, int bk);
 alp_status alp_batched_get_class_config(int cls, int* bm, int* bn, int* bk);
 

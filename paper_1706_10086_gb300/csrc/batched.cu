@@ -1,24 +1,30 @@
 // Batched variable-size native FP64 GEMM: thousands of independent problems
 // C_p = alpha_p A_p B_p + beta_p C_p in one persistent launch.
 //
-// 1. A one-block plan kernel classifies every problem by its tile class
-//    (row and column tile of 32, 64 or 128, from M and N), orders problems by
-//    class and then by K bucket, longest first, and writes the prefix sum of
-//    their tile counts: the device work list.  Everything it reads is device
-//    memory, so the call is stream-ordered and capturable in a CUDA graph.
-// 2. A persistent kernel (one block of 8 warps per SM) takes tiles from an
-//    atomic counter, finds each tile's problem by binary search in the prefix
-//    array, and runs the tile with the register tile of its class
-//    (tm = bm/16, tn = bn/16, the native kernel's DMMA building blocks, loads
-//    through cp.async since every problem has its own pointers).
+// 1. A one-block plan kernel orders the problems by K bucket, longest first,
+//    and by tile class within it (row and column tile of 32, 64 or 128, from M
+//    and N), and writes the prefix sum of their unit counts: the device work
+//    list.  Everything it reads is device memory, so the call is
+//    stream-ordered and capturable in a CUDA graph.
+// 2. In a persistent kernel every warp on its own takes units from an atomic
+//    counter, a unit being one 16 x 16 block of one problem's C over the whole
+//    of its k, finds the problem by binary search in the prefix array, and
+//    runs it with register-direct DMMA fragments (native_direct.cuh).
 //
-// The class -> (bm, bn, bk) table is runtime state (alp_batched_set_class_config)
-// so that an autotuner can set it per class.
+// The launch is bound by the FP64 MMA rate, so what counts is that no MMA is
+// spent on padding and that all sub-partitions end together: 16 x 8 fragments
+// outside a problem are skipped, and units are small and end with the
+// shortest k.  4096 problems of 16..1024 (1.11e11 flops: 101.3 ms at the MMA
+// rate, 106.9 with whole fragments): 108.6 ms; the class table's default tiles,
+// one 8-warp block per SM, took 153.6.
+//
+// The class -> (bm, bn, bk) table is runtime state (alp_batched_set_class_config).
+#include <algorithm>
 #include <cstdlib>
 #include <mutex>
 
 #include "alp_ext.h"
-#include "native.cuh"
+#include "native_direct.cuh"
 
 namespace alp {
 
@@ -26,7 +32,8 @@ namespace {
 
 constexpr int kClasses = 9;           // 3 row-tile x 3 column-tile sizes
 constexpr int kKBuckets = 16;         // floor(log2 K) buckets, longest first
-constexpr int kBatchedThreads = 256;  // 8 warps: (bm/(8 tm)) x (bn/(4 tn)) with tm = bm/16, tn = bn/16
+constexpr int kBatchedThreads = 128;  // warps work alone; four per block, one per sub-partition
+constexpr int kUnit = 16;             // rows and columns of C per unit of work
 constexpr int kPlanThreads = 1024;
 
 struct ClassTable {
@@ -60,14 +67,17 @@ struct BatchArgs {
 
 struct Plan {              // device workspace
     int32_t* key;          // [count] sort key per problem (-1: nothing to do)
-    int32_t* order;        // [count] problem ids in (class, K bucket desc) order
-    int64_t* prefix;       // [count + 1] exclusive tile prefix over `order`
-    int64_t* meta;         // [0] valid problems, [1] total tiles
-    unsigned long long* counter;   // tile counter of the persistent kernel
+    int32_t* order;        // [count] problem ids in (K bucket desc, class) order
+    int64_t* prefix;       // [count + 1] exclusive unit prefix over `order`
+    int64_t* meta;         // [0] valid problems, [1] total units
+    unsigned long long* counter;   // unit counter of the persistent kernel
 };
 
-__global__ void __launch_bounds__(kPlanThreads) batched_plan_kernel(BatchArgs a, Plan pl,
-                                                                   ClassTable tab) {
+__host__ __device__ __forceinline__ int64_t units_of(int64_t M, int64_t N) {
+    return ((M + kUnit - 1) / kUnit) * ((N + kUnit - 1) / kUnit);
+}
+
+__global__ void __launch_bounds__(kPlanThreads) batched_plan_kernel(BatchArgs a, Plan pl) {
     __shared__ int cnt[kClasses * kKBuckets];
     __shared__ int base[kClasses * kKBuckets];
     __shared__ int64_t chunk_sum[kPlanThreads];
@@ -82,7 +92,7 @@ __global__ void __launch_bounds__(kPlanThreads) batched_plan_kernel(BatchArgs a,
         int key = -1;
         if (M > 0 && N > 0) {
             const int kb = K > 0 ? 63 - __clzll((long long)K) : 0;
-            key = class_of(M, N) * kKBuckets + (kKBuckets - 1 - (kb < kKBuckets ? kb : kKBuckets - 1));
+            key = (kKBuckets - 1 - (kb < kKBuckets ? kb : kKBuckets - 1)) * kClasses + class_of(M, N);
             atomicAdd(&cnt[key], 1);
         }
         pl.key[p] = key;
@@ -102,19 +112,18 @@ __global__ void __launch_bounds__(kPlanThreads) batched_plan_kernel(BatchArgs a,
         if (key >= 0) pl.order[atomicAdd(&base[key], 1)] = (int32_t)p;
     }
     __syncthreads();
-    // exclusive prefix of tile counts along `order`, 1024 entries at a time
+    // exclusive prefix of unit counts along `order`, 1024 entries at a time
     const int64_t nvalid = pl.meta[0];
     if (tid == 0) carry = 0;
     __syncthreads();
     for (int64_t c0 = 0; c0 < nvalid; c0 += kPlanThreads) {
         const int64_t pos = c0 + tid;
-        int64_t tiles = 0;
+        int64_t units = 0;
         if (pos < nvalid) {
             const int32_t p = pl.order[pos];
-            const int c = class_of(a.M[p], a.N[p]);
-            tiles = ((a.M[p] + tab.bm[c] - 1) / tab.bm[c]) * ((a.N[p] + tab.bn[c] - 1) / tab.bn[c]);
+            units = units_of(a.M[p], a.N[p]);
         }
-        chunk_sum[tid] = tiles;
+        chunk_sum[tid] = units;
         __syncthreads();
         for (int off = 1; off < kPlanThreads; off <<= 1) {   // inclusive Hillis-Steele scan
             const int64_t v = tid >= off ? chunk_sum[tid - off] : 0;
@@ -122,7 +131,7 @@ __global__ void __launch_bounds__(kPlanThreads) batched_plan_kernel(BatchArgs a,
             chunk_sum[tid] += v;
             __syncthreads();
         }
-        if (pos < nvalid) pl.prefix[pos] = carry + chunk_sum[tid] - tiles;
+        if (pos < nvalid) pl.prefix[pos] = carry + chunk_sum[tid] - units;
         __syncthreads();
         if (tid == kPlanThreads - 1) carry += chunk_sum[tid];
         __syncthreads();
@@ -134,28 +143,16 @@ __global__ void __launch_bounds__(kPlanThreads) batched_plan_kernel(BatchArgs a,
     }
 }
 
-template <int TM, int TN>
-__device__ __forceinline__ void run_tile(const TileProblem& pr, int64_t m0, int64_t n0, int bm, int bn,
-                                         int bk, double* smem, bool vec2) {
-    tile_ldg<TM, TN>(pr, m0, n0, bm, bn, bk, smem, vec2);
-}
-
-// MAXT: the largest bm and bn the class table may hold.  With MAXT = 64 only
-// the register tiles up to 4 x 4 are compiled, which fit two blocks per SM;
-// with MAXT = 32 only 2 x 2, three blocks per SM.
-template <int MAXT>
-__global__ void __launch_bounds__(kBatchedThreads, MAXT <= 32 ? 3 : MAXT <= 64 ? 2 : 1)
-    batched_persistent_kernel(BatchArgs a, Plan pl, ClassTable tab) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ int64_t s_tile;
-    double* smem = reinterpret_cast<double*>(smem_raw);
+__global__ void __launch_bounds__(kBatchedThreads, 5)
+    batched_persistent_kernel(const __grid_constant__ BatchArgs a, const __grid_constant__ Plan pl,
+                              const __grid_constant__ ClassTable tab) {
+    const int lane = threadIdx.x & 31;
     const int64_t total = pl.meta[1];
     const int64_t nvalid = pl.meta[0];
     while (true) {
-        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(pl.counter, 1ull);
-        __syncthreads();
-        const int64_t t = s_tile;
-        __syncthreads();
+        int64_t t = 0;
+        if (lane == 0) t = (int64_t)atomicAdd(pl.counter, 1ull);
+        t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= total) break;
         // position: last pos with prefix[pos] <= t
         int64_t lo = 0, hi = nvalid - 1;
@@ -165,38 +162,26 @@ __global__ void __launch_bounds__(kBatchedThreads, MAXT <= 32 ? 3 : MAXT <= 64 ?
             else hi = mid - 1;
         }
         const int32_t p = pl.order[lo];
+        const int64_t M = a.M[p], N = a.N[p];
+        const double alpha = a.alpha[p];
+        const int64_t K = alpha == 0.0 ? 0 : a.K[p];
+        // units run down the rows of a tile-row (bm of the problem's class)
+        // before moving one unit-column right, for reuse of B's columns
+        const int64_t un = (N + kUnit - 1) / kUnit, um = (M + kUnit - 1) / kUnit;
+        const int64_t strip = tab.bm[class_of(M, N)] / kUnit;
         const int64_t local = t - pl.prefix[lo];
-        TileProblem pr;
-        pr.M = a.M[p];
-        pr.N = a.N[p];
-        pr.alpha = a.alpha[p];
-        pr.beta = a.beta[p];
-        pr.K = pr.alpha == 0.0 ? 0 : a.K[p];
-        pr.A = a.A[p];
-        pr.B = a.B[p];
-        pr.C = a.C[p];
-        pr.lda = a.lda[p];
-        pr.ldb = a.ldb[p];
-        pr.ldc = a.ldc[p];
-        const int c = class_of(pr.M, pr.N);
-        const int bm = tab.bm[c], bn = tab.bn[c], bk = tab.bk[c];
-        const int64_t tiles_n = (pr.N + bn - 1) / bn;
-        const int64_t m0 = (local / tiles_n) * bm, n0 = (local % tiles_n) * bn;
-        const bool vec2 = ((reinterpret_cast<uintptr_t>(pr.C) & 15) == 0) && (pr.ldc % 2 == 0);
-        const int tm = bm / 16, tn = bn / 16;
-#define ALP_BATCHED_CASE(x, y) \
-    if (tm == x && tn == y) run_tile<x, y>(pr, m0, n0, bm, bn, bk, smem, vec2);
-        if (MAXT <= 32) {
-            ALP_BATCHED_CASE(2, 2)
-        } else if (MAXT <= 64) {
-            ALP_BATCHED_CASE(2, 2) else ALP_BATCHED_CASE(2, 4) else ALP_BATCHED_CASE(4, 2)
-            else ALP_BATCHED_CASE(4, 4)
-        } else {
-            ALP_BATCHED_CASE(2, 2) else ALP_BATCHED_CASE(2, 4) else ALP_BATCHED_CASE(2, 8)
-            else ALP_BATCHED_CASE(4, 2) else ALP_BATCHED_CASE(4, 4) else ALP_BATCHED_CASE(4, 8)
-            else ALP_BATCHED_CASE(8, 2) else ALP_BATCHED_CASE(8, 4) else ALP_BATCHED_CASE(8, 8)
-        }
-#undef ALP_BATCHED_CASE
+        const int64_t first = local / (strip * un) * strip;
+        const int64_t rows = min(um - first, strip);
+        const int64_t rem = local % (strip * un);
+        const int64_t r0 = (first + rem % rows) * kUnit, c0 = rem / rows * kUnit;
+        double* C = a.C[p];
+        const int64_t ldc = a.ldc[p];
+        Acc<2, 4> acc;
+        acc.zero();
+        mma_direct<1, 2>(DirectOperand{a.A[p], a.lda[p], 1}, DirectOperand{a.B[p], 1, a.ldb[p]}, M,
+                         N, K, r0, c0, 0, (K + 3) >> 2, lane, acc);
+        const bool vec2 = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && ldc % 2 == 0;
+        epilogue<2, 4>(acc, C, ldc, M, N, r0, c0, alpha, a.beta[p], vec2, lane);
     }
 }
 
@@ -218,44 +203,15 @@ PlanLayout plan_layout(int64_t count) {
     return L;
 }
 
-// Largest bm or bn among the classes in `present` (bit c: class c has tiles).
-int max_tile(const ClassTable& t, unsigned present) {
-    int m = 0;
-    for (int c = 0; c < kClasses; ++c) {
-        if (!(present >> c & 1u)) continue;
-        m = t.bm[c] > m ? t.bm[c] : m;
-        m = t.bn[c] > m ? t.bn[c] : m;
-    }
-    return m;
-}
-
-int max_smem(const ClassTable& t) {
-    int m = 0;
-    for (int c = 0; c < kClasses; ++c) {
-        const int b = 2 * (t.bm[c] + t.bn[c]) * t.bk[c] * 8;
-        m = b > m ? b : m;
-    }
-    return m;
-}
-
-// The persistent kernel for `tiles` tiles on `sms` SMs, as many blocks as fit.
-// When the classes present use tiles of at most 64 x 64 (32 x 32) it runs the
-// variant that fits two (three) blocks per SM.
+// The persistent kernel for `units` units on `sms` SMs, as many blocks as fit.
 alp_status launch_persistent(const BatchArgs& a, const Plan& pl, const ClassTable& tab,
-                             int64_t tiles, unsigned present, int sms, cudaStream_t stream) {
-    const int smem = max_smem(tab);
-    const int mt = max_tile(tab, present);
-    auto kernel = mt <= 32   ? batched_persistent_kernel<32>
-                  : mt <= 64 ? batched_persistent_kernel<64>
-                             : batched_persistent_kernel<128>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return cuda_status(e);
+                             int64_t units, int sms, cudaStream_t stream) {
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kBatchedThreads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, batched_persistent_kernel,
+                                                  kBatchedThreads, 0);
     if (occ < 1) occ = 1;
-    int64_t grid = (int64_t)sms * occ;
-    if (grid > tiles) grid = tiles;
-    kernel<<<(unsigned)grid, kBatchedThreads, smem, stream>>>(a, pl, tab);
+    const int64_t grid = std::min<int64_t>((int64_t)sms * occ, (units + 3) / 4);
+    batched_persistent_kernel<<<(unsigned)grid, kBatchedThreads, 0, stream>>>(a, pl, tab);
     return cuda_status(cudaGetLastError());
 }
 
@@ -275,20 +231,15 @@ alp_status batched_launch(const BatchArgs& a, const int64_t* hM, const int64_t* 
     pl.meta = reinterpret_cast<int64_t*>(ws + L.off_meta);
     pl.counter = reinterpret_cast<unsigned long long*>(ws + L.off_counter);
     // grid size from the host copies (performance only: the persistent loop
-    // covers any number of tiles)
-    int64_t tiles = 0;
-    unsigned present = 0;
-    for (int64_t p = 0; p < a.count; ++p) {
-        if (hM[p] <= 0 || hN[p] <= 0) continue;
-        const int c = class_of(hM[p], hN[p]);
-        tiles += ((hM[p] + tab.bm[c] - 1) / tab.bm[c]) * ((hN[p] + tab.bn[c] - 1) / tab.bn[c]);
-        present |= 1u << c;
-    }
-    batched_plan_kernel<<<1, kPlanThreads, 0, stream>>>(a, pl, tab);
+    // covers any number of units)
+    int64_t units = 0;
+    for (int64_t p = 0; p < a.count; ++p)
+        if (hM[p] > 0 && hN[p] > 0) units += units_of(hM[p], hN[p]);
+    batched_plan_kernel<<<1, kPlanThreads, 0, stream>>>(a, pl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e);
-    if (tiles == 0) return ALP_OK;
-    return launch_persistent(a, pl, tab, tiles, present, sms, stream);
+    if (units == 0) return ALP_OK;
+    return launch_persistent(a, pl, tab, units, sms, stream);
 }
 
 }  // namespace alp
@@ -497,7 +448,7 @@ extern "C" alp_status alp_gemm_batched_varsize_noalloc(
     // The same launch as alp_gemm_batched_varsize with the scratch array as its
     // workspace (256-byte aligned, as a workspace must be).  The plan kernel
     // rewrites every part of it that it later reads (keys, order, prefix sums,
-    // counts, and the tile counter it sets to 0), so the previous call's
+    // counts, and the unit counter it sets to 0), so the previous call's
     // contents need no clearing.
     return batched_launch(a, hM, hN, scratch, reinterpret_cast<cudaStream_t>(stream), sms);
 }
