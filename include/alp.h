@@ -159,7 +159,8 @@ size_t alp_gemm_f64_emul_workspace(int64_t M, int64_t N, int64_t K, int nslices,
 
 /*
  * Stages of the emulated GEMM, exposed for testing and per-stage timing (the
- * same kernels alp_gemm_f64_emul launches, in this order).
+ * GEMM calls' results bit for bit, in this order; the calls themselves scan
+ * and split their operands in one launch where that is faster).
  * alp_emul_exponents: e[i] (int32, device) for the `rows` rows of a row-major
  * rows x cols X (trans == 0), or f[j] for the `rows` columns of a row-major
  * cols x rows X (trans == 1).  alp_emul_split: digits of a
@@ -180,7 +181,7 @@ alp_status alp_emul_split(int64_t R, int64_t K, const double* X, int64_t ldx, in
  * second time from L2) instead of scanning the matrix in a launch of its own;
  * exps receives the row exponents.  The same results as the two calls bit for
  * bit.  out_bf16 8-byte aligned, kpad a multiple of 64 and >= K, ldx >= K;
- * alp_gemm_f64_emul uses it for A when nslices > 0 and A is not transposed.
+ * the GEMM calls prepare their operands the same way, together in one launch.
  * ALP_ERR_INVALID_ARG for other kinds. */
 alp_status alp_emul_scan_split_rows(int64_t R, int64_t K, const double* X, int64_t ldx,
                                     int32_t* exps, int nslices, alp_slice_kind kind,
@@ -216,8 +217,8 @@ alp_status alp_emul_recombine(int64_t M, int64_t N, int nslices, alp_slice_kind 
  *   C = alpha * RN(P 2^(e_i + f_j - 2k))  (+ fma(beta, C, .) when beta != 0).
  * P is reached through its residues: the split writes out[l][r][k] = a residue
  * of A'_rk modulo m_{l+1} of magnitude at most 128 (exact in bf16; the one
- * nearest to zero, or, for k <= 51, one modulus off it when A'/m lies within
- * 0.003 of a half-integer); the tensor-core stage sums
+ * nearest to zero, or one modulus off it when A'/m lies next to a
+ * half-integer); the tensor-core stage sums
  * Q_l = sum_k a_l b_l exactly (|Q_l| <= K 2^14, Q_l = P mod m_l) and writes
  * the byte x_l = (Q_l y_l) mod m_l, y_l = (Mn/m_l)^-1 mod m_l, into plane
  * l-1 of G; the recombination forms sum_l x_l (Mn/m_l) = P mod Mn in 128-bit
@@ -276,8 +277,10 @@ alp_status alp_emul_recombine_crt(int64_t M, int64_t N, int64_t K, int nmoduli,
  * alp_emul_recombine_crt, bit for bit.  One persistent launch of CTA pairs
  * takes the 256 x 256 tiles of C from a counter; the product kernel's
  * reconstruction warps rebuild each finished tile from its byte planes while
- * the next tile's products run, and a small second launch rebuilds the tiles
- * of the last wave, whose moduli several pairs share.  alp_gemm_f64_emul runs
+ * the next tile's products run, and a small second launch rebuilds the last
+ * tiles, whose moduli all pairs share.  Where a tile's products are too short
+ * to hide its reconstruction, a second launch rebuilds every tile.
+ * alp_gemm_f64_emul runs
  * its modular scheme this way (ALP_EMUL_CRT_FUSE=0 in the environment: as the
  * two stages; the one-block arrangement, ALP_EMUL_CLUSTER=1, always so).
  * da_bf16, db_bf16: the residue slices of A and B^T as alp_emul_split writes

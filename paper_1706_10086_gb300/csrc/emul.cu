@@ -18,6 +18,7 @@
 #include "alp_ext.h"
 #include "alp_internal.cuh"
 #include "emul.cuh"
+#include "emul_prep.cuh"
 #include "emul_split.cuh"
 
 namespace alp {
@@ -30,37 +31,13 @@ alp_status validate_gemm(int64_t M, int64_t N, int64_t K, double alpha, const vo
 bool select_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                    cudaStream_t stream);
 alp_status crt_choose_moduli(int ta, int tb, int64_t M, int64_t N, int64_t K, const double* A,
-                             int64_t lda, const double* B, int64_t ldb, const int32_t* e,
-                             const int32_t* f, void* scratch, cudaStream_t stream, int* n_out,
-                             double* comp_u, double* norm_ratio);
+                             int64_t lda, const double* B, int64_t ldb, int32_t* e, int32_t* f,
+                             void* scratch, cudaStream_t stream, int* n_out, double* comp_u,
+                             double* norm_ratio);
 
 // ---------------------------------------------------------------------------
 // 1. exponent scan
 // ---------------------------------------------------------------------------
-constexpr uint64_t kAbsMask = 0x7FFFFFFFFFFFFFFFull;
-
-
-// |x| as ordered integer keys (larger key, larger |x|): the bits of a double
-// without its sign, or of a float.  A key at or above the infinity's is Inf
-// or NaN.  The float key converts to the double bits of the same value for
-// the exponent (FP32 operands convert exactly, so frexp and the digits are
-// the same as for the double of equal value).
-template <typename T> struct ScanKey;
-template <> struct ScanKey<double> {
-    using type = uint64_t;
-    static constexpr uint64_t kInf = 0x7FF0000000000000ull;
-    __device__ static uint64_t of(uint64_t bits) { return bits & kAbsMask; }
-    __device__ static uint64_t to_double_bits(uint64_t k) { return k; }
-};
-template <> struct ScanKey<float> {
-    using type = uint32_t;
-    static constexpr uint32_t kInf = 0x7F800000u;
-    __device__ static uint32_t of(uint32_t bits) { return bits & 0x7FFFFFFFu; }
-    __device__ static uint64_t to_double_bits(uint32_t k) {
-        return (uint64_t)__double_as_longlong((double)__int_as_float((int)k));
-    }
-};
-
 // Largest key of the V = 16 / sizeof(T) elements of a 16-byte vector.
 template <typename T>
 __device__ __forceinline__ typename ScanKey<T>::type vec_key(uint4 v) {
@@ -426,6 +403,9 @@ alp_status emul_exponents(int64_t rows, int64_t cols, const T* X, int64_t ldx, i
     return cuda_status(cudaGetLastError());
 }
 
+template alp_status emul_exponents<double>(int64_t, int64_t, const double*, int64_t, int, int32_t*,
+                                           cudaStream_t);
+
 template <typename T, int B>
 static alp_status emul_split_b(int64_t R, int64_t K, const T* X, int64_t ldx, int trans,
                                const int32_t* exps, int s, __nv_bfloat16* out, int64_t kpad,
@@ -463,6 +443,28 @@ alp_status emul_split(int64_t R, int64_t K, const T* X, int64_t ldx, int trans,
                       cudaStream_t st, int b) {
     if (b == 7) return emul_split_b<T, 7>(R, K, X, ldx, trans, exps, s, out, kpad, st);
     if (b == 8) return emul_split_b<T, 8>(R, K, X, ldx, trans, exps, s, out, kpad, st);
+    return ALP_ERR_INVALID_ARG;
+}
+
+// Exponents and digits of both operands in one launch.
+template <typename T>
+alp_status emul_prep_digits(const PrepParams<T>& p, int s, int b, cudaStream_t st) {
+#define ALP_PREP_CASE(x, B) \
+    case 10 * B + x: return launch_prep<T, x>(p, DigitSplit<B>{}, st);
+    if constexpr (sizeof(T) == 4) {
+        switch (10 * b + s) {
+            ALP_PREP_CASE(2, 7) ALP_PREP_CASE(3, 7) ALP_PREP_CASE(4, 7)
+            ALP_PREP_CASE(2, 8) ALP_PREP_CASE(3, 8) ALP_PREP_CASE(4, 8)
+        }
+    } else {
+        switch (10 * b + s) {
+            ALP_PREP_CASE(3, 7) ALP_PREP_CASE(4, 7) ALP_PREP_CASE(5, 7) ALP_PREP_CASE(6, 7)
+            ALP_PREP_CASE(7, 7) ALP_PREP_CASE(8, 7)
+            ALP_PREP_CASE(3, 8) ALP_PREP_CASE(4, 8) ALP_PREP_CASE(5, 8) ALP_PREP_CASE(6, 8)
+            ALP_PREP_CASE(7, 8)
+        }
+    }
+#undef ALP_PREP_CASE
     return ALP_ERR_INVALID_ARG;
 }
 
@@ -631,12 +633,6 @@ alp_status emul_gemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, T alp
     // rows of op(A): rows of A, or columns of its K x M storage; columns of
     // op(B): columns of B, or rows of its N x K storage
     alp_status st;
-    // the modular scheme with a given count and A not transposed scans A's
-    // rows inside its split (emul_scan_split_crt), after B's scan
-    bool fused_a = false;
-    if constexpr (!kF32) fused_a = sc.crt && !auto_n && ta == 0;
-    if (!fused_a && (st = emul_exponents(M, K, A, lda, ta, e, s)) != ALP_OK) return st;
-    if ((st = emul_exponents(N, K, B, ldb, 1 - tb, f, s)) != ALP_OK) return st;
     if constexpr (!kF32) {
         if (auto_n) {   // statistics in the (not yet written) residue-byte section
             if ((st = crt_choose_moduli(ta, tb, M, N, K, A, lda, B, ldb, e, f, ws + L0.off_g, s,
@@ -650,21 +646,48 @@ alp_status emul_gemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, T alp
     auto* da = reinterpret_cast<__nv_bfloat16*>(ws + L.off_da);
     auto* db = reinterpret_cast<__nv_bfloat16*>(ws + L.off_db);
     auto* G = reinterpret_cast<int32_t*>(ws + L.off_g);
-    if constexpr (kF32) {
-        if ((st = emul_split(M, K, A, lda, ta, e, nslices, da, L.kpad, s, b)) != ALP_OK) return st;
-        if ((st = emul_split(N, K, B, ldb, 1 - tb, f, nslices, db, L.kpad, s, b)) != ALP_OK)
-            return st;
-    } else if (sc.crt) {
-        if ((st = fused_a ? emul_scan_split_crt(M, K, A, lda, e, nslices, da, L.kpad, kcrt, s)
-                          : emul_split_crt(M, K, A, lda, ta, e, nslices, da, L.kpad, kcrt, s)) !=
-            ALP_OK)
-            return st;
-        if ((st = emul_split_crt(N, K, B, ldb, 1 - tb, f, nslices, db, L.kpad, kcrt, s)) != ALP_OK)
-            return st;
-    } else {
-        if ((st = emul_split(M, K, A, lda, ta, e, nslices, da, L.kpad, s, b)) != ALP_OK) return st;
-        if ((st = emul_split(N, K, B, ldb, 1 - tb, f, nslices, db, L.kpad, s, b)) != ALP_OK)
-            return st;
+    auto* sched = reinterpret_cast<int*>(ws + L0.off_sched);
+    // large strided operands by a scan (unless the exponents are known) and a
+    // split each, then the others in one launch, which also sets the schedule
+    // and lets the products start early
+    struct {
+        const T* X;
+        int64_t R, ldx;
+        int cols;
+        int32_t* exps;
+        __nv_bfloat16* out;
+    } ops[2] = {{A, M, lda, ta, e, da}, {B, N, ldb, 1 - tb, f, db}};
+    PrepParams<T> p = {};
+    p.K = K;
+    p.kpad = L.kpad;
+    p.known = auto_n ? 1 : 0;
+    p.err = device_error_word();
+    if (!kF32 && sc.crt) {
+        p.fill = sched;
+        p.fill_words = (int64_t)emul_crt_sched_words(M, N);
+    }
+    bool prepared = false;
+    for (int i = 0; i < 2; ++i) {
+        const auto& o = ops[i];
+        if (!o.cols || prep_in_strips<T>(o.R, K)) {
+            p.op[i] = {o.X, o.R, o.ldx, o.exps, o.out, o.cols, 0};
+            prepared = true;
+            continue;
+        }
+        if (!auto_n && (st = emul_exponents(o.R, K, o.X, o.ldx, 1, o.exps, s)) != ALP_OK) return st;
+        if constexpr (kF32) {
+            st = emul_split(o.R, K, o.X, o.ldx, 1, o.exps, nslices, o.out, L.kpad, s, b);
+        } else {
+            st = sc.crt ? emul_split_crt(o.R, K, o.X, o.ldx, 1, o.exps, nslices, o.out, L.kpad,
+                                         kcrt, s)
+                        : emul_split(o.R, K, o.X, o.ldx, 1, o.exps, nslices, o.out, L.kpad, s, b);
+        }
+        if (st != ALP_OK) return st;
+    }
+    if (prepared) {
+        if constexpr (kF32) st = emul_prep_digits(p, nslices, b, s);
+        else st = sc.crt ? emul_prep_crt(p, nslices, kcrt, s) : emul_prep_digits(p, nslices, b, s);
+        if (st != ALP_OK) return st;
     }
     alp_config cfg;
     const bool have = select_config(M, N, K, ALP_PATH_EMUL, &cfg, s) && emul_config_valid(cfg);
@@ -672,8 +695,8 @@ alp_status emul_gemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, T alp
         if (sc.crt)   // products and reconstruction (one launch with CTA pairs)
             return emul_crt_products_recombine(
                 M, N, K, nslices, da, db, L.kpad, reinterpret_cast<uint8_t*>(G), L.ldg, e, f,
-                kcrt, alpha, beta, C, ldc, reinterpret_cast<int*>(ws + L0.off_sched),
-                L0.sched_bytes, s, have ? cfg.stages : 0, have ? emul_arrangement_of(cfg) : 0);
+                kcrt, alpha, beta, C, ldc, sched, L0.sched_bytes, s, have ? cfg.stages : 0,
+                have ? emul_arrangement_of(cfg) : 0, -1, prepared);
     }
     if ((st = emul_slice_gemm(M, N, K, nslices, da, db, L.kpad, G, L.ldg, s,
                               have ? cfg.stages : 0, have ? emul_arrangement_of(cfg) : 0, b,
@@ -723,11 +746,8 @@ alp_status alp_emul_crt_choose(int trans_a, int trans_b, int64_t M, int64_t N, i
     auto* e = reinterpret_cast<int32_t*>(ws + L0.off_e);
     auto* f = reinterpret_cast<int32_t*>(ws + L0.off_f);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    alp_status st;
-    if ((st = emul_exponents(M, K, A, lda, trans_a, e, s)) != ALP_OK) return st;
-    if ((st = emul_exponents(N, K, B, ldb, 1 - trans_b, f, s)) != ALP_OK) return st;
     double c = 0.0, r = 0.0;
-    st = crt_choose_moduli(trans_a, trans_b, M, N, K, A, lda, B, ldb, e, f, ws + L0.off_g, s,
+    const alp_status st = crt_choose_moduli(trans_a, trans_b, M, N, K, A, lda, B, ldb, e, f, ws + L0.off_g, s,
                            nmoduli, &c, &r);
     if (st == ALP_OK && predicted) {
         predicted[0] = c;

@@ -52,8 +52,8 @@ constexpr int kCrtMaxModuli = 16;
 // reduction's range.
 constexpr int64_t kCrtMaxK = 1023 * 64;
 int crt_bits(int64_t K, int n);
-// y_l = (Mn / m_l)^-1 mod m_l for the first n moduli (host).
-uint32_t crt_weight(int n, int l);
+// y[l] = (Mn / m_l)^-1 mod m_l for the first n moduli, 0 past them (host).
+void crt_weights(int n, uint8_t (&y)[kCrtMaxModuli]);
 template <typename T>
 alp_status emul_split_crt(int64_t R, int64_t K, const T* X, int64_t ldx, int trans,
                           const int32_t* exps, int n, __nv_bfloat16* out, int64_t kpad, int k,
@@ -66,7 +66,15 @@ alp_status emul_scan_split_crt(int64_t R, int64_t K, const double* X, int64_t ld
 alp_status launch_recombine_crt(int n, int k, dim3 grid, cudaStream_t st, const uint8_t* R,
                                 int64_t rplane, int64_t ldr, const int32_t* e, const int32_t* f,
                                 int64_t M, int64_t N, double alpha, double beta, double* C,
-                                int64_t ldc);
+                                int64_t ldc, bool early = false);
+// Scale exponents of `rows` lines (emul.cu).
+template <typename T>
+alp_status emul_exponents(int64_t rows, int64_t cols, const T* X, int64_t ldx, int trans,
+                          int32_t* exps, cudaStream_t st);
+template <typename T>
+struct PrepParams;   // emul_prep.cuh
+// Exponents and residues of both operands in one launch (emul_prep.cuh).
+alp_status emul_prep_crt(const PrepParams<double>& p, int n, int k, cudaStream_t st);
 // Slice counts a GEMM call accepts: 3..emul_max_slices(b) digits for FP64,
 // 2..32/b for FP32, kCrtMinModuli..kCrtMaxModuli moduli for the modular scheme.
 inline bool emul_slices_ok(const EmulScheme& sc, int s, bool f32) {
@@ -121,15 +129,18 @@ dim3 recombine_grid(int64_t M, int64_t N);
 // with ALP_EMUL_CRT_FUSE=0) the product stage and the reconstruction kernel.
 // sched: the fused launch's schedule (emul_crt_sched_bytes(M, N) bytes of
 // device memory, 4-byte aligned; without it the two launches run).  fuse: 1
-// fuse, 0 do not, -1 as ALP_EMUL_CRT_FUSE says.
+// fuse, 0 do not, -1 as ALP_EMUL_CRT_FUSE says.  prepared: the previous launch
+// on the stream has written the operands and set emul_crt_sched_words(M, N)
+// words of sched to all ones, and lets this one start early.
 alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
                                        const __nv_bfloat16* da, const __nv_bfloat16* db,
                                        int64_t kpad, uint8_t* G, int64_t ldg, const int32_t* e,
                                        const int32_t* f, int k, double alpha, double beta,
                                        double* C, int64_t ldc, int* sched, size_t sched_bytes,
                                        cudaStream_t stream, int group_m = 0, int cluster = 0,
-                                       int fuse = -1);
+                                       int fuse = -1, bool prepared = false);
 size_t emul_crt_sched_bytes(int64_t M, int64_t N);
+size_t emul_crt_sched_words(int64_t M, int64_t N);
 
 // Tail split of the slice-product launch (see emul_gemm.cu): whole tiles for
 // blocks [0, n_full), then each remaining tile cut into `pieces` blocks by

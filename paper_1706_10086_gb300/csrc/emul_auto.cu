@@ -16,6 +16,7 @@
 
 #include "alp_ext.h"
 #include "emul.cuh"
+#include "emul_prep.cuh"
 
 namespace alp {
 
@@ -43,28 +44,6 @@ __device__ __forceinline__ void record_stats(float s1, float s2, float* out) {
         atomic_max_pos(out + 1, s2 / (s1 * s1));
         atomic_max_pos(out + 2, 1.0f / s2);
     }
-}
-
-// One warp per row of a row-major R x K matrix.
-__global__ void crt_stats_rows_kernel(const double* __restrict__ X, int64_t R, int64_t K,
-                                      int64_t ldx, const int32_t* __restrict__ e, float* out) {
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (row >= R) return;
-    const double* p = X + row * ldx;
-    const int er = e[row];
-    float s1 = 0.0f, s2 = 0.0f;
-    for (int64_t k = lane; k < K; k += 32) {
-        const float x = scaled_abs_f32((uint64_t)__double_as_longlong(__ldg(p + k)), er);
-        s1 += x;
-        s2 = fmaf(x, x, s2);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if (lane == 0) record_stats(s1, s2, out);
 }
 
 // Columns of a row-major K x N matrix: blocks of 32 columns x 256 rows, 8
@@ -107,18 +86,11 @@ __global__ void crt_stats_finish_kernel(int64_t N, const float* __restrict__ s1,
     if (j < N) record_stats(s1[j], s2[j], out);
 }
 
-// Statistics of the R lines of X (rows of a row-major R x L matrix when
-// !trans, else columns of a row-major L x R one), scale exponents `exps`,
-// into out[0..2]; s1, s2: R floats of scratch.
-alp_status line_stats(const double* X, int64_t R, int64_t L, int64_t ldx, int trans,
-                      const int32_t* exps, float* out, float* s1, float* s2, cudaStream_t st) {
+// Statistics of the R columns of a row-major L x R matrix X, scale exponents
+// `exps`, into out[0..2]; s1, s2: R floats of scratch.
+alp_status column_stats(const double* X, int64_t R, int64_t L, int64_t ldx, const int32_t* exps,
+                        float* out, float* s1, float* s2, cudaStream_t st) {
     if (R == 0 || L == 0) return ALP_OK;
-    if (!trans) {
-        const int wpb = 8;
-        crt_stats_rows_kernel<<<(unsigned)((R + wpb - 1) / wpb), 32 * wpb, 0, st>>>(X, R, L, ldx,
-                                                                                  exps, out);
-        return cuda_status(cudaGetLastError());
-    }
     if (cudaMemsetAsync(s1, 0, (size_t)R * 4, st) != cudaSuccess ||
         cudaMemsetAsync(s2, 0, (size_t)R * 4, st) != cudaSuccess)
         return ALP_ERR_CUDA;
@@ -126,6 +98,140 @@ alp_status line_stats(const double* X, int64_t R, int64_t L, int64_t ldx, int tr
     crt_stats_cols_kernel<<<grid, dim3(32, 8), 0, st>>>(X, L, R, ldx, exps, s1, s2);
     crt_stats_finish_kernel<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, s1, s2, out);
     return cuda_status(cudaGetLastError());
+}
+
+// ---- exponents and statistics of both operands in one launch, with the
+// line walks of emul_prep.cuh (contiguous lines by warps or blocks, strided
+// ones in strips through shared memory) ----
+
+// The sums of a contiguous line's elements k = 4 t, 4 t + 1, .. of one thread.
+template <int TEAM>
+__device__ __forceinline__ void stat_line(const double* x, int64_t K, bool vec, int t, int e,
+                                          float& s1, float& s2) {
+#pragma unroll 1
+    for (int64_t k0 = 4 * (int64_t)t; k0 < K; k0 += 16 * TEAM) {
+        double a[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) prep_load4(x, k0 + (int64_t)q * 4 * TEAM, K, vec, a[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float v = scaled_abs_f32((uint64_t)__double_as_longlong(a[q][u]), e);
+                s1 += v;
+                s2 = fmaf(v, v, s2);
+            }
+    }
+}
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+template <int TEAM>
+__device__ __forceinline__ void stat_rows(const PrepParams<double>& p,
+                                          const PrepOperand<double>& o, int block, float* out,
+                                          uint64_t (*red)[kPrepWarps], float2 (*sums)[kPrepWarps]) {
+    constexpr int kTeams = kPrepThreads / TEAM;
+    const int t = threadIdx.x % TEAM;
+    int par = 0;
+    for (int64_t r = (int64_t)block * kTeams + threadIdx.x / TEAM; r < o.R;
+         r += (int64_t)o.blocks * kTeams, par ^= 1) {
+        const double* x = o.X + r * o.ldx;
+        const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+        const uint64_t mx = prep_line_max<TEAM>(x, p.K, vec, t, red, par);
+        const int e = frexp_exponent_of_bits(mx);
+        if (t == 0) {
+            o.exps[r] = e;
+            if (mx >= ScanKey<double>::kInf) set_device_error(p.err, ALP_ERR_UNSUPPORTED);
+        }
+        float s1 = 0.0f, s2 = 0.0f;
+        stat_line<TEAM>(x, p.K, vec, t, e, s1, s2);
+        s1 = warp_sum(s1);
+        s2 = warp_sum(s2);
+        if constexpr (TEAM > 32) {
+            if ((t & 31) == 0) sums[par][t >> 5] = make_float2(s1, s2);
+            __syncthreads();
+            s1 = s2 = 0.0f;
+#pragma unroll
+            for (int w = 0; w < TEAM / 32; ++w) {
+                s1 += sums[par][w].x;
+                s2 += sums[par][w].y;
+            }
+        }
+        if (t == 0) record_stats(s1, s2, out);
+    }
+}
+
+__device__ __forceinline__ void stat_cols(const PrepParams<double>& p,
+                                          const PrepOperand<double>& o, int block, double* tile,
+                                          float* out, uint64_t* red, uint64_t* cmax, int* sexp,
+                                          float2* csum) {
+    constexpr int W = kPrepStrip<double>;
+    const uint32_t rank = cluster_ctarank(), size = cluster_nctarank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t j0 = (int64_t)(block / (int)size) * W, kb0 = (int64_t)rank * p.block_k;
+    const int rows = (int)min((int64_t)p.block_k, max(p.kpad - kb0, (int64_t)0));
+    uint64_t mx[kPrepV<double>];
+    prep_fill(o, p.K, j0, kb0, rows, p.block_k, tile, mx);
+    const uint64_t m = prep_column_max<double>(mx, red, cmax, size);
+    if (threadIdx.x < W) {
+        const int e = frexp_exponent_of_bits(m);
+        sexp[threadIdx.x] = e;
+        if (rank == 0 && j0 + threadIdx.x < o.R) {
+            o.exps[j0 + threadIdx.x] = e;
+            if (m >= ScanKey<double>::kInf) set_device_error(p.err, ALP_ERR_UNSUPPORTED);
+        }
+    }
+    __syncthreads();
+    const int Q = prep_q<double>(p.block_k);
+    const double* col = tile + (warp % W) * prep_ld<double>(p.block_k);
+    float s1 = 0.0f, s2 = 0.0f;
+    for (int k = lane; k < (warp < W ? rows : 0); k += 32) {
+        const float v = scaled_abs_f32(
+            (uint64_t)__double_as_longlong(col[(k & 3) * Q + (k >> 2)]), sexp[warp % W]);
+        s1 += v;
+        s2 = fmaf(v, v, s2);
+    }
+    s1 = warp_sum(s1);
+    s2 = warp_sum(s2);
+    if (lane == 0 && warp < W) csum[warp] = make_float2(s1, s2);
+    cluster_sync_all();
+    if (rank == 0 && threadIdx.x < W && j0 + threadIdx.x < o.R) {
+        s1 = s2 = 0.0f;
+        for (uint32_t q = 0; q < size; ++q) {
+            float a, b;
+            asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+                         : "=f"(a), "=f"(b)
+                         : "r"(cluster_addr(&csum[threadIdx.x], q))
+                         : "memory");
+            s1 += a;
+            s2 += b;
+        }
+        record_stats(s1, s2, out);
+    }
+    cluster_sync_all();   // csum and cmax read by the whole cluster
+}
+
+__global__ void __launch_bounds__(kPrepThreads, 3)
+    crt_prep_stats_kernel(const __grid_constant__ PrepParams<double> p, float* out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint64_t red[kPrepWarps * kPrepStrip<double>];
+    __shared__ uint64_t cmax[kPrepStrip<double>];
+    __shared__ int sexp[kPrepStrip<double>];
+    __shared__ __align__(8) float2 sums[2][kPrepWarps];
+    const bool second = (int)blockIdx.x >= p.op[0].blocks;
+    const PrepOperand<double>& o = p.op[second ? 1 : 0];
+    const int block = (int)blockIdx.x - (second ? p.op[0].blocks : 0);
+    float* st = out + (second ? 3 : 0);
+    if (o.cols)
+        stat_cols(p, o, block, reinterpret_cast<double*>(smem_raw), st, red, cmax, sexp, sums[0]);
+    else if (p.K <= kPrepWarpRowK)
+        stat_rows<32>(p, o, block, st, reinterpret_cast<uint64_t(*)[kPrepWarps]>(red), sums);
+    else
+        stat_rows<kPrepThreads>(p, o, block, st, reinterpret_cast<uint64_t(*)[kPrepWarps]>(red),
+                                sums);
 }
 
 }  // namespace
@@ -173,22 +279,42 @@ int crt_moduli_rule(int64_t M, int64_t N, int64_t K, const double st[6], double*
     return best;
 }
 
-// Runs the statistics of op(A) and op(B) (exponents e, f already scanned) on
-// `stream`, waits for them, and applies the rule.  scratch: 8 + 2 max(M, N)
-// floats of device memory.
+// Finds the exponents e, f and the statistics of op(A) and op(B) on `stream`,
+// waits for them, and applies the rule.  scratch: 8 + 2 max(M, N) floats of
+// device memory.
 alp_status crt_choose_moduli(int ta, int tb, int64_t M, int64_t N, int64_t K, const double* A,
-                             int64_t lda, const double* B, int64_t ldb, const int32_t* e,
-                             const int32_t* f, void* scratch, cudaStream_t stream, int* n_out,
-                             double* comp_u, double* norm_ratio) {
+                             int64_t lda, const double* B, int64_t ldb, int32_t* e, int32_t* f,
+                             void* scratch, cudaStream_t stream, int* n_out, double* comp_u,
+                             double* norm_ratio) {
     float* out = static_cast<float*>(scratch);
-    float* s1 = out + 8;
-    float* s2 = s1 + (M > N ? M : N);
     if (cudaMemsetAsync(out, 0, 8 * sizeof(float), stream) != cudaSuccess) return ALP_ERR_CUDA;
     alp_status st;
     // rows of op(A): rows of A, or columns of its K x M storage; columns of
     // op(B): columns of B, or rows of its N x K storage
-    if ((st = line_stats(A, M, K, lda, ta, e, out, s1, s2, stream)) != ALP_OK) return st;
-    if ((st = line_stats(B, N, K, ldb, 1 - tb, f, out + 3, s1, s2, stream)) != ALP_OK) return st;
+    PrepParams<double> p = {};
+    p.K = K;
+    p.kpad = (K + kEmulBK - 1) / kEmulBK * kEmulBK;
+    p.err = device_error_word();
+    float* s1 = out + 8;
+    float* s2 = s1 + (M > N ? M : N);
+    const struct {
+        const double* X;
+        int64_t R, ldx;
+        int cols;
+        int32_t* exps;
+    } ops[2] = {{A, M, lda, ta, e}, {B, N, ldb, 1 - tb, f}};
+    for (int i = 0; i < 2; ++i) {
+        const auto& o = ops[i];
+        if (!o.cols || prep_in_strips<double>(o.R, K))
+            p.op[i] = {o.X, o.R, o.ldx, o.exps, nullptr, o.cols, 0};
+        else if ((st = emul_exponents<double>(o.R, K, o.X, o.ldx, 1, o.exps, stream)) != ALP_OK ||
+                 (st = column_stats(o.X, o.R, K, o.ldx, o.exps, out + 3 * i, s1, s2, stream)) !=
+                     ALP_OK)
+            return st;
+    }
+    if ((p.op[0].X || p.op[1].X) &&
+        (st = launch_prep_kernel(crt_prep_stats_kernel, p, stream, out)) != ALP_OK)
+        return st;
     float h[8];
     if (cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)

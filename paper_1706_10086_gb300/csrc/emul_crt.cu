@@ -14,6 +14,7 @@
 #include "crt.cuh"
 #include "crt_rec.cuh"
 #include "emul.cuh"
+#include "emul_prep.cuh"
 #include "emul_split.cuh"
 
 namespace alp {
@@ -38,99 +39,136 @@ int crt_bits(int64_t K, int n) {
     return 0;
 }
 
-uint32_t crt_weight(int n, int l) {
-    if (n < 1 || n > kCrtMaxModuli || l < 0 || l >= n) return 0;
-    const uint32_t m = crt_modulus(l);
-    uint32_t r = 1;   // Mn / m_l mod m_l = prod_{i != l} m_i mod m_l
-    for (int i = 0; i < n; ++i)
-        if (i != l) r = (r * (crt_modulus(i) % m)) % m;
-    for (uint32_t y = 1; y < m; ++y)
-        if ((r * y) % m == 1u) return y;
-    return 0;
+namespace {
+// Per modulus count n: the weights and the reconstruction constants that do
+// not depend on k, formed once per process.
+struct CrtTables {
+    uint8_t y[kCrtMaxModuli + 1][kCrtMaxModuli] = {};
+    CrtRecConsts rec[kCrtMaxModuli + 1] = {};
+    CrtTables() {
+        for (int n = 1; n <= kCrtMaxModuli; ++n) {
+            for (int l = 0; l < n; ++l) {
+                const uint32_t m = crt_modulus(l);
+                uint32_t r = 1;   // Mn / m_l mod m_l = prod_{i != l} m_i mod m_l
+                for (int i = 0; i < n; ++i)
+                    if (i != l) r = (r * (crt_modulus(i) % m)) % m;
+                for (uint32_t w = 1; w < m; ++w)
+                    if ((r * w) % m == 1u) y[n][l] = (uint8_t)w;
+            }
+            CrtRecConsts& c = rec[n];
+            unsigned __int128 M = 1;
+            for (int l = 0; l < n; ++l) M *= crt_modulus(l);
+            for (int i = 0; i < 4; ++i) c.mn[i] = (uint32_t)(M >> (32 * i));
+            for (int g = 0; 3 * g < n && g < kCrtMaxGroups; ++g) {
+                uint32_t mg = 1;
+                for (int l = 3 * g; l < 3 * g + 3 && l < n; ++l) mg *= crt_modulus(l);
+                const unsigned __int128 Mg = M / mg;
+                for (int i = 0; i < 4; ++i) c.mg[g][i] = (uint32_t)(Mg >> (32 * i));
+                const uint64_t F = (uint64_t)(((unsigned __int128)1 << 58) + mg / 2) / mg;
+                c.fg_lo[g] = (uint32_t)F;
+                c.fg_hi[g] = (uint32_t)(F >> 32);
+                for (int l = 3 * g; l < 3 * g + 3 && l < n; ++l) c.cl[l] = mg / crt_modulus(l);
+            }
+            c.n = n;
+        }
+    }
+};
+const CrtTables& crt_tables() {
+    static const CrtTables t;
+    return t;
+}
+}  // namespace
+
+void crt_weights(int n, uint8_t (&y)[kCrtMaxModuli]) {
+    for (int l = 0; l < kCrtMaxModuli; ++l)
+        y[l] = n >= 1 && n <= kCrtMaxModuli ? crt_tables().y[n][l] : 0;
 }
 
-// The splitter.  A' = RN(a 2^(k - e)): for k <= 51 (and a normal power of two
-// 2^(k - e)) by one FP64 fma, else straight from the IEEE fields: a =
-// +-mant 2^E, shifted left when sh = E + k - e >= 0 (exact; |A'| <= 2^k since
-// |a| < 2^e), else rounded half to even at bit -sh (0 below 2^-54 of mant).
-// The residues, written as the bf16 encodings of integers r = A' (mod m)
-// with |r| <= 128 (the tensor-core stage's exactness bound):
-//  * for k <= 51 (|A'| <= 2^51) in f32 arithmetic: A' = c3 2^39 + c2 2^26 +
-//    c1 2^13 + c0 (c3 signed, |c3| <= 2^12; c2, c1, c0 in [0, 2^13)), each
-//    chunk turned into a float through its encoding (no conversion
-//    instruction), and per modulus x = c3 (2^39 mod m) + c2 (2^26 mod m) +
-//    c1 (2^13 mod m) + c0 by three fmas, exact (|x| < 2^23); q = x * RN(1/m)
-//    rounded to an integer through 1.5 2^23, and r = x - q m by one fma,
-//    exact: q is RN(x / m) or one off it when x / m lies within 0.003 of a
-//    half-integer, so |r| <= m / 2 + 0.7, an integer at most 128;
-//  * otherwise in integers: A' = hi 2^40 + mid 2^20 + lo (hi signed, |hi| <=
-//    2^20; mid, lo in [0, 2^20)) and x = hi (2^40 mod m) + mid (2^20 mod m) +
-//    lo + b_m with b_m = m ceil(2^28 / m) + floor(m / 2), so that 0 < x < 2^30
-//    and x = A' + floor(m / 2) (mod m); r = (x mod m) - floor(m / 2) in
-//    [-floor(m/2), ceil(m/2)).
+// The splitter.  A' = RN(a 2^(k - e)) is formed as U = A' + kSplitBias, an
+// unsigned 64-bit integer, and each residue from U's bytes.
+//
+// U, where 2^(k - e) is a normal power of two (a scaling by it is exact; a
+// result below the normal range is below 1/2 in magnitude):
+//  * k <= 51: one FP64 fma with 1.5 2^52 rounds to the nearest integer, ties to
+//    even: |a 2^(k - e)| <= 2^51 keeps the sum in [2^52, 2^53], where the
+//    encoding grows by one per unit, so the sum's encoding is U (the bias is
+//    the encoding of 1.5 2^52);
+//  * k >= 52: the same with 2^52 of a's sign, exact up to |A'| = 2^52; beyond, the
+//    scaled value is an integer already and its mantissa, shifted, is |A'|.
+// Otherwise straight from the IEEE fields: a = +-mant 2^E, shifted left when
+// sh = E + k - e >= 0, else rounded half to even at bit -sh.
+//
+// The residues are written as the bf16 encodings of integers r = A' (mod m)
+// with |r| <= 128 (the tensor-core stage's exactness bound): with w_i = 256^i
+// mod m (symmetric, |w_i| <= 127) two four-way byte dot products give sum_i
+// U_i w_i, below 2^18 in magnitude, added into the encoding of 1.5 2^23, whose
+// float minus 1.5 2^23 and kSplitBias mod m is an integer x = A' (mod m); q =
+// RN(x / m) by RN(1/m) and 1.5 2^23, and r = x - q m by one fma, exact.
+// x RN(1/m) is off by at most 2^-13, so q is RN(x / m) or one off it next to a
+// half-integer, and |r| <= m / 2 + 0.04, an integer at most 128.  Six instructions per modulus and none to cut A' up (three 13-bit
+// chunks turned into floats and three fmas each before, six and some 14 per
+// value, and eleven integer ones for k >= 52: 2048 x 2048 with 15 moduli, k = 52).
 // A float holding an integer of at most 8 significant bits has that
 // integer's bf16 encoding in its upper 16 bits, so packing two residues is
 // one byte permutation.
-__host__ __device__ constexpr uint32_t crt_split_bias(uint32_t m) {
-    return m * (((1u << 28) + m - 1) / m) + m / 2;
+constexpr uint64_t kSplitBias = 0x4338000000000000ull;   // the encoding of 1.5 2^52
+
+__host__ __device__ constexpr int crt_symmetric(uint32_t r, uint32_t m) {
+    return r > m / 2 - (m % 2 == 0 ? 1 : 0) ? (int)r - (int)m : (int)r;
 }
-// The f32 path's constants per modulus l: 2^13, 2^26, 2^39 mod m_l, RN(1/m_l)
-// and m_l, read from the constant bank as fma operands.
-struct CrtSplitF32 {
-    float p13[kCrtMaxModuli], p26[kCrtMaxModuli], p39[kCrtMaxModuli], inv[kCrtMaxModuli],
-        m[kCrtMaxModuli];
+// Bytes 256^i0 .. 256^(i0+3) mod m, symmetric.
+__host__ __device__ constexpr uint32_t crt_byte_weights(uint32_t m, int i0) {
+    uint32_t w = 0;
+    for (int i = 0; i < 4; ++i)
+        w |= ((uint32_t)crt_symmetric(crt_pow2_mod(8 * (i0 + i), m), m) & 0xFFu) << (8 * i);
+    return w;
+}
+// d = c + the dot product of a's unsigned and b's signed bytes.
+__device__ __forceinline__ int dp4a_us(uint32_t a, int b, int c) {
+    int d;
+    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+// The constants of modulus l, as literals: kept in the constant bank, the
+// weights would be hoisted into registers, which spill.
+template <int L>
+struct CrtSplitConsts {
+    static constexpr uint32_t m = crt_modulus(L);
+    static constexpr int wlo = (int)crt_byte_weights(m, 0), whi = (int)crt_byte_weights(m, 4);
+    static constexpr float off =
+        12582912.0f + (float)crt_symmetric((uint32_t)(kSplitBias % m), m);
+    static constexpr float inv = 1.0f / (float)m, mf = (float)m;
 };
-constexpr CrtSplitF32 make_crt_split_f32() {
-    CrtSplitF32 c{};
-    for (int l = 0; l < kCrtMaxModuli; ++l) {
-        const uint32_t m = crt_modulus(l);
-        c.p13[l] = (float)crt_pow2_mod(13, m);
-        c.p26[l] = (float)crt_pow2_mod(26, m);
-        c.p39[l] = (float)crt_pow2_mod(39, m);
-        c.inv[l] = 1.0f / (float)m;
-        c.m[l] = (float)m;
-    }
-    return c;
-}
-__constant__ CrtSplitF32 c_crt_split_f32 = make_crt_split_f32();
 
 struct CrtSplit {
     int k;
-    template <int S>
-    __device__ __forceinline__ void split(double a, int e, int (&d)[S]) const {
+    __device__ __forceinline__ uint64_t biased(double a, int e) const {
         const uint64_t bits = (uint64_t)__double_as_longlong(a);
-        const int ex = (int)((bits >> 52) & 0x7FF);
         const int se = k - e;
-        if (k <= 51 && se >= -1022 && se <= 1023) {
-            // a 2^se is exact (a scaling by a normal power of two; a result
-            // below the normal range is below 1/2 in magnitude), so one fma
-            // with 1.5 2^52 rounds it to the nearest integer, ties to even:
-            // |a 2^se| <= 2^51 keeps the sum in [2^52, 2^53], where the
-            // encoding grows by one per unit, and the difference of the two
-            // encodings is the integer
-            const double y =
-                __fma_rn(a, __longlong_as_double((long long)(se + 1023) << 52), 6755399441055744.0);
-            const int64_t v =
-                ex == 0x7FF ? 0 : (int64_t)__double_as_longlong(y) - 0x4338000000000000ll;
-            const uint32_t vl = (uint32_t)v, vh = (uint32_t)((uint64_t)v >> 32);
-            const float f0 = __int_as_float(0x4B000000 | (vl & 0x1FFFu)) - 8388608.0f;
-            const float f1 = __int_as_float(0x4B000000 | ((vl >> 13) & 0x1FFFu)) - 8388608.0f;
-            const float f2 = __int_as_float(0x4B000000 | (__funnelshift_r(vl, vh, 26) & 0x1FFFu)) -
-                             8388608.0f;
-            const float f3 = __int_as_float(0x4B400000 + ((int32_t)vh >> 7)) - 12582912.0f;
-            const CrtSplitF32& c = c_crt_split_f32;
-#pragma unroll
-            for (int l = 0; l < S; ++l) {
-                const float x =
-                    __fmaf_rn(f3, c.p39[l], __fmaf_rn(f2, c.p26[l], __fmaf_rn(f1, c.p13[l], f0)));
-                const float q = __fadd_rn(__fmaf_rn(x, c.inv[l], 12582912.0f), -12582912.0f);
-                d[l] = __float_as_int(__fmaf_rn(-q, c.m[l], x));
-            }
-            return;
+        if (se >= -1022 && se <= 1023) {
+            const double scale = __longlong_as_double((long long)(se + 1023) << 52);
+            if (k <= 51)
+                return (uint64_t)__double_as_longlong(__fma_rn(a, scale, 6755399441055744.0));
+            // 2^52 with a's sign, so that the sum's encoding without its sign
+            // is 2^52's plus |A'|.  Signs are set and dropped in the high word:
+            // on a double's 64 bits the compiler makes them FP64 operations,
+            // each of which holds the sub-partition's FP64 pipe for 73 clocks
+            const int hi = __double2hiint(a);
+            const double y = __fma_rn(
+                a, scale, __hiloint2double(0x43300000 | (hi & (int)0x80000000), 0));
+            uint64_t v = ((uint64_t)(uint32_t)((__double2hiint(y) & 0x7FFFFFFF) - 0x43300000) << 32) |
+                         (uint32_t)__double2loint(y);
+            const int sh = (int)((bits >> 52) & 0x7FF) - 1075 + se;
+            if (k > 52 && sh >= 0)   // at least 2^52: an integer, at most 2^60 (finite a)
+                v = ((bits & ((1ull << 52) - 1)) | (1ull << 52)) << (sh > 8 ? 0 : sh);
+            const uint64_t s = (uint64_t)((int64_t)bits >> 63);   // 0 or all ones
+            return kSplitBias + ((v ^ s) - s);
         }
+        const int ex = (int)((bits >> 52) & 0x7FF);
         uint64_t mant = bits & ((1ull << 52) - 1);
         int E = -1074;
-        if (ex == 0x7FF) mant = 0;   // Inf/NaN: reported by the scan; residues 0
+        if (ex == 0x7FF) mant = 0;   // Inf/NaN: reported by the scan
         else if (ex) {
             mant |= 1ull << 52;
             E = ex - 1075;
@@ -146,17 +184,18 @@ struct CrtSplit {
             const uint64_t q = mant >> r, rem = mant & ((1ull << r) - 1), half = 1ull << (r - 1);
             u = q + ((rem > half || (rem == half && (q & 1))) ? 1 : 0);
         }
-        const int64_t v = (int64_t)bits < 0 ? -(int64_t)u : (int64_t)u;
-        const int32_t hi = (int32_t)(v >> 40);
-        const uint32_t mid = (uint32_t)(v >> 20) & 0xFFFFFu, lo = (uint32_t)v & 0xFFFFFu;
-#pragma unroll
-        for (int l = 0; l < S; ++l) {
-            const uint32_t m = crt_modulus(l);
-            const int32_t x = hi * (int32_t)crt_pow2_mod(40, m) +
-                              (int32_t)(mid * crt_pow2_mod(20, m) + (lo + crt_split_bias(m)));
-            const int r = (int)crt_mod((uint32_t)x, m) - (int)(m / 2);
-            d[l] = __float_as_int(__int_as_float(0x4B400000 + r) - 12582912.0f);
-        }
+        return (int64_t)bits < 0 ? kSplitBias - u : kSplitBias + u;
+    }
+    // What the residues are formed from, and the residue of modulus L.
+    using State = uint64_t;
+    __device__ __forceinline__ State init(double a, int e) const { return biased(a, e); }
+    template <int L>
+    __device__ __forceinline__ int next(State& u) const {
+        using C = CrtSplitConsts<L>;
+        const int f = dp4a_us((uint32_t)(u >> 32), C::whi, dp4a_us((uint32_t)u, C::wlo, 0x4B400000));
+        const float x = __fadd_rn(__int_as_float(f), -C::off);
+        const float q = __fadd_rn(__fmaf_rn(x, C::inv, 12582912.0f), -12582912.0f);
+        return __float_as_int(__fmaf_rn(-q, C::mf, x));
     }
     // two residues (float encodings) as packed bf16
     __device__ __forceinline__ uint32_t pack(int lo, int hi) const {
@@ -184,7 +223,7 @@ alp_status emul_split_crt(int64_t R, int64_t K, const T* X, int64_t ldx, int tra
 #define ALP_CRT_SPLIT_CASE(x)                                                                    \
     case x:                                                                                      \
         if (!trans && vec)                                                                       \
-            split_rows4_kernel<T, x, CrtSplit, 128, 6><<<grid4, 128, 0, st>>>(X, R, K, ldx, exps, \
+            split_rows4_kernel<T, x, CrtSplit, 128, 8><<<grid4, 128, 0, st>>>(X, R, K, ldx, exps, \
                                                                               out, kpad, sp);     \
         else if (!trans)                                                                         \
             split_rows_kernel<T, x, CrtSplit><<<(unsigned)blocks, 256, 0, st>>>(                  \
@@ -219,7 +258,7 @@ alp_status emul_scan_split_crt(int64_t R, int64_t K, const double* X, int64_t ld
     int* err = device_error_word();
 #define ALP_CRT_SCAN_SPLIT_CASE(x)                                                            \
     case x:                                                                                  \
-        scan_split_rows4_kernel<x, CrtSplit, 128, 6>                                         \
+        scan_split_rows4_kernel<x, CrtSplit, 128, 8>                                         \
             <<<(unsigned)blocks, 128, 0, st>>>(X, R, K, ldx, exps, out, kpad, sp, err);      \
         break;
     switch (n) {
@@ -239,23 +278,24 @@ template alp_status emul_split_crt<double>(int64_t, int64_t, const double*, int6
                                            cudaStream_t);
 
 CrtRecConsts crt_rec_consts(int n, int k) {
-    CrtRecConsts c{};
-    unsigned __int128 M = 1;
-    for (int l = 0; l < n; ++l) M *= crt_modulus(l);
-    for (int i = 0; i < 4; ++i) c.mn[i] = (uint32_t)(M >> (32 * i));
-    for (int g = 0; 3 * g < n && g < kCrtMaxGroups; ++g) {
-        uint32_t mg = 1;
-        for (int l = 3 * g; l < 3 * g + 3 && l < n; ++l) mg *= crt_modulus(l);
-        const unsigned __int128 Mg = M / mg;
-        for (int i = 0; i < 4; ++i) c.mg[g][i] = (uint32_t)(Mg >> (32 * i));
-        const uint64_t F = (uint64_t)(((unsigned __int128)1 << 58) + mg / 2) / mg;
-        c.fg_lo[g] = (uint32_t)F;
-        c.fg_hi[g] = (uint32_t)(F >> 32);
-        for (int l = 3 * g; l < 3 * g + 3 && l < n; ++l) c.cl[l] = mg / crt_modulus(l);
-    }
-    c.n = n;
+    CrtRecConsts c = crt_tables().rec[n];
     c.k = k;
     return c;
+}
+
+alp_status emul_prep_crt(const PrepParams<double>& p, int n, int k, cudaStream_t st) {
+    if (k < 1 || k > 60) return ALP_ERR_UNSUPPORTED;
+    const CrtSplit sp{k};
+#define ALP_CRT_PREP_CASE(x) \
+    case x: return launch_prep<double, x>(p, sp, st);
+    switch (n) {
+        ALP_CRT_PREP_CASE(4) ALP_CRT_PREP_CASE(5) ALP_CRT_PREP_CASE(6) ALP_CRT_PREP_CASE(7)
+        ALP_CRT_PREP_CASE(8) ALP_CRT_PREP_CASE(9) ALP_CRT_PREP_CASE(10) ALP_CRT_PREP_CASE(11)
+        ALP_CRT_PREP_CASE(12) ALP_CRT_PREP_CASE(13) ALP_CRT_PREP_CASE(14) ALP_CRT_PREP_CASE(15)
+        ALP_CRT_PREP_CASE(16)
+        default: return ALP_ERR_INVALID_ARG;
+    }
+#undef ALP_CRT_PREP_CASE
 }
 
 // Four columns per thread: the n bytes of four adjacent columns arrive in one
@@ -269,6 +309,7 @@ __global__ void __launch_bounds__(128, 5) recombine_crt_kernel(
     const int32_t* __restrict__ f, int64_t M, int64_t N, double alpha, double beta,
     double* __restrict__ C, int64_t ldc, bool rvec, int amode, int bmode,
     const CrtRecConsts cc) {
+    pdl_wait();
     for (int64_t i = blockIdx.y; i < M; i += gridDim.y) {
         const int ei = e[i] - 2 * cc.k;
         const uint8_t* ri = R + i * ldr;
@@ -342,6 +383,7 @@ __global__ void __launch_bounds__(128, 5) recombine_crt_staged_kernel(
     const int32_t* __restrict__ f, int64_t M, int64_t N, double alpha, double beta,
     double* __restrict__ C, int64_t ldc, int amode, int bmode, const CrtRecConsts cc,
     uint64_t tmo, int* err) {
+    pdl_wait();
     __shared__ __align__(16) uint8_t slots[kCrtRecSlots][S][512];
     __shared__ uint64_t full[kCrtRecSlots];
     const int64_t j0 = (int64_t)blockIdx.x * 512;
@@ -422,7 +464,7 @@ __global__ void __launch_bounds__(128, 5) recombine_crt_staged_kernel(
 alp_status launch_recombine_crt(int n, int k, dim3 grid, cudaStream_t st, const uint8_t* R,
                                 int64_t rplane, int64_t ldr, const int32_t* e, const int32_t* f,
                                 int64_t M, int64_t N, double alpha, double beta, double* C,
-                                int64_t ldc) {
+                                int64_t ldc, bool early) {
     if (k < 1 || k > 60) return ALP_ERR_UNSUPPORTED;
     const CrtRecConsts cc = crt_rec_consts(n, k);
     const bool rvec = (reinterpret_cast<uintptr_t>(R) & 3) == 0 && rplane % 4 == 0 && ldr % 4 == 0;
@@ -434,14 +476,24 @@ alp_status launch_recombine_crt(int n, int k, dim3 grid, cudaStream_t st, const 
     int* err = device_error_word();
     // four columns per thread, 128-thread blocks: 512 columns per block, as
     // the grid was sized
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(128);
+    lc.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = early ? 1 : 0;   // the kernel before it lets it start early
+    cudaError_t ce = cudaSuccess;
 #define ALP_CRT_REC_CASE(x)                                                                       \
     case x:                                                                                      \
         if (staged)                                                                              \
-            recombine_crt_staged_kernel<x><<<grid, 128, 0, st>>>(                                 \
-                R, rplane, ldr, e, f, M, N, alpha, beta, C, ldc, amode, bmode, cc, tmo, err);    \
+            ce = cudaLaunchKernelEx(&lc, recombine_crt_staged_kernel<x>, R, rplane, ldr, e, f, M, \
+                                    N, alpha, beta, C, ldc, amode, bmode, cc, tmo, err);         \
         else                                                                                     \
-            recombine_crt_kernel<x><<<grid, 128, 0, st>>>(R, rplane, ldr, e, f, M, N, alpha,     \
-                                                          beta, C, ldc, rvec, amode, bmode, cc); \
+            ce = cudaLaunchKernelEx(&lc, recombine_crt_kernel<x>, R, rplane, ldr, e, f, M, N,     \
+                                    alpha, beta, C, ldc, rvec, amode, bmode, cc);                \
         break;
     switch (n) {
         ALP_CRT_REC_CASE(4) ALP_CRT_REC_CASE(5) ALP_CRT_REC_CASE(6) ALP_CRT_REC_CASE(7)
@@ -451,7 +503,7 @@ alp_status launch_recombine_crt(int n, int k, dim3 grid, cudaStream_t st, const 
         default: return ALP_ERR_INVALID_ARG;
     }
 #undef ALP_CRT_REC_CASE
-    return cuda_status(cudaGetLastError());
+    return cuda_status(ce);
 }
 
 }  // namespace alp

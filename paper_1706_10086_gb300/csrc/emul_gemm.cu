@@ -33,6 +33,7 @@
 // (|S^t| < 2^31, |Q_l| <= K 2^14 for the K limits).  At the end of a group
 // the block writes S^t to G[t-2] (int32), or, for the modular scheme, the byte
 // (Q_l y_l) mod m_l to plane l-1 of G.
+#include <algorithm>
 #include <cstdlib>
 
 #include "crt.cuh"
@@ -513,6 +514,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
+    pdl_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kPairStages; ++i) {
             mbar_init(&full[i], 1);    // block 0's producer; bytes of both blocks
@@ -545,6 +547,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     tc_fence_before();
     cluster_sync_all();   // both blocks' barriers and TMEM exist before any signal
     tc_fence_after();
+    pdl_wait();           // the operands are written
     const uint32_t tmem_base = *tmem_slot;
     const int njobs = *njobs_slot;
 
@@ -702,7 +705,10 @@ struct CrtFuse {
     int64_t ldc;
     int amode;          // alpha: 0 one, 1 minus one, 2 any
     int bmode;          // beta: 0 zero (C not read), 1 any
-    int n_items;        // whole tiles n_full, then (pair tiles - n_full) * pieces
+    int n_items;        // whole tiles n_full, then the parts of the tail tiles
+    int parts;
+    int tail_tiles;     // pair tiles - n_full
+    int rec;            // whole tiles are reconstructed in the launch
     // the schedule (workspace, all bytes 0xff before the launch): sched[0] the
     // item counter, sched[1 + c * stride + k] the k-th item of cluster c
     // (n_items or more: no more items), stride = n_items + 1
@@ -718,20 +724,29 @@ constexpr int kMaxFusedClusters = 128;   // clusters of one launch (the schedule
 static_assert(2 * 128 * kFusedEpiRegs + 2 * 128 * kFusedLowRegs == kFusedThreads * 128,
               "register split of the fused kernel");
 
-// Item i: the pair tile and its moduli q_lo..q_hi (planes, 0-based).
-__device__ __forceinline__ void fused_item(const EmulGemmParams& prm, int i, int& pid, int& q_lo,
-                                           int& q_hi) {
-    if (i < prm.n_full) {
-        pid = i;
-        q_lo = 0;
-        q_hi = prm.s - 1;
-        return;
+// Item i's units, a unit being one modulus of one pair tile: the moduli of the
+// whole tile i, or, past the n_full whole ones, every parts-th unit of the tail
+// tiles from i - n_full on.  The tail's units are ordered by modulus, then by
+// tile, so that clusters side by side in time multiply the same residue slices,
+// which then come from L2 (shared by tile instead, each cluster at another
+// modulus, 2048^3 read 2 GB from HBM and ran its products in 211 us, not 150).
+struct FusedUnits {
+    int v, end, step, tile;   // tile >= 0: v is its modulus; -1: v counts tail units
+};
+__device__ __forceinline__ FusedUnits fused_item(const EmulGemmParams& prm, const CrtFuse& fz,
+                                                 int i) {
+    if (i < prm.n_full) return {0, prm.s, 1, i};
+    return {i - prm.n_full, fz.tail_tiles * prm.s, fz.parts, -1};
+}
+__device__ __forceinline__ void fused_unit(const EmulGemmParams& prm, const CrtFuse& fz,
+                                           const FusedUnits& it, int& pid, int& q) {
+    if (it.tile >= 0) {
+        pid = it.tile;
+        q = it.v;
+    } else {
+        q = it.v / fz.tail_tiles;
+        pid = prm.n_full + it.v - q * fz.tail_tiles;
     }
-    const int pc = (i - prm.n_full) % prm.pieces;
-    pid = prm.n_full + (i - prm.n_full) / prm.pieces;
-    const uint32_t r = (uint32_t)(prm.t_ranges >> (8 * pc)) & 0xffu;
-    q_lo = (int)(r & 15u);
-    q_hi = (int)(r >> 4);
 }
 
 // The k-th item of cluster c: block 0's producer takes it from the counter
@@ -867,11 +882,11 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
     for (int k = 0; ok && k < fz.stride; ++k) {
         const int it = fused_next(fz, cid, k, tmo, abort_flag, prm.err);
         if (it >= fz.n_items) break;
-        int pid, qlo, qhi, m0, n0;
-        fused_item(prm, it, pid, qlo, qhi);
-        pair_tile_origin(prm, pid, rank, m0, n0);
-        const int gm = m0 + row;
-        for (int q = qlo; q <= qhi && ok; ++q) {
+        for (FusedUnits fu = fused_item(prm, fz, it); fu.v < fu.end && ok; fu.v += fu.step) {
+            int pid, q, m0, n0;
+            fused_unit(prm, fz, fu, pid, q);
+            pair_tile_origin(prm, pid, rank, m0, n0);
+            const int gm = m0 + row;
 #pragma unroll
             for (int x = 0; x < 128; ++x) acc[x] = 0;
             for (int c = 0; c < cpm; ++c, ++job) {
@@ -902,9 +917,9 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
                 for (int i = 0; i < 8; ++i) {
                     uint32_t w[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int c = 16 * i + 4 * u;
-                        w[u] = crt_mod(crt_residue((int32_t)acc[c], m, magic) * y, m, magic) |
+                    for (int x = 0; x < 4; ++x) {
+                        const int c = 16 * i + 4 * x;
+                        w[x] = crt_mod(crt_residue((int32_t)acc[c], m, magic) * y, m, magic) |
                                crt_mod(crt_residue((int32_t)acc[c + 1], m, magic) * y, m, magic)
                                    << 8 |
                                crt_mod(crt_residue((int32_t)acc[c + 2], m, magic) * y, m, magic)
@@ -916,7 +931,7 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
                 }
             }
         }
-        if (ok && it < prm.n_full) {
+        if (ok && fz.rec && it < prm.n_full) {
             // every plane of this whole tile is stored: count it
             __threadfence_block();
             __syncwarp();
@@ -937,7 +952,7 @@ __device__ __forceinline__ void fused_reconstruction(const EmulGemmParams& prm, 
     const int w = warp - kFusedRecWarp0;                     // 0..3
     const int cid = (int)blockIdx.x / 2;
     uint32_t k = 0;   // whole tiles of this cluster so far
-    for (int x = 0; x < fz.stride; ++x) {
+    for (int x = 0; fz.rec && x < fz.stride; ++x) {
         const int it = fused_next(fz, cid, x, tmo, abort_flag, prm.err);
         if (it >= fz.n_items) return;
         if (it >= prm.n_full) continue;   // a tail piece: reconstructed after the launch
@@ -985,6 +1000,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
+    pdl_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kPairStages; ++i) {
             mbar_init(&full[i], 1);    // block 0's producer; bytes of both blocks
@@ -1007,6 +1023,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     tc_fence_before();
     cluster_sync_all();   // both blocks' barriers and TMEM exist before any signal
     tc_fence_after();
+    pdl_wait();           // the operands, exponents and schedule are written
     const uint32_t tmem_base = *tmem_slot;
     const uint64_t tmo = prm.timeout_ns;
     const uint32_t full0 = cluster_addr(full, 0);   // block 0's full barriers
@@ -1036,10 +1053,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                 const int item = leader ? fused_take(fz, cid, k)
                                         : fused_next(fz, cid, k, tmo, abort_flag, prm.err);
                 if (item >= fz.n_items) break;
-                int pid, qlo, qhi, m0, n0;
-                fused_item(prm, item, pid, qlo, qhi);
-                pair_tile_origin(prm, pid, rank, m0, n0);
-                for (int q = qlo; q <= qhi && ok; ++q) {
+                for (FusedUnits fu = fused_item(prm, fz, item); fu.v < fu.end && ok;
+                     fu.v += fu.step) {
+                    int pid, q, m0, n0;
+                    fused_unit(prm, fz, fu, pid, q);
+                    pair_tile_origin(prm, pid, rank, m0, n0);
                     for (int kb = 0; kb < kblocks; ++kb, ++it) {
                         const uint32_t st = it % kPairStages, round = it / kPairStages;
                         if (it >= (uint32_t)kPairStages &&
@@ -1080,9 +1098,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             for (int k = 0; ok && k < fz.stride; ++k) {
                 const int item = fused_next(fz, cid, k, tmo, abort_flag, prm.err);
                 if (item >= fz.n_items) break;
-                int pid, qlo, qhi;
-                fused_item(prm, item, pid, qlo, qhi);
-                for (int q = qlo; q <= qhi && ok; ++q) {
+                for (FusedUnits fu = fused_item(prm, fz, item); fu.v < fu.end && ok;
+                     fu.v += fu.step) {
                     for (int c = 0; c < cpm && ok; ++c, ++job) {
                         const uint32_t b = job & 1;
                         if (job >= 2 && !mbar_wait_bounded(&acce[b], ((job >> 1) - 1) & 1, tmo,
@@ -1137,22 +1154,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     }
 }
 
-// The tail tiles of a fused launch (pair tiles n_full..): 16 blocks of 256
-// threads per tile, block b holding rows 16 (b % 8) .. + 16 of the tile's
-// half (b / 8) % 2, four rows per step.
+// The tail tiles of a fused launch (pair tiles n_full..): 64 blocks of 256
+// threads per tile, four rows each, so that a few tiles still fill the SMs.
 __global__ void __launch_bounds__(256) crt_tail_recombine_kernel(EmulGemmParams prm, CrtFuse fz) {
+    pdl_wait();
     const int b = (int)blockIdx.x;
-    const int strip = b & 7, r = (b >> 3) & 1, pid = prm.n_full + (b >> 4);
+    const int strip = b & 31, r = (b >> 5) & 1, pid = prm.n_full + (b >> 6);
     int m0, n0;
     pair_tile_origin(prm, pid, (uint32_t)r, m0, n0);
     const int64_t j = (int64_t)n0 + 4 * (threadIdx.x & 63);
-#pragma unroll 1
-    for (int step = 0; step < 4; ++step) {
-        const int64_t i = (int64_t)m0 + 16 * strip + 4 * step + (threadIdx.x >> 6);
-        uint32_t v[16];
-        crt_fused_load(prm, i, j, v);
-        crt_fused_finish(prm, fz, i, j, v);
-    }
+    const int64_t i = (int64_t)m0 + 4 * strip + (threadIdx.x >> 6);
+    uint32_t v[16];
+    crt_fused_load(prm, i, j, v);
+    crt_fused_finish(prm, fz, i, j, v);
 }
 
 }  // namespace
@@ -1251,7 +1265,8 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     p.digit_bits = digit_bits;
     p.trim = trim ? 1 : 0;
     p.crt = crt ? 1 : 0;
-    for (int l = 0; l < kCrtMaxModuli; ++l) p.crt_y[l] = crt && l < s ? crt_weight(s, l) : 0;
+    if (crt) crt_weights(s, p.crt_y);
+    else std::fill(p.crt_y, p.crt_y + kCrtMaxModuli, uint8_t(0));
     p.G = G;
     p.ldg = ldg;
     p.gplane = M * ldg;
@@ -1351,12 +1366,58 @@ size_t emul_crt_sched_bytes(int64_t M, int64_t N) {
     return (size_t)4 * (1 + (size_t)kMaxFusedClusters * (size_t)(pair_tiles + 7 * kMaxFusedClusters + 1));
 }
 
+// Words of the schedule a launch on this device may read: the counter and the
+// lists of as many clusters as it can run, each with room for every item.
+size_t emul_crt_sched_words(int64_t M, int64_t N) {
+    const int64_t pair_tiles = ((M + 2 * kTM - 1) / (2 * kTM)) * ((N + kTN - 1) / kTN);
+    const int64_t P = std::min(fused_active_clusters(), kMaxFusedClusters);
+    const int64_t items = pair_tiles + P;   // at most: whole tiles, then up to P parts
+    return (size_t)(1 + std::min(items, P) * (items + 1));
+}
+
+// How a fused launch of `tiles` pair tiles, n moduli and kblocks 64-k blocks is
+// cut for P resident clusters: the whole tiles, handed out from the counter,
+// fill whole waves; the units (tile, modulus) of the rest are shared evenly,
+// up to P parts (2048^3: 13 units per cluster instead of a whole tile's 15).
+// rec: whole tiles are reconstructed by the launch's own warps, while later
+// products run; the tail tiles then follow in a small launch.  A block's four
+// reconstruction warps need about as long for a tile as 450 of its k-blocks
+// take (150 us), so that is done only when a tile's products outlast it, and
+// the last whole tiles' reconstruction must find products to hide behind (else
+// those tiles join the tail: 2048^3 and 3000 x 1500 x 2100 ran 435 and 553 us
+// with it exposed at the end of the launch, 323 and 399 as two launches).
+// Otherwise every tile is reconstructed by the following kernel, which takes
+// 0.55 us per tile with all SMs.
+struct FusedCut {
+    int64_t n_full;
+    int parts;
+    bool rec;
+};
+static FusedCut fused_cut(int64_t tiles, int n, int64_t kblocks, int P) {
+    FusedCut c{tiles, 0, true};
+    if (!emul_tail_split_on()) return c;
+    constexpr int64_t kRecBlocks = 600;    // k-blocks of a tile that hide its reconstruction
+    constexpr int64_t kTailBlocks = 320;   // k-blocks after the last whole tile that do
+    const int64_t waves = tiles / P, rest = tiles % P;
+    c.n_full = waves * P;
+    c.rec = waves > 0 && n * kblocks >= kRecBlocks;
+    if (c.rec && (rest * n + P - 1) / P * kblocks < kTailBlocks) {
+        c.n_full -= P;
+        c.rec = c.n_full > 0;
+        if (!c.rec) c.n_full = waves * P;
+    }
+    const int64_t units = (tiles - c.n_full) * n;
+    c.parts = (int)std::min<int64_t>(P, units);
+    return c;
+}
+
 alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
                                        const __nv_bfloat16* da, const __nv_bfloat16* db,
                                        int64_t kpad, uint8_t* G, int64_t ldg, const int32_t* e,
                                        const int32_t* f, int k, double alpha, double beta,
                                        double* C, int64_t ldc, int* sched, size_t sched_bytes,
-                                       cudaStream_t stream, int group_m, int cluster, int fuse) {
+                                       cudaStream_t stream, int group_m, int cluster, int fuse,
+                                       bool prepared) {
     if (n < kCrtMinModuli || n > kCrtMaxModuli || K > kCrtMaxK || k < 1 || k > 60)
         return ALP_ERR_UNSUPPORTED;
     const int arr = (cluster == kEmulSingle || cluster == kEmulPair) ? cluster : emul_cluster();
@@ -1382,7 +1443,7 @@ alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
     p.digit_bits = kDigitBits;
     p.trim = 0;
     p.crt = 1;
-    for (int l = 0; l < kCrtMaxModuli; ++l) p.crt_y[l] = l < n ? crt_weight(n, l) : 0;
+    crt_weights(n, p.crt_y);
     p.G = reinterpret_cast<int32_t*>(G);
     p.ldg = ldg;
     p.gplane = M * ldg;
@@ -1401,19 +1462,15 @@ alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
     if (ce != cudaSuccess) return cuda_status(ce);
     const int P = fused_active_clusters() < kMaxFusedClusters ? fused_active_clusters()
                                                                : kMaxFusedClusters;
-    p.n_full = (int)pair_tiles;
     p.pieces = 1;
-    p.t_ranges = (uint64_t)(n - 1) << 4;
-    if (emul_tail_split_on()) {   // whole tiles fill the waves of P clusters
-        const TailSplit ts = tail_split((int)pair_tiles, n, P, false, true);
-        p.n_full = ts.n_full;
-        p.pieces = ts.pieces;
-        p.t_ranges = 0;
-        for (int i = 0; i < ts.pieces; ++i)
-            p.t_ranges |= (uint64_t)((ts.t_lo[i] - 2) | (ts.t_hi[i] - 2) << 4) << (8 * i);
-    }
-    const int64_t items = p.n_full + (pair_tiles - p.n_full) * p.pieces;
+    p.t_ranges = 0;
     CrtFuse fz;
+    const FusedCut cut = fused_cut(pair_tiles, n, (K + kTK - 1) / kTK, P);
+    p.n_full = (int)cut.n_full;
+    fz.parts = cut.parts;
+    fz.rec = cut.rec ? 1 : 0;
+    fz.tail_tiles = (int)(pair_tiles - cut.n_full);
+    const int64_t items = cut.n_full + cut.parts;
     fz.e = e;
     fz.f = f;
     fz.alpha = alpha;
@@ -1427,27 +1484,39 @@ alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
     fz.stride = (int)items + 1;
     fz.cc = crt_rec_consts(n, k);
     const int64_t clusters = items < P ? items : P;
-    // the counter and every cluster's list start at all ones (-1: not yet taken)
-    ce = cudaMemsetAsync(sched, 0xff, (size_t)4 * (1 + (size_t)clusters * fz.stride), stream);
-    if (ce != cudaSuccess) return cuda_status(ce);
+    // the counter and every cluster's list start at all ones (-1: not yet
+    // taken); a caller that prepared the operands in one launch set them there
+    if (!prepared) {
+        ce = cudaMemsetAsync(sched, 0xff, emul_crt_sched_words(M, N) * 4, stream);
+        if (ce != cudaSuccess) return cuda_status(ce);
+    }
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)(2 * clusters));
     lc.blockDim = dim3(kFusedThreads);
     lc.dynamicSmemBytes = kFusedSmemBytes;
     lc.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
-    lc.numAttrs = 1;
+    lc.numAttrs = prepared ? 2 : 1;   // after a kernel that lets it start early
     ce = cudaLaunchKernelEx(&lc, emul_crt_fused_pair_kernel, ta, tb, p, fz);
     if (ce != cudaSuccess) return cuda_status(ce);
+    if (!cut.rec)
+        return launch_recombine_crt(n, k, recombine_grid(M, N), stream, G, M * ldg, ldg, e, f, M,
+                                    N, alpha, beta, C, ldc, true);
     if (p.n_full < pair_tiles) {
-        crt_tail_recombine_kernel<<<(unsigned)((pair_tiles - p.n_full) * 16), 256, 0, stream>>>(
-            p, fz);
-        ce = cudaGetLastError();
+        cudaLaunchConfig_t tc = {};
+        tc.gridDim = dim3((unsigned)((pair_tiles - p.n_full) * 64));
+        tc.blockDim = dim3(256);
+        tc.stream = stream;
+        tc.attrs = attr + 1;
+        tc.numAttrs = 1;
+        ce = cudaLaunchKernelEx(&tc, crt_tail_recombine_kernel, p, fz);
     }
     return cuda_status(ce);
 }

@@ -7,6 +7,8 @@
 
 #include <cuda_bf16.h>
 
+#include <utility>
+
 #include "alp_internal.cuh"
 
 namespace alp {
@@ -19,6 +21,29 @@ __device__ __forceinline__ int frexp_exponent_of_bits(uint64_t mb) {
     if (ex == 0) return (63 - __clzll((long long)mb)) - 1073;   // subnormal
     return ex - 1022;
 }
+
+constexpr uint64_t kAbsMask = 0x7FFFFFFFFFFFFFFFull;
+
+// |x| as ordered integer keys (larger key, larger |x|): the bits of a double
+// without its sign, or of a float.  A key at or above the infinity's is Inf
+// or NaN.  The float key converts to the double bits of the same value for
+// the exponent (FP32 operands convert exactly, so frexp and the digits are
+// the same as for the double of equal value).
+template <typename T> struct ScanKey;
+template <> struct ScanKey<double> {
+    using type = uint64_t;
+    static constexpr uint64_t kInf = 0x7FF0000000000000ull;
+    __device__ static uint64_t of(uint64_t bits) { return bits & kAbsMask; }
+    __device__ static uint64_t to_double_bits(uint64_t k) { return k; }
+};
+template <> struct ScanKey<float> {
+    using type = uint32_t;
+    static constexpr uint32_t kInf = 0x7F800000u;
+    __device__ static uint32_t of(uint32_t bits) { return bits & 0x7FFFFFFFu; }
+    __device__ static uint64_t to_double_bits(uint32_t k) {
+        return (uint64_t)__double_as_longlong((double)__int_as_float((int)k));
+    }
+};
 
 // ---------------------------------------------------------------------------
 // 2. split
@@ -56,26 +81,10 @@ __device__ __forceinline__ uint64_t fixed_point_r0(double a, int e) {
     return neg ? (0ull - Y) : Y;   // two's complement of the signed value
 }
 
-template <int S, int B>
-__device__ __forceinline__ void split_digits(double a, int e, int (&d)[S]) {
-    constexpr int SH = 62 - B;   // the digit's unit in the fixed point
-    uint64_t X = fixed_point_r0(a, e);
-#pragma unroll
-    for (int p = 0; p < S; ++p) {
-        // round half to even of X / 2^SH: floor((X + 2^(SH-1) - 1 + odd) / 2^SH),
-        // odd = the parity of floor(X / 2^SH)
-        const uint64_t odd = (X >> SH) & 1;
-        const int64_t dd = (int64_t)(X + ((1ull << (SH - 1)) - 1) + odd) >> SH;
-        d[p] = (int)dd;
-        // (X - dd 2^SH) 2^B, |.| <= 2^61; SH + B = 62
-        X = (X << B) - ((uint64_t)dd << 62);
-    }
-}
-
-// The splitter of the digit schemes: s digits of B bits (split_digits).  The
-// split kernels below take a splitter object, so that other integer
+// The split kernels take a splitter object, so that other integer
 // representations of the operands (the residues of the modular scheme) reuse
-// them.
+// them: init(a, e) gives what one value's slices are formed from, next<L> its
+// L-th slice (asked for in order), pack two slices as bf16.
 // Two digits (|v| <= 256) as packed bf16: the float 1.5*2^23 + v - 1.5*2^23
 // is exactly v, and its upper 16 bits are its bf16 encoding (at most 9
 // significant bits), so no conversion instruction is needed.
@@ -85,14 +94,63 @@ __device__ __forceinline__ uint32_t pack_bf16x2(int lo, int hi) {
     return __byte_perm((uint32_t)__float_as_int(fl), (uint32_t)__float_as_int(fh), 0x7632);
 }
 
+// The digit schemes' splitter: digits of B bits.
 template <int B>
 struct DigitSplit {
-    template <int S>
-    __device__ __forceinline__ void split(double a, int e, int (&d)[S]) const {
-        split_digits<S, B>(a, e, d);
+    using State = uint64_t;
+    __device__ __forceinline__ State init(double a, int e) const { return fixed_point_r0(a, e); }
+    template <int L>
+    __device__ __forceinline__ int next(State& X) const {
+        constexpr int SH = 62 - B;   // the digit's unit in the fixed point
+        // round half to even of X / 2^SH: floor((X + 2^(SH-1) - 1 + odd) / 2^SH),
+        // odd = the parity of floor(X / 2^SH)
+        const uint64_t odd = (X >> SH) & 1;
+        const int64_t d = (int64_t)(X + ((1ull << (SH - 1)) - 1) + odd) >> SH;
+        // (X - d 2^SH) 2^B, |.| <= 2^61; SH + B = 62
+        X = (X << B) - ((uint64_t)d << 62);
+        return (int)d;
     }
     __device__ __forceinline__ uint32_t pack(int lo, int hi) const { return pack_bf16x2(lo, hi); }
 };
+
+// The S slices of two or four consecutive elements of a line, slice by slice
+// (one store per plane, so that no more than one slice of each is live).
+template <typename Sp, int... L>
+__device__ __forceinline__ void split2_planes(const Sp& sp, typename Sp::State (&u)[2], uint32_t* o,
+                                              int64_t step, std::integer_sequence<int, L...>) {
+    auto put = [&](int a, int b) {
+        *o = sp.pack(a, b);
+        o += step;
+    };
+    (put(sp.template next<L>(u[0]), sp.template next<L>(u[1])), ...);
+}
+template <int S, typename Sp>
+__device__ __forceinline__ void split2(const Sp& sp, double a0, double a1, int e,
+                                       __nv_bfloat16* out, int64_t plane) {
+    typename Sp::State u[2] = {sp.init(a0, e), sp.init(a1, e)};
+    split2_planes(sp, u, reinterpret_cast<uint32_t*>(out), plane >> 1,
+                  std::make_integer_sequence<int, S>());
+}
+template <typename Sp, int... L>
+__device__ __forceinline__ void split4_planes(const Sp& sp, typename Sp::State (&u)[4], uint2* o,
+                                              int64_t step, std::integer_sequence<int, L...>) {
+    auto put = [&](int a, int b, int c, int d) {
+        *o = make_uint2(sp.pack(a, b), sp.pack(c, d));
+        o += step;
+    };
+    (put(sp.template next<L>(u[0]), sp.template next<L>(u[1]), sp.template next<L>(u[2]),
+         sp.template next<L>(u[3])),
+     ...);
+}
+template <int S, typename Sp, typename T>
+__device__ __forceinline__ void split4(const Sp& sp, const T (&a)[4], int e, __nv_bfloat16* out,
+                                       int64_t plane) {
+    typename Sp::State u[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) u[i] = sp.init((double)a[i], e);
+    split4_planes(sp, u, reinterpret_cast<uint2*>(out), plane >> 2,
+                  std::make_integer_sequence<int, S>());
+}
 
 // A (R x K, row-major) -> out[p][r][k] (row stride kpad, zero beyond K); each
 // thread handles two consecutive k.
@@ -108,12 +166,9 @@ __global__ void split_rows_kernel(const T* __restrict__ X, int64_t R, int64_t K,
         const int64_t r = idx / half;
         const int64_t k = (idx - r * half) * 2;
         const int er = e[r];
-        int d0[S], d1[S];
-        sp.template split<S>(k < K ? (double)__ldg(X + r * ldx + k) : 0.0, er, d0);
-        sp.template split<S>(k + 1 < K ? (double)__ldg(X + r * ldx + k + 1) : 0.0, er, d1);
-        uint32_t* o = reinterpret_cast<uint32_t*>(out + r * kpad + k);
-#pragma unroll
-        for (int p = 0; p < S; ++p, o += plane >> 1) *o = sp.pack(d0[p], d1[p]);
+        split2<S>(sp, k < K ? (double)__ldg(X + r * ldx + k) : 0.0,
+                  k + 1 < K ? (double)__ldg(X + r * ldx + k + 1) : 0.0, er, out + r * kpad + k,
+                  plane);
     }
 }
 
@@ -155,22 +210,7 @@ __global__ void __launch_bounds__(THREADS, MINB) split_rows4_kernel(const T* __r
 #pragma unroll
                 for (int u = 0; u < 4; ++u) a[u] = k + u < K ? (double)__ldg(xr + k + u) : 0.0;
             }
-            // pairs packed as soon as they are split, so that only the packed
-            // words of the first pair stay live
-            uint32_t w01[S];
-            {
-                int d0[S], d1[S];
-                sp.template split<S>(a[0], er, d0);
-                sp.template split<S>(a[1], er, d1);
-#pragma unroll
-                for (int p = 0; p < S; ++p) w01[p] = sp.pack(d0[p], d1[p]);
-            }
-            int d2[S], d3[S];
-            sp.template split<S>(a[2], er, d2);
-            sp.template split<S>(a[3], er, d3);
-            uint2* o = reinterpret_cast<uint2*>(out + r * kpad + k);
-#pragma unroll
-            for (int p = 0; p < S; ++p, o += plane >> 2) *o = make_uint2(w01[p], sp.pack(d2[p], d3[p]));
+            split4<S>(sp, a, er, out + r * kpad + k, plane);
         }
     }
 }
@@ -258,20 +298,7 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_split_rows4_kernel(
         for (int64_t k = 4 * (int64_t)threadIdx.x; k < kpad; k += 4 * THREADS) {
             const double a[4] = {an[0], an[1], an[2], an[3]};
             if (k + 4 * THREADS < kpad) load4(k + 4 * THREADS, an);
-            uint32_t w01[S];
-            {
-                int d0[S], d1[S];
-                sp.template split<S>(a[0], er, d0);
-                sp.template split<S>(a[1], er, d1);
-#pragma unroll
-                for (int p = 0; p < S; ++p) w01[p] = sp.pack(d0[p], d1[p]);
-            }
-            int d2[S], d3[S];
-            sp.template split<S>(a[2], er, d2);
-            sp.template split<S>(a[3], er, d3);
-            uint2* o = reinterpret_cast<uint2*>(out + r * kpad + k);
-#pragma unroll
-            for (int p = 0; p < S; ++p, o += plane >> 2) *o = make_uint2(w01[p], sp.pack(d2[p], d3[p]));
+            split4<S>(sp, a, er, out + r * kpad + k, plane);
         }
     }
 }
@@ -297,14 +324,9 @@ __global__ void split_cols_kernel(const T* __restrict__ X, int64_t K, int64_t N,
         const int64_t j = j0 + jj;
         if (j >= N) continue;
         const int fj = f[j];
-        int d0[S], d1[S];
-        sp.template split<S>(t[jj][2 * tx], fj, d0);
-        sp.template split<S>(t[jj][2 * tx + 1], fj, d1);
         const int64_t k = k0 + 2 * tx;
         if (k >= kpad) continue;
-        uint32_t* o = reinterpret_cast<uint32_t*>(out + j * kpad + k);
-#pragma unroll
-        for (int p = 0; p < S; ++p, o += plane >> 1) *o = sp.pack(d0[p], d1[p]);
+        split2<S>(sp, t[jj][2 * tx], t[jj][2 * tx + 1], fj, out + j * kpad + k, plane);
     }
 }
 
@@ -316,7 +338,7 @@ __global__ void split_cols_kernel(const T* __restrict__ X, int64_t K, int64_t N,
 // per digit plane (256 contiguous bytes per warp).  Needs out 8-byte aligned
 // and kpad a multiple of 4 (the launch checks).
 template <typename T, int S, typename Sp>
-__global__ void __launch_bounds__(256, 3) split_cols4_kernel(
+__global__ void __launch_bounds__(256, 4) split_cols4_kernel(
     const T* __restrict__ X, int64_t K, int64_t N, int64_t ldx, const int32_t* __restrict__ f,
     __nv_bfloat16* __restrict__ out, int64_t kpad, const Sp sp) {
     __shared__ double t[32][129];
@@ -337,20 +359,8 @@ __global__ void __launch_bounds__(256, 3) split_cols4_kernel(
         const int64_t j = j0 + jj;
         if (j >= N) break;
         const int fj = f[j];
-        uint32_t w01[S];
-        {
-            int d0[S], d1[S];
-            sp.template split<S>(t[jj][tx], fj, d0);
-            sp.template split<S>(t[jj][32 + tx], fj, d1);
-#pragma unroll
-            for (int p = 0; p < S; ++p) w01[p] = sp.pack(d0[p], d1[p]);
-        }
-        int d2[S], d3[S];
-        sp.template split<S>(t[jj][64 + tx], fj, d2);
-        sp.template split<S>(t[jj][96 + tx], fj, d3);
-        uint2* o = reinterpret_cast<uint2*>(out + j * kpad + k);
-#pragma unroll
-        for (int p = 0; p < S; ++p, o += plane >> 2) *o = make_uint2(w01[p], sp.pack(d2[p], d3[p]));
+        const double a[4] = {t[jj][tx], t[jj][32 + tx], t[jj][64 + tx], t[jj][96 + tx]};
+        split4<S>(sp, a, fj, out + j * kpad + k, plane);
     }
 }
 

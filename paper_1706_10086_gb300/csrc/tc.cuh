@@ -40,6 +40,15 @@ __device__ __forceinline__ void cluster_sync_all() {
                      : "memory");
 }
 
+// ---- dependent launches: a kernel launched with programmatic stream
+// serialization may start while its predecessor drains.  pdl_launch lets the
+// successor start, pdl_wait returns once the predecessor has completed and its
+// writes are visible (at once when the launch had no such attribute). ----
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- TMEM allocation (one warp executes each) ----
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
