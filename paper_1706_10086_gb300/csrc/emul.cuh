@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include "alp_internal.cuh"
+#include "crt.cuh"
 
 namespace alp {
 
@@ -52,8 +53,9 @@ constexpr int kCrtMaxModuli = 16;
 // reduction's range.
 constexpr int64_t kCrtMaxK = 1023 * 64;
 int crt_bits(int64_t K, int n);
-// y[l] = (Mn / m_l)^-1 mod m_l for the first n moduli, 0 past them (host).
-void crt_weights(int n, uint8_t (&y)[kCrtMaxModuli]);
+// The weighted reductions of the first n moduli's sums (crt.cuh), zeros past
+// them (host).
+void crt_weights(int n, CrtByte (&b)[kCrtMaxModuli]);
 template <typename T>
 alp_status emul_split_crt(int64_t R, int64_t K, const T* X, int64_t ldx, int trans,
                           const int32_t* exps, int n, __nv_bfloat16* out, int64_t kpad, int k,

@@ -43,7 +43,7 @@ namespace {
 // Per modulus count n: the weights and the reconstruction constants that do
 // not depend on k, formed once per process.
 struct CrtTables {
-    uint8_t y[kCrtMaxModuli + 1][kCrtMaxModuli] = {};
+    CrtByte byte[kCrtMaxModuli + 1][kCrtMaxModuli] = {};   // of the weight y_l = (Mn/m_l)^-1 mod m_l
     CrtRecConsts rec[kCrtMaxModuli + 1] = {};
     CrtTables() {
         for (int n = 1; n <= kCrtMaxModuli; ++n) {
@@ -52,8 +52,11 @@ struct CrtTables {
                 uint32_t r = 1;   // Mn / m_l mod m_l = prod_{i != l} m_i mod m_l
                 for (int i = 0; i < n; ++i)
                     if (i != l) r = (r * (crt_modulus(i) % m)) % m;
-                for (uint32_t w = 1; w < m; ++w)
-                    if ((r * w) % m == 1u) y[n][l] = (uint8_t)w;
+                uint32_t y = 1;
+                while (y < m && (r * y) % m != 1u) ++y;
+                const int shift = crt_symmetric(y * crt_pow2_mod(31, m) % m, m);
+                byte[n][l] = {(int)crt_byte_weights(m, 0, y), 0x4B400000 - shift,
+                              12582912.0f + (float)((m - 1) / 2), 1.0f / (float)m, (float)m};
             }
             CrtRecConsts& c = rec[n];
             unsigned __int128 M = 1;
@@ -79,9 +82,9 @@ const CrtTables& crt_tables() {
 }
 }  // namespace
 
-void crt_weights(int n, uint8_t (&y)[kCrtMaxModuli]) {
+void crt_weights(int n, CrtByte (&b)[kCrtMaxModuli]) {
     for (int l = 0; l < kCrtMaxModuli; ++l)
-        y[l] = n >= 1 && n <= kCrtMaxModuli ? crt_tables().y[n][l] : 0;
+        b[l] = n >= 1 && n <= kCrtMaxModuli ? crt_tables().byte[n][l] : CrtByte{};
 }
 
 // The splitter.  A' = RN(a 2^(k - e)) is formed as U = A' + kSplitBias, an
@@ -112,23 +115,6 @@ void crt_weights(int n, uint8_t (&y)[kCrtMaxModuli]) {
 // integer's bf16 encoding in its upper 16 bits, so packing two residues is
 // one byte permutation.
 constexpr uint64_t kSplitBias = 0x4338000000000000ull;   // the encoding of 1.5 2^52
-
-__host__ __device__ constexpr int crt_symmetric(uint32_t r, uint32_t m) {
-    return r > m / 2 - (m % 2 == 0 ? 1 : 0) ? (int)r - (int)m : (int)r;
-}
-// Bytes 256^i0 .. 256^(i0+3) mod m, symmetric.
-__host__ __device__ constexpr uint32_t crt_byte_weights(uint32_t m, int i0) {
-    uint32_t w = 0;
-    for (int i = 0; i < 4; ++i)
-        w |= ((uint32_t)crt_symmetric(crt_pow2_mod(8 * (i0 + i), m), m) & 0xFFu) << (8 * i);
-    return w;
-}
-// d = c + the dot product of a's unsigned and b's signed bytes.
-__device__ __forceinline__ int dp4a_us(uint32_t a, int b, int c) {
-    int d;
-    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
 
 // The constants of modulus l, as literals: kept in the constant bank, the
 // weights would be hoisted into registers, which spill.
@@ -192,7 +178,7 @@ struct CrtSplit {
     template <int L>
     __device__ __forceinline__ int next(State& u) const {
         using C = CrtSplitConsts<L>;
-        const int f = dp4a_us((uint32_t)(u >> 32), C::whi, dp4a_us((uint32_t)u, C::wlo, 0x4B400000));
+        const int f = crt_dp4a((uint32_t)(u >> 32), C::whi, crt_dp4a((uint32_t)u, C::wlo, 0x4B400000));
         const float x = __fadd_rn(__int_as_float(f), -C::off);
         const float q = __fadd_rn(__fmaf_rn(x, C::inv, 12582912.0f), -12582912.0f);
         return __float_as_int(__fmaf_rn(-q, C::mf, x));

@@ -114,7 +114,7 @@ constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*align*/ + 256 /*barrie
 
 struct EmulGemmParams {
     int64_t M, N, K;
-    int s, digit_bits, trim, crt;
+    int s, digit_bits, trim, modular;
     int32_t* G;
     int64_t ldg, gplane;
     int tiles_m, tiles_n, group_m;
@@ -130,8 +130,8 @@ struct EmulGemmParams {
     // test hook: block 0's producer arms pipeline stage inject_skip_it (its
     // running stage count) without issuing the copies (-1: off)
     int64_t inject_skip_it;
-    // modular scheme: y_l = (Mn / m_l)^-1 mod m_l, the weight of residue l
-    uint8_t crt_y[kCrtMaxModuli];
+    // modular scheme: the weighted reduction of modulus l's sums
+    CrtByte crt[kCrtMaxModuli];
 };
 
 // K chunk of pair (p, q): the largest multiple of 64 with |partial sums| <= 2^24,
@@ -238,8 +238,9 @@ __device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const u
     const int row = quarter * 32 + lane;
     const int gm = m0 + row;
     uint32_t acc[128];
+    const uint32_t zero = prm.modular ? kCrtSumZero : 0u;
 #pragma unroll
-    for (int i = 0; i < 128; ++i) acc[i] = 0;
+    for (int i = 0; i < 128; ++i) acc[i] = zero;
     int t_group = 2;
     for (int job = 0; job < njobs; ++job) {
         const uint32_t b = job & 1;
@@ -253,11 +254,11 @@ __device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const u
         __syncwarp();
         if (lane == 0) hand_back(acce, acce_remote, agg, b, job, ew + 2, tmo, abort_flag, prm.err);
         const uint32_t jd = jobs[job];
-        if (job_last(jd) && prm.crt) {
+        if (job_last(jd) && prm.modular) {
             // modular scheme: plane l of modulus m_l receives x = (Q y_l) mod
             // m_l = (P y_l) mod m_l, one byte per column (rows padded as below)
             const int l = job_p(jd) - 1;
-            const uint32_t m = crt_modulus(l), magic = crt_magic(m), y = prm.crt_y[l];
+            const CrtByte k = prm.crt[l];
             uint8_t* g = reinterpret_cast<uint8_t*>(prm.G) + (int64_t)l * prm.gplane +
                          (int64_t)gm * prm.ldg + n0 + half * 128;
             const uint32_t do_store = gm < prm.M ? 1u : 0u;
@@ -265,18 +266,12 @@ __device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const u
             for (int i = 0; i < 8; ++i) {
                 uint32_t w[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = 16 * i + 4 * q;
-                    w[q] = crt_mod(crt_residue((int32_t)acc[c], m, magic) * y, m, magic) |
-                           crt_mod(crt_residue((int32_t)acc[c + 1], m, magic) * y, m, magic) << 8 |
-                           crt_mod(crt_residue((int32_t)acc[c + 2], m, magic) * y, m, magic) << 16 |
-                           crt_mod(crt_residue((int32_t)acc[c + 3], m, magic) * y, m, magic) << 24;
-                }
+                for (int x = 0; x < 4; ++x) w[x] = crt_bytes4(acc + 16 * i + 4 * x, k);
                 store4_and_zero(reinterpret_cast<int32_t*>(g + 16 * i), do_store, w[0], w[1],
                                 w[2], w[3]);
             }
 #pragma unroll
-            for (int i = 0; i < 128; ++i) acc[i] = 0;
+            for (int i = 0; i < 128; ++i) acc[i] = zero;
         } else if (job_last(jd)) {
             // plane of G: t - 2 for the digit pair (p, q), t = p + q
             t_group = job_p(jd) + job_q(jd);
@@ -331,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             t_lo = (int)(r & 15u) + 2;
             t_hi = (int)(r >> 4) + 2;
         }
-        *njobs_slot = build_jobs(prm.s, (int)prm.K, prm.digit_bits, prm.trim != 0, prm.crt != 0,
+        *njobs_slot = build_jobs(prm.s, (int)prm.K, prm.digit_bits, prm.trim != 0, prm.modular != 0,
                                  t_lo, t_hi, jobs);
         fence_barrier_init();
     }
@@ -536,7 +531,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             t_lo = (int)(r & 15u) + 2;
             t_hi = (int)(r >> 4) + 2;
         }
-        *njobs_slot = build_jobs(prm.s, (int)prm.K, prm.digit_bits, prm.trim != 0, prm.crt != 0,
+        *njobs_slot = build_jobs(prm.s, (int)prm.K, prm.digit_bits, prm.trim != 0, prm.modular != 0,
                                  t_lo, t_hi, jobs);
         fence_barrier_init();
     }
@@ -888,7 +883,7 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
             pair_tile_origin(prm, pid, rank, m0, n0);
             const int gm = m0 + row;
 #pragma unroll
-            for (int x = 0; x < 128; ++x) acc[x] = 0;
+            for (int x = 0; x < 128; ++x) acc[x] = kCrtSumZero;
             for (int c = 0; c < cpm; ++c, ++job) {
                 const uint32_t b = job & 1;
                 if (!mbar_wait_bounded(&accf[b], (job >> 1) & 1, tmo, abort_flag, prm.err)) {
@@ -909,26 +904,15 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
             }
             if (!ok) break;
             // plane q receives x = (Q y_q) mod m_q, one byte per column
-            const uint32_t m = crt_modulus(q), magic = crt_magic(m), y = prm.crt_y[q];
+            const CrtByte kb = prm.crt[q];
             uint8_t* g = reinterpret_cast<uint8_t*>(prm.G) + (int64_t)q * prm.gplane +
                          (int64_t)gm * prm.ldg + n0 + half * 128;
             if (gm < prm.M) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const int c = 16 * i + 4 * x;
-                        w[x] = crt_mod(crt_residue((int32_t)acc[c], m, magic) * y, m, magic) |
-                               crt_mod(crt_residue((int32_t)acc[c + 1], m, magic) * y, m, magic)
-                                   << 8 |
-                               crt_mod(crt_residue((int32_t)acc[c + 2], m, magic) * y, m, magic)
-                                   << 16 |
-                               crt_mod(crt_residue((int32_t)acc[c + 3], m, magic) * y, m, magic)
-                                   << 24;
-                    }
-                    *reinterpret_cast<uint4*>(g + 16 * i) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
+                for (int i = 0; i < 8; ++i)
+                    *reinterpret_cast<uint4*>(g + 16 * i) = make_uint4(
+                        crt_bytes4(acc + 16 * i, kb), crt_bytes4(acc + 16 * i + 4, kb),
+                        crt_bytes4(acc + 16 * i + 8, kb), crt_bytes4(acc + 16 * i + 12, kb));
             }
         }
         if (ok && fz.rec && it < prm.n_full) {
@@ -1264,9 +1248,8 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     p.s = s;
     p.digit_bits = digit_bits;
     p.trim = trim ? 1 : 0;
-    p.crt = crt ? 1 : 0;
-    if (crt) crt_weights(s, p.crt_y);
-    else std::fill(p.crt_y, p.crt_y + kCrtMaxModuli, uint8_t(0));
+    p.modular = crt ? 1 : 0;
+    crt_weights(crt ? s : 0, p.crt);
     p.G = G;
     p.ldg = ldg;
     p.gplane = M * ldg;
@@ -1442,8 +1425,8 @@ alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
     p.s = n;
     p.digit_bits = kDigitBits;
     p.trim = 0;
-    p.crt = 1;
-    crt_weights(n, p.crt_y);
+    p.modular = 1;
+    crt_weights(n, p.crt);
     p.G = reinterpret_cast<int32_t*>(G);
     p.ldg = ldg;
     p.gplane = M * ldg;
