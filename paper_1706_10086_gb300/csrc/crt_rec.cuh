@@ -9,8 +9,13 @@
 // with Mn / m_g (three or four 32-bit limbs) serves three moduli.  c is the
 // nearest integer to sum_g X_g / m_g, formed in 6.58 fixed point from
 // F_g = round(2^58 / m_g) with an error below 2^-30 (|P| / Mn <= 1/2 - 2^-19 by
-// the choice of k, so the rounding is exact), and P = sum - c Mn follows by one
-// carry pass, exact modulo 2^128, which holds it.
+// the choice of k, so the rounding is exact), and P = sum + c (2^128 - Mn) follows
+// by one carry pass, exact modulo 2^128, which holds it.
+//
+// The reconstruction is bound by the integer ALU pipe (half the rate of the
+// multiply-add pipe; 55 % active at 2048^2 with 100 of 208 instructions on it),
+// so additions go into wide multiply-adds where they can: the rounding constant
+// starts the quotient sum and the multiple of Mn is added limb by limb.
 #pragma once
 
 #include <cstdint>
@@ -23,7 +28,7 @@ namespace alp {
 constexpr int kCrtMaxGroups = 6;   // ceil(16 / 3)
 
 struct CrtRecConsts {
-    uint32_t mn[4];                   // Mn, 32-bit limbs
+    uint32_t nm[4];                   // 2^128 - Mn, 32-bit limbs
     uint32_t mg[kCrtMaxGroups][4];    // Mn / m_g per group
     uint32_t fg_lo[kCrtMaxGroups];    // F_g = round(2^58 / m_g), low and high words
     uint32_t fg_hi[kCrtMaxGroups];
@@ -40,6 +45,18 @@ __device__ __forceinline__ uint64_t crt_mad_wide(uint32_t a, uint32_t b, uint64_
     return d;
 }
 
+// sum_i a_i 2^(32 i) + c (2^128 - Mn) modulo 2^128.
+__device__ __forceinline__ void crt_carry(uint64_t a0, uint64_t a1, uint64_t a2, uint64_t a3,
+                                          uint32_t c, const CrtRecConsts& cc, int64_t& hi,
+                                          uint64_t& lo) {
+    a0 = crt_mad_wide(c, cc.nm[0], a0);
+    a1 = crt_mad_wide(c, cc.nm[1], a1) + (a0 >> 32);
+    a2 = crt_mad_wide(c, cc.nm[2], a2) + (a1 >> 32);
+    const uint32_t w3 = (uint32_t)a3 + c * cc.nm[3] + (uint32_t)(a2 >> 32);
+    lo = (a1 << 32) | (uint32_t)a0;
+    hi = (int64_t)(((uint64_t)w3 << 32) | (uint32_t)a2);
+}
+
 // P (signed 128-bit hi:lo) of four adjacent columns whose residue bytes are
 // the bytes of v[l], l < S (byte u = column u).  Every group's constants are
 // read once for the four columns.  The limbs of Mn / m_g that can be nonzero:
@@ -53,7 +70,7 @@ __device__ __forceinline__ void crt_reconstruct4(const uint32_t (&v)[S], const C
     uint64_t a0[4], a1[4], a2[4], a3[4], q[4];
     uint32_t qh[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) a0[u] = a1[u] = a2[u] = a3[u] = q[u] = 0, qh[u] = 0;
+    for (int u = 0; u < 4; ++u) a0[u] = a1[u] = a2[u] = a3[u] = 0, q[u] = 1ull << 57, qh[u] = 0;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         // X_g by two-way dot products: every weight m_g / m_l is a product of
@@ -93,22 +110,11 @@ __device__ __forceinline__ void crt_reconstruct4(const uint32_t (&v)[S], const C
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        // sum_g X_g F_g < 2^62 (X_g / m_g < 3, at most six groups), so its
-        // value modulo 2^64 is the value
-        const uint64_t qt = q[u] + ((uint64_t)qh[u] << 32);
-        const uint32_t c = (uint32_t)((qt + (1ull << 57)) >> 58);
-        // the column sums are below 6 * 2^26 * 2^32 < 2^61: signed 64-bit
-        // holds each step of the carry pass
-        int64_t t = (int64_t)a0[u] - (int64_t)((uint64_t)c * cc.mn[0]);
-        const uint32_t w0 = (uint32_t)t;
-        t = (t >> 32) + (int64_t)a1[u] - (int64_t)((uint64_t)c * cc.mn[1]);
-        const uint32_t w1 = (uint32_t)t;
-        t = (t >> 32) + (int64_t)a2[u] - (int64_t)((uint64_t)c * cc.mn[2]);
-        const uint32_t w2 = (uint32_t)t;
-        t = (t >> 32) + (int64_t)a3[u] - (int64_t)((uint64_t)c * cc.mn[3]);
-        const uint32_t w3 = (uint32_t)t;
-        hi[u] = (int64_t)(((uint64_t)w3 << 32) | w2);
-        lo[u] = ((uint64_t)w1 << 32) | w0;
+        // 2^57 + sum_g X_g F_g < 2^62 + 2^57 (X_g / m_g < 3, at most six groups),
+        // so its value modulo 2^64 is the value
+        const uint32_t c = ((uint32_t)(q[u] >> 32) + qh[u]) >> 26;
+        // the column sums stay below 6 * 2^26 * 2^32 + 2^37 < 2^61
+        crt_carry(a0[u], a1[u], a2[u], a3[u], c, cc, hi[u], lo[u]);
     }
 }
 
@@ -123,7 +129,7 @@ __device__ __forceinline__ void crt_reconstruct4_n(const uint32_t (&v)[16], int 
     uint64_t a0[4], a1[4], a2[4], a3[4], q[4];
     uint32_t qh[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) a0[u] = a1[u] = a2[u] = a3[u] = q[u] = 0, qh[u] = 0;
+    for (int u = 0; u < 4; ++u) a0[u] = a1[u] = a2[u] = a3[u] = 0, q[u] = 1ull << 57, qh[u] = 0;
     const bool four = n > 15;
 #pragma unroll
     for (int g = 0; g < kCrtMaxGroups; ++g) {
@@ -160,18 +166,8 @@ __device__ __forceinline__ void crt_reconstruct4_n(const uint32_t (&v)[16], int 
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         // as in crt_reconstruct4
-        const uint64_t qt = q[u] + ((uint64_t)qh[u] << 32);
-        const uint32_t c = (uint32_t)((qt + (1ull << 57)) >> 58);
-        int64_t t = (int64_t)a0[u] - (int64_t)((uint64_t)c * cc.mn[0]);
-        const uint32_t w0 = (uint32_t)t;
-        t = (t >> 32) + (int64_t)a1[u] - (int64_t)((uint64_t)c * cc.mn[1]);
-        const uint32_t w1 = (uint32_t)t;
-        t = (t >> 32) + (int64_t)a2[u] - (int64_t)((uint64_t)c * cc.mn[2]);
-        const uint32_t w2 = (uint32_t)t;
-        t = (t >> 32) + (int64_t)a3[u] - (int64_t)((uint64_t)c * cc.mn[3]);
-        const uint32_t w3 = (uint32_t)t;
-        hi[u] = (int64_t)(((uint64_t)w3 << 32) | w2);
-        lo[u] = ((uint64_t)w1 << 32) | w0;
+        const uint32_t c = ((uint32_t)(q[u] >> 32) + qh[u]) >> 26;
+        crt_carry(a0[u], a1[u], a2[u], a3[u], c, cc, hi[u], lo[u]);
     }
 }
 

@@ -61,7 +61,7 @@ struct CrtTables {
             CrtRecConsts& c = rec[n];
             unsigned __int128 M = 1;
             for (int l = 0; l < n; ++l) M *= crt_modulus(l);
-            for (int i = 0; i < 4; ++i) c.mn[i] = (uint32_t)(M >> (32 * i));
+            for (int i = 0; i < 4; ++i) c.nm[i] = (uint32_t)((0 - M) >> (32 * i));
             for (int g = 0; 3 * g < n && g < kCrtMaxGroups; ++g) {
                 uint32_t mg = 1;
                 for (int l = 3 * g; l < 3 * g + 3 && l < n; ++l) mg *= crt_modulus(l);

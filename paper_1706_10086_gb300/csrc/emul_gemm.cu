@@ -1370,7 +1370,7 @@ size_t emul_crt_sched_words(int64_t M, int64_t N) {
 // those tiles join the tail: 2048^3 and 3000 x 1500 x 2100 ran 435 and 553 us
 // with it exposed at the end of the launch, 323 and 399 as two launches).
 // Otherwise every tile is reconstructed by the following kernel, which takes
-// 0.55 us per tile with all SMs.
+// 0.44 us per tile with all SMs.
 struct FusedCut {
     int64_t n_full;
     int parts;
