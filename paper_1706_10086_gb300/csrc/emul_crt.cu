@@ -111,9 +111,6 @@ void crt_weights(int n, CrtByte (&b)[kCrtMaxModuli]) {
 // half-integer, and |r| <= m / 2 + 0.04, an integer at most 128.  Six instructions per modulus and none to cut A' up (three 13-bit
 // chunks turned into floats and three fmas each before, six and some 14 per
 // value, and eleven integer ones for k >= 52: 2048 x 2048 with 15 moduli, k = 52).
-// A float holding an integer of at most 8 significant bits has that
-// integer's bf16 encoding in its upper 16 bits, so packing two residues is
-// one byte permutation.
 constexpr uint64_t kSplitBias = 0x4338000000000000ull;   // the encoding of 1.5 2^52
 
 // The constants of modulus l, as literals: kept in the constant bank, the
@@ -173,20 +170,21 @@ struct CrtSplit {
         return (int64_t)bits < 0 ? kSplitBias - u : kSplitBias + u;
     }
     // What the residues are formed from, and the residue of modulus L.
+    template <int S, typename T>
     using State = uint64_t;
-    __device__ __forceinline__ State init(double a, int e) const { return biased(a, e); }
+    template <int S>
+    __device__ __forceinline__ uint64_t init(double a, int e) const {
+        return biased(a, e);
+    }
     template <int L>
-    __device__ __forceinline__ int next(State& u) const {
+    __device__ __forceinline__ int next(uint64_t& u) const {
         using C = CrtSplitConsts<L>;
         const int f = crt_dp4a((uint32_t)(u >> 32), C::whi, crt_dp4a((uint32_t)u, C::wlo, 0x4B400000));
         const float x = __fadd_rn(__int_as_float(f), -C::off);
         const float q = __fadd_rn(__fmaf_rn(x, C::inv, 12582912.0f), -12582912.0f);
         return __float_as_int(__fmaf_rn(-q, C::mf, x));
     }
-    // two residues (float encodings) as packed bf16
-    __device__ __forceinline__ uint32_t pack(int lo, int hi) const {
-        return __byte_perm((uint32_t)lo, (uint32_t)hi, 0x7632);
-    }
+    __device__ __forceinline__ uint32_t pack(int lo, int hi) const { return pack_bf16x2(lo, hi); }
 };
 
 template <typename T>

@@ -7,6 +7,7 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
 #include <utility>
 
 #include "alp_internal.cuh"
@@ -48,75 +49,113 @@ template <> struct ScanKey<float> {
 // ---------------------------------------------------------------------------
 // 2. split
 // ---------------------------------------------------------------------------
-// Digits of a * 2^-e.  r0 = a * 2^-e is held as a 64-bit fixed-point number
-// with 62 fraction bits, rounded to odd (truncate, then set the last bit if
-// anything was cut off): every later rounding happens at least 2 bits above
-// that last bit, so the digits equal those of the exact value ((s-1) b + 2 <=
-// 62 - b).  Each step is d = round-half-even(X / 2^(62-b)), X = (X - d 2^(62-b))
-// * 2^b, which is x = r * 2^b, d = nearest integer (ties to even), r = x - d in
-// fixed point.
-__device__ __forceinline__ uint64_t fixed_point_r0(double a, int e) {
-    const uint64_t bits = (uint64_t)__double_as_longlong(a);
-    const bool neg = (bits >> 63) != 0;
-    const int ex = (int)((bits >> 52) & 0x7FF);
-    uint64_t m = bits & ((1ull << 52) - 1);
-    int E;
-    if (ex == 0x7FF) {
-        m = 0;
-        E = 0;   // Inf/NaN: reported by the scan; digits 0
-    } else if (ex == 0) {
-        E = -1074;
-    } else {
-        m |= 1ull << 52;
-        E = ex - 1075;
-    }
-    const int sh = E - e + 62;
-    uint64_t Y;
-    if (m == 0) Y = 0;
-    else if (sh >= 0) Y = m << (sh > 63 ? 63 : sh);
-    else if (sh > -64) {
-        const int r = -sh;
-        Y = (m >> r) | ((m & ((1ull << r) - 1)) != 0 ? 1ull : 0ull);
-    } else Y = 1;   // nonzero but below 2^-62: sticky bit only
-    return neg ? (0ull - Y) : Y;   // two's complement of the signed value
-}
-
 // The split kernels take a splitter object, so that other integer
 // representations of the operands (the residues of the modular scheme) reuse
-// them: init(a, e) gives what one value's slices are formed from, next<L> its
-// L-th slice (asked for in order), pack two slices as bf16.
-// Two digits (|v| <= 256) as packed bf16: the float 1.5*2^23 + v - 1.5*2^23
-// is exactly v, and its upper 16 bits are its bf16 encoding (at most 9
-// significant bits), so no conversion instruction is needed.
+// them: init<S>(a, e) gives what the S slices of one value are formed from,
+// next<L> its L-th slice (asked for in order) as the encoding of a float, pack
+// two of those as bf16: a float holding an integer of at most 8 significant
+// bits has that integer's bf16 encoding in its upper 16 bits, so packing is
+// one byte permutation.
 __device__ __forceinline__ uint32_t pack_bf16x2(int lo, int hi) {
-    const float fl = __int_as_float(0x4B400000 + lo) - 12582912.0f;
-    const float fh = __int_as_float(0x4B400000 + hi) - 12582912.0f;
-    return __byte_perm((uint32_t)__float_as_int(fl), (uint32_t)__float_as_int(fh), 0x7632);
+    return __byte_perm((uint32_t)lo, (uint32_t)hi, 0x7632);
 }
 
-// The digit schemes' splitter: digits of B bits.
+// Digits of a * 2^-e.  |a| 2^-e is held as a 64-bit fixed-point number Y with 62
+// fraction bits, rounded to odd (truncate, then set the last bit if anything
+// was cut off): every later rounding happens at least 2 bits above that last
+// bit, so the digits equal those of the exact value ((s-1) b + 2 <= 62 - b).
+// T: the mantissa with its leading one at bit 61, D: how far down it belongs.
+__device__ __forceinline__ uint64_t fixed_point_mag(uint64_t T, int D) {
+    const int d = D < 0 ? 0 : D > 63 ? 63 : D;
+    const uint64_t Y = T >> d;
+    return Y | ((Y << d) != T ? 1ull : 0ull);
+}
+__device__ __forceinline__ uint64_t fixed_point_mag(double a, int e) {
+    const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
+    const int ex = (int)((hi >> 20) & 0x7FF);
+    // Inf/NaN are reported by the scan (digits 0); subnormals have no hidden bit
+    const uint32_t mh = ex == 0x7FF ? 0u : (hi & 0xFFFFFu) | (ex ? 0x100000u : 0u);
+    const uint64_t m = ((uint64_t)mh << 32) | (ex == 0x7FF ? 0u : lo);
+    return fixed_point_mag(m << 9, e + 1022 - (ex ? ex : 1));
+}
+__device__ __forceinline__ bool is_negative(double a) { return __double2hiint(a) < 0; }
+
+// The digit schemes' splitter: digits of B bits, d_p = R_p - 2^B R_{p-1} with R_p
+// the signed value X = +-Y rounded half to even at bit SH_p = 62 - B p (what
+// rounding digit by digit, each from the exact remainder of the last, gives).
+// Rounded half up instead, d_p is the signed B-bit field of X above SH_p plus
+// the bit below it, read from one field of B + 1 bits; the two roundings differ
+// only when X ends in exactly half a unit of some digit (at one digit, since
+// nothing is left below it) above an even multiple: then half up of -X, negated,
+// is half down of X, which is the even one.  Five instructions per digit where
+// the digit-by-digit remainder in 64 bits took about fourteen (operands of 2048^3
+// with 8 slices 62 -> 53 us).
+//
+// Floats are cut digit by digit in float arithmetic: x = a 2^(B - e), d = x
+// rounded to the nearest integer, ties to even, by adding 1.5 2^23, and x = (x -
+// d) 2^B, every step exact (x keeps at most a's 24 bits; what a scaling below
+// the normal range could lose is far below the last digit's half).  Converted
+// to double first (an FP64 operation each) and cut as one, the operands of an
+// FP32 4096^3 took 112 us, now 67 (floor 50).
 template <int B>
 struct DigitSplit {
-    using State = uint64_t;
-    __device__ __forceinline__ State init(double a, int e) const { return fixed_point_r0(a, e); }
+    struct Wide {
+        uint32_t lo, hi;   // X, negated where half up would round to the odd side
+        float sgn, off;    // 1 or -1, and -1.5 2^23 times it
+    };
+    struct Single {
+        float x;
+    };
+    template <int S, typename T>
+    using State = std::conditional_t<sizeof(T) == 8, Wide, Single>;
+    template <int S>
+    static constexpr uint64_t half_bits() {
+        uint64_t m = 0;
+        for (int p = 1; p <= S; ++p) m |= 1ull << (61 - B * p);
+        return m;
+    }
+    template <int S>
+    __device__ __forceinline__ Wide init(double a, int e) const {
+        const uint64_t Y = fixed_point_mag(a, e), last = Y & (0ull - Y);
+        const bool neg = __double2hiint(a) < 0;
+        // in a tie the bit above the lowest set one is the parity of Y's
+        // neighbour below, so opposite for -Y
+        const bool minus = (last & half_bits<S>()) != 0 ? (Y & (last << 1)) == 0 : neg;
+        const uint64_t s = minus ? ~0ull : 0ull, X = (Y ^ s) - s;
+        const float sgn = minus == neg ? 1.0f : -1.0f;
+        return {(uint32_t)X, (uint32_t)(X >> 32), sgn, -12582912.0f * sgn};
+    }
+    template <int S>
+    __device__ __forceinline__ Single init(float a, int e) const {
+        // 2^(B - e) as two normal factors (e is the same along a line)
+        const int k = min(max(B - e, -240), 240), k1 = k / 2;
+        return {a * __int_as_float((k1 + 127) << 23) * __int_as_float((k - k1 + 127) << 23)};
+    }
     template <int L>
-    __device__ __forceinline__ int next(State& X) const {
-        constexpr int SH = 62 - B;   // the digit's unit in the fixed point
-        // round half to even of X / 2^SH: floor((X + 2^(SH-1) - 1 + odd) / 2^SH),
-        // odd = the parity of floor(X / 2^SH)
-        const uint64_t odd = (X >> SH) & 1;
-        const int64_t d = (int64_t)(X + ((1ull << (SH - 1)) - 1) + odd) >> SH;
-        // (X - d 2^SH) 2^B, |.| <= 2^61; SH + B = 62
-        X = (X << B) - ((uint64_t)d << 62);
-        return (int)d;
+    __device__ __forceinline__ int next(Wide& u) const {
+        constexpr int SH = 62 - B * (L + 1);
+        constexpr int k = 64 - SH - B;   // the field's top bit to bit 63
+        int v;                           // the field with the bit below it, signed
+        if constexpr (L == 0) v = (int)u.hi >> (SH - 33);
+        else if constexpr (k < 32) v = (int)__funnelshift_l(u.lo, u.hi, k) >> (31 - B);
+        else v = (int)(u.lo << (k - 32)) >> (31 - B);
+        // 0x4B400000 + ((v + 1) >> 1): the encoding of 1.5 2^23 + d
+        const float f = __int_as_float((int)(((uint32_t)v + 0x96800001u) >> 1));
+        return __float_as_int(__fmaf_rn(f, u.sgn, u.off));
+    }
+    template <int L>
+    __device__ __forceinline__ int next(Single& u) const {
+        const float d = __fadd_rn(__fadd_rn(u.x, 12582912.0f), -12582912.0f);
+        u.x = __fmul_rn(__fadd_rn(u.x, -d), (float)(1 << B));
+        return __float_as_int(d);
     }
     __device__ __forceinline__ uint32_t pack(int lo, int hi) const { return pack_bf16x2(lo, hi); }
 };
 
 // The S slices of two or four consecutive elements of a line, slice by slice
 // (one store per plane, so that no more than one slice of each is live).
-template <typename Sp, int... L>
-__device__ __forceinline__ void split2_planes(const Sp& sp, typename Sp::State (&u)[2], uint32_t* o,
+template <typename Sp, typename State, int... L>
+__device__ __forceinline__ void split2_planes(const Sp& sp, State (&u)[2], uint32_t* o,
                                               int64_t step, std::integer_sequence<int, L...>) {
     auto put = [&](int a, int b) {
         *o = sp.pack(a, b);
@@ -124,15 +163,15 @@ __device__ __forceinline__ void split2_planes(const Sp& sp, typename Sp::State (
     };
     (put(sp.template next<L>(u[0]), sp.template next<L>(u[1])), ...);
 }
-template <int S, typename Sp>
-__device__ __forceinline__ void split2(const Sp& sp, double a0, double a1, int e,
-                                       __nv_bfloat16* out, int64_t plane) {
-    typename Sp::State u[2] = {sp.init(a0, e), sp.init(a1, e)};
+template <int S, typename Sp, typename T>
+__device__ __forceinline__ void split2(const Sp& sp, T a0, T a1, int e, __nv_bfloat16* out,
+                                       int64_t plane) {
+    typename Sp::template State<S, T> u[2] = {sp.template init<S>(a0, e), sp.template init<S>(a1, e)};
     split2_planes(sp, u, reinterpret_cast<uint32_t*>(out), plane >> 1,
                   std::make_integer_sequence<int, S>());
 }
-template <typename Sp, int... L>
-__device__ __forceinline__ void split4_planes(const Sp& sp, typename Sp::State (&u)[4], uint2* o,
+template <typename Sp, typename State, int... L>
+__device__ __forceinline__ void split4_planes(const Sp& sp, State (&u)[4], uint2* o,
                                               int64_t step, std::integer_sequence<int, L...>) {
     auto put = [&](int a, int b, int c, int d) {
         *o = make_uint2(sp.pack(a, b), sp.pack(c, d));
@@ -145,9 +184,9 @@ __device__ __forceinline__ void split4_planes(const Sp& sp, typename Sp::State (
 template <int S, typename Sp, typename T>
 __device__ __forceinline__ void split4(const Sp& sp, const T (&a)[4], int e, __nv_bfloat16* out,
                                        int64_t plane) {
-    typename Sp::State u[4];
+    typename Sp::template State<S, T> u[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) u[i] = sp.init((double)a[i], e);
+    for (int i = 0; i < 4; ++i) u[i] = sp.template init<S>(a[i], e);
     split4_planes(sp, u, reinterpret_cast<uint2*>(out), plane >> 2,
                   std::make_integer_sequence<int, S>());
 }
@@ -166,9 +205,8 @@ __global__ void split_rows_kernel(const T* __restrict__ X, int64_t R, int64_t K,
         const int64_t r = idx / half;
         const int64_t k = (idx - r * half) * 2;
         const int er = e[r];
-        split2<S>(sp, k < K ? (double)__ldg(X + r * ldx + k) : 0.0,
-                  k + 1 < K ? (double)__ldg(X + r * ldx + k + 1) : 0.0, er, out + r * kpad + k,
-                  plane);
+        split2<S>(sp, k < K ? __ldg(X + r * ldx + k) : T(0),
+                  k + 1 < K ? __ldg(X + r * ldx + k + 1) : T(0), er, out + r * kpad + k, plane);
     }
 }
 
@@ -190,7 +228,7 @@ __global__ void __launch_bounds__(THREADS, MINB) split_rows4_kernel(const T* __r
         const bool xvec = (reinterpret_cast<uintptr_t>(xr) & 15) == 0;
         for (int64_t k = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); k < kpad;
              k += 4 * (int64_t)gridDim.x * blockDim.x) {
-            double a[4];
+            T a[4];
             if (xvec && k + 3 < K) {
                 if constexpr (sizeof(T) == 8) {
                     const double2 p0 = __ldg(reinterpret_cast<const double2*>(xr + k));
@@ -208,7 +246,7 @@ __global__ void __launch_bounds__(THREADS, MINB) split_rows4_kernel(const T* __r
                 }
             } else {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) a[u] = k + u < K ? (double)__ldg(xr + k + u) : 0.0;
+                for (int u = 0; u < 4; ++u) a[u] = k + u < K ? __ldg(xr + k + u) : T(0);
             }
             split4<S>(sp, a, er, out + r * kpad + k, plane);
         }
@@ -309,13 +347,13 @@ template <typename T, int S, typename Sp>
 __global__ void split_cols_kernel(const T* __restrict__ X, int64_t K, int64_t N,
                                   int64_t ldx, const int32_t* __restrict__ f,
                                   __nv_bfloat16* __restrict__ out, int64_t kpad, const Sp sp) {
-    __shared__ double t[32][65];
+    __shared__ T t[32][65];
     const int64_t j0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 64;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 8 warps
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int64_t k = k0 + ty + 8 * r, j = j0 + tx;
-        t[tx][ty + 8 * r] = (k < K && j < N) ? (double)__ldg(X + k * ldx + j) : 0.0;
+        t[tx][ty + 8 * r] = (k < K && j < N) ? __ldg(X + k * ldx + j) : T(0);
     }
     __syncthreads();
     const int64_t plane = N * kpad;
@@ -333,22 +371,22 @@ __global__ void split_cols_kernel(const T* __restrict__ X, int64_t K, int64_t N,
 // As split_cols_kernel with four consecutive k per thread: 128 x 32 tiles, the
 // tile row of column jj holding k = 4q + i at position 32 i + q (q < 32, i <
 // 4), so that the tile's fill (one k of 32 columns per warp, a row stride of
-// 129 doubles) and the reads of four consecutive k by each lane (32
-// consecutive doubles per access) are free of bank conflicts; one 8-byte store
+// 129 elements) and the reads of four consecutive k by each lane (32
+// consecutive elements per access) are free of bank conflicts; one 8-byte store
 // per digit plane (256 contiguous bytes per warp).  Needs out 8-byte aligned
 // and kpad a multiple of 4 (the launch checks).
 template <typename T, int S, typename Sp>
 __global__ void __launch_bounds__(256, 4) split_cols4_kernel(
     const T* __restrict__ X, int64_t K, int64_t N, int64_t ldx, const int32_t* __restrict__ f,
     __nv_bfloat16* __restrict__ out, int64_t kpad, const Sp sp) {
-    __shared__ double t[32][129];
+    __shared__ T t[32][129];
     const int64_t j0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 128;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 8 warps
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
         const int kk = ty + 8 * r;
         const int64_t k = k0 + kk, j = j0 + tx;
-        t[tx][(kk & 3) * 32 + (kk >> 2)] = (k < K && j < N) ? (double)__ldg(X + k * ldx + j) : 0.0;
+        t[tx][(kk & 3) * 32 + (kk >> 2)] = (k < K && j < N) ? __ldg(X + k * ldx + j) : T(0);
     }
     __syncthreads();
     const int64_t plane = N * kpad;
@@ -359,7 +397,7 @@ __global__ void __launch_bounds__(256, 4) split_cols4_kernel(
         const int64_t j = j0 + jj;
         if (j >= N) break;
         const int fj = f[j];
-        const double a[4] = {t[jj][tx], t[jj][32 + tx], t[jj][64 + tx], t[jj][96 + tx]};
+        const T a[4] = {t[jj][tx], t[jj][32 + tx], t[jj][64 + tx], t[jj][96 + tx]};
         split4<S>(sp, a, fj, out + j * kpad + k, plane);
     }
 }
