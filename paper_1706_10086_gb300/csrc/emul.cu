@@ -242,6 +242,7 @@ __global__ void recombine_kernel(const int32_t* __restrict__ G, int64_t gplane, 
                                  const int32_t* __restrict__ e, const int32_t* __restrict__ f,
                                  int64_t M, int64_t N, double alpha, double beta,
                                  double* __restrict__ C, int64_t ldc) {
+    pdl_wait();
     const int shift0 = (S + 1) * B;
     for (int64_t i = blockIdx.y; i < M; i += gridDim.y) {
         const int ei = e[i] - shift0;
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(256) recombine4_kernel(
     const int32_t* __restrict__ G, int64_t gplane, int64_t ldg, const int32_t* __restrict__ e,
     const int32_t* __restrict__ f, int64_t M, int64_t N, double alpha, double beta,
     double* __restrict__ C, int64_t ldc) {
+    pdl_wait();
     const int shift0 = (S + 1) * B;
     for (int64_t i = blockIdx.y; i < M; i += gridDim.y) {
         const int ei = e[i] - shift0;
@@ -308,39 +310,52 @@ __global__ void __launch_bounds__(256) recombine4_kernel(
     }
 }
 
+// Launch of a recombination kernel; early: the kernel before it on the stream
+// lets it start while that one drains.
+template <typename... P, typename... A>
+static alp_status launch_after(void (*kernel)(P...), dim3 grid, cudaStream_t st, bool early,
+                               A... args) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(256);
+    lc.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = early ? 1 : 0;
+    return cuda_status(cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...));
+}
+
 template <int B>
 static alp_status launch_recombine_b(int s, dim3 grid, cudaStream_t st, const int32_t* G,
                                      int64_t gplane, int64_t ldg, const int32_t* e,
                                      const int32_t* f, int64_t M, int64_t N, double alpha,
-                                     double beta, double* C, int64_t ldc) {
+                                     double beta, double* C, int64_t ldc, bool early) {
     const bool vec = (reinterpret_cast<uintptr_t>(G) & 15) == 0 && gplane % 4 == 0 && ldg % 4 == 0;
     if (vec) grid.x = (unsigned)((grid.x + 1) / 2);   // four columns per thread instead of two
 #define ALP_RECOMBINE_CASE(x)                                                                     \
     case x:                                                                                      \
-        if (vec)                                                                                 \
-            recombine4_kernel<x, B><<<grid, 256, 0, st>>>(G, gplane, ldg, e, f, M, N, alpha, beta, \
-                                                          C, ldc);                               \
-        else                                                                                     \
-            recombine_kernel<x, B><<<grid, 256, 0, st>>>(G, gplane, ldg, e, f, M, N, alpha, beta,  \
-                                                         C, ldc);                                \
-        break;
+        return launch_after(vec ? recombine4_kernel<x, B> : recombine_kernel<x, B>, grid, st,    \
+                            early, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc);
     switch (s) {
         ALP_RECOMBINE_CASE(1) ALP_RECOMBINE_CASE(2) ALP_RECOMBINE_CASE(3) ALP_RECOMBINE_CASE(4)
         ALP_RECOMBINE_CASE(5) ALP_RECOMBINE_CASE(6) ALP_RECOMBINE_CASE(7) ALP_RECOMBINE_CASE(8)
-        default: return ALP_ERR_INVALID_ARG;
     }
 #undef ALP_RECOMBINE_CASE
-    return cuda_status(cudaGetLastError());
+    return ALP_ERR_INVALID_ARG;
 }
 
 static alp_status launch_recombine(int s, int b, dim3 grid, cudaStream_t st, const int32_t* G,
                                    int64_t gplane, int64_t ldg, const int32_t* e, const int32_t* f,
                                    int64_t M, int64_t N, double alpha, double beta, double* C,
-                                   int64_t ldc) {
+                                   int64_t ldc, bool early = false) {
     if (b == 7)
-        return launch_recombine_b<7>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc);
+        return launch_recombine_b<7>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc,
+                                     early);
     if (b == 8)
-        return launch_recombine_b<8>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc);
+        return launch_recombine_b<8>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc,
+                                     early);
     return ALP_ERR_INVALID_ARG;
 }
 
@@ -423,6 +438,11 @@ static alp_status emul_split_b(int64_t R, int64_t K, const T* X, int64_t ldx, in
         else if (!trans)                                                                         \
             split_rows_kernel<T, x, DigitSplit<B>><<<grid_for(R * (kpad / 2), 256), 256, 0, st>>>( \
                 X, R, K, ldx, exps, out, kpad, {});                                              \
+        else if (vec)                                                                            \
+            split_cols4_kernel<T, x, DigitSplit<B>><<<dim3((unsigned)((R + 31) / 32),             \
+                                                           (unsigned)((kpad + 127) / 128)),      \
+                                                      256, 0, st>>>(X, K, R, ldx, exps, out,     \
+                                                                    kpad, {});                   \
         else                                                                                     \
             split_cols_kernel<T, x, DigitSplit<B>><<<dim3((unsigned)((R + 31) / 32),              \
                                                           (unsigned)(kpad / 64)),                \
@@ -490,6 +510,7 @@ __global__ void __launch_bounds__(256) recombine_f32_kernel(
     const int32_t* __restrict__ G, int64_t gplane, int64_t ldg, const int32_t* __restrict__ e,
     const int32_t* __restrict__ f, int64_t M, int64_t N, float alpha, float beta,
     float* __restrict__ C, int64_t ldc, bool gvec) {
+    pdl_wait();
     const int shift0 = (S + 1) * B;
     for (int64_t i = blockIdx.y; i < M; i += gridDim.y) {
         const int ei = e[i] - shift0;
@@ -539,31 +560,31 @@ template <int B>
 static alp_status launch_recombine_f32_b(int s, dim3 grid, cudaStream_t st, const int32_t* G,
                                          int64_t gplane, int64_t ldg, const int32_t* e,
                                          const int32_t* f, int64_t M, int64_t N, float alpha,
-                                         float beta, float* C, int64_t ldc) {
+                                         float beta, float* C, int64_t ldc, bool early) {
     const bool gvec = (reinterpret_cast<uintptr_t>(G) & 15) == 0 && gplane % 4 == 0 && ldg % 4 == 0;
     grid.x = (unsigned)((grid.x + 1) / 2);   // four columns per thread
-#define ALP_RECOMBINE_F32_CASE(x)                                                                 \
-    case x:                                                                                      \
-        recombine_f32_kernel<x, B><<<grid, 256, 0, st>>>(G, gplane, ldg, e, f, M, N, alpha, beta,  \
-                                                         C, ldc, gvec);                          \
-        break;
+#define ALP_RECOMBINE_F32_CASE(x)                                                               \
+    case x:                                                                                    \
+        return launch_after(recombine_f32_kernel<x, B>, grid, st, early, G, gplane, ldg, e, f, \
+                            M, N, alpha, beta, C, ldc, gvec);
     switch (s) {
         ALP_RECOMBINE_F32_CASE(1) ALP_RECOMBINE_F32_CASE(2) ALP_RECOMBINE_F32_CASE(3)
         ALP_RECOMBINE_F32_CASE(4)
-        default: return ALP_ERR_INVALID_ARG;
     }
 #undef ALP_RECOMBINE_F32_CASE
-    return cuda_status(cudaGetLastError());
+    return ALP_ERR_INVALID_ARG;
 }
 
 static alp_status launch_recombine_f32(int s, int b, dim3 grid, cudaStream_t st, const int32_t* G,
                                        int64_t gplane, int64_t ldg, const int32_t* e,
                                        const int32_t* f, int64_t M, int64_t N, float alpha,
-                                       float beta, float* C, int64_t ldc) {
+                                       float beta, float* C, int64_t ldc, bool early = false) {
     if (b == 7)
-        return launch_recombine_f32_b<7>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc);
+        return launch_recombine_f32_b<7>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C,
+                                         ldc, early);
     if (b == 8)
-        return launch_recombine_f32_b<8>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C, ldc);
+        return launch_recombine_f32_b<8>(s, grid, st, G, gplane, ldg, e, f, M, N, alpha, beta, C,
+                                         ldc, early);
     return ALP_ERR_INVALID_ARG;
 }
 
@@ -698,16 +719,17 @@ alp_status emul_gemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, T alp
                 kcrt, alpha, beta, C, ldc, sched, L0.sched_bytes, s, have ? cfg.stages : 0,
                 have ? emul_arrangement_of(cfg) : 0, -1, prepared);
     }
+    bool paired = false;   // the CTA-pair kernel lets its successor start early
     if ((st = emul_slice_gemm(M, N, K, nslices, da, db, L.kpad, G, L.ldg, s,
                               have ? cfg.stages : 0, have ? emul_arrangement_of(cfg) : 0, b,
-                              sc.trim, sc.crt)) != ALP_OK)
+                              sc.trim, sc.crt, prepared, &paired)) != ALP_OK)
         return st;
     if constexpr (kF32)
         return launch_recombine_f32(nslices, b, recombine_grid(M, N), s, G, M * L.ldg, L.ldg, e,
-                                    f, M, N, alpha, beta, C, ldc);
+                                    f, M, N, alpha, beta, C, ldc, paired);
     else
         return launch_recombine(nslices, b, recombine_grid(M, N), s, G, M * L.ldg, L.ldg, e, f,
-                                M, N, alpha, beta, C, ldc);
+                                M, N, alpha, beta, C, ldc, paired);
 }
 
 }  // namespace alp

@@ -114,11 +114,14 @@ enum EmulArrangement { kEmulSingle = 1, kEmulPair = 3 };
 // the residue slices instead, and G holds s byte planes [l][M][ldg] of
 // (Q_l y_l) mod m_l.  group_m: tile-rows per raster group (0 = default, the
 // tunable of the emulated path).  cluster: the EmulArrangement (0 = default,
-// emul_cluster()).
+// emul_cluster()).  early: the previous launch on the stream lets this one
+// start while it drains (CTA pairs only); *paired: whether CTA pairs ran, which
+// let their successor do the same.
 alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bfloat16* da,
                            const __nv_bfloat16* db, int64_t kpad, int32_t* G, int64_t ldg,
                            cudaStream_t stream, int group_m = 0, int cluster = 0,
-                           int digit_bits = kDigitBits, bool trim = false, bool crt = false);
+                           int digit_bits = kDigitBits, bool trim = false, bool crt = false,
+                           bool early = false, bool* paired = nullptr);
 
 // Grid of the reconstruction kernels: 512 columns per block, rows strided.
 dim3 recombine_grid(int64_t M, int64_t N);

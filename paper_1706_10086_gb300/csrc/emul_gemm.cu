@@ -125,6 +125,10 @@ struct EmulGemmParams {
     // Groups write disjoint planes of G.
     int n_full, pieces;
     uint64_t t_ranges;
+    // CTA pairs: cluster c takes the whole tiles c, c + stride, .. < n_full, then,
+    // as the (c - tail_first)-th of `parts` clusters, its share of the tail
+    // tiles n_full.. (pair_segment)
+    int stride, tail_tiles, tail_first, parts;
     uint64_t timeout_ns;
     int* err;
     // test hook: block 0's producer arms pipeline stage inject_skip_it (its
@@ -221,14 +225,16 @@ __device__ __forceinline__ void hand_back(uint64_t* acce, uint32_t acce_remote, 
         mbar_arrive_cluster(acce_remote + b * 8, kEpiWarps);
 }
 
-// Epilogue warps (2..9): for each finished chunk, drain this warp's 32 TMEM
-// lanes x 128 columns of accumulator b into exact int32 sums, hand the
-// accumulator back (hand_back), and at the end of a group store S^t to
-// G[t-2].
-__device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const uint32_t* jobs,
-                                              int njobs, uint32_t tmem_base, uint64_t* accf,
-                                              uint64_t* acce, uint32_t acce_remote, uint64_t* agg,
-                                              int m0, int n0, int warp, int lane, uint64_t tmo,
+// Epilogue warps (2..9): the jobs j_lo..j_hi-1 (whole groups) of the tile at
+// m0, n0, `job` counting the block's jobs so far.  For each finished chunk,
+// drain this warp's 32 TMEM lanes x 128 columns of accumulator b into exact
+// int32 sums, hand the accumulator back (hand_back), and at the end of a group
+// store S^t to G[t-2].  False when a wait gave up.
+__device__ __forceinline__ bool epilogue_jobs(const EmulGemmParams& prm, const uint32_t* jobs,
+                                              int j_lo, int j_hi, int& job, uint32_t tmem_base,
+                                              uint64_t* accf, uint64_t* acce,
+                                              uint32_t acce_remote, uint64_t* agg, int m0, int n0,
+                                              int warp, int lane, uint64_t tmo,
                                               volatile int* abort_flag, int ew) {
     // ew: this warp's index among the eight epilogue warps (the first one
     // forwards block 1's hand-backs); warp: its index in the block, whose
@@ -242,9 +248,9 @@ __device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const u
 #pragma unroll
     for (int i = 0; i < 128; ++i) acc[i] = zero;
     int t_group = 2;
-    for (int job = 0; job < njobs; ++job) {
+    for (int j = j_lo; j < j_hi; ++j, ++job) {
         const uint32_t b = job & 1;
-        if (!mbar_wait_bounded(&accf[b], (job >> 1) & 1, tmo, abort_flag, prm.err)) break;
+        if (!mbar_wait_bounded(&accf[b], (job >> 1) & 1, tmo, abort_flag, prm.err)) return false;
         tc_fence_after();
         const uint32_t taddr =
             tmem_base + ((uint32_t)(quarter * 32) << 16) + b * kTN + half * 128;
@@ -253,7 +259,7 @@ __device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const u
         tc_fence_before();
         __syncwarp();
         if (lane == 0) hand_back(acce, acce_remote, agg, b, job, ew + 2, tmo, abort_flag, prm.err);
-        const uint32_t jd = jobs[job];
+        const uint32_t jd = jobs[j];
         if (job_last(jd) && prm.modular) {
             // modular scheme: plane l of modulus m_l receives x = (Q y_l) mod
             // m_l = (P y_l) mod m_l, one byte per column (rows padded as below)
@@ -287,6 +293,7 @@ __device__ __forceinline__ void epilogue_role(const EmulGemmParams& prm, const u
                                 acc[4 * i + 3]);
         }
     }
+    return true;
 }
 
 // One block per 128 x 256 tile.
@@ -434,8 +441,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_wait_bounded(done, 0, tmo, nullptr, prm.err, false);
         }
     } else {
-        epilogue_role(prm, jobs, njobs, tmem_base, accf, &acce[0], 0u, nullptr, m0, n0, warp,
-                      lane, tmo, abort_flag, warp - 2);
+        int job = 0;
+        epilogue_jobs(prm, jobs, 0, njobs, job, tmem_base, accf, &acce[0], 0u, nullptr, m0, n0,
+                      warp, lane, tmo, abort_flag, warp - 2);
     }
     tc_fence_before();
     __syncwarp();
@@ -470,7 +478,7 @@ constexpr uint64_t kDrainNs = 2000000ull;
 constexpr uint32_t kPairBTile = kBTile / 2;
 constexpr uint32_t kPairStageBytes = kATile + kPairBTile;
 constexpr int kPairSmemBytes = kPairStages * kPairStageBytes + 1024 /*align*/ + 256 /*barriers*/ +
-                               4 * kMaxJobs;
+                               4 * kMaxJobs + 128 /*first job of each group*/;
 
 constexpr int kFusedSmemBytes = kPairStages * kPairStageBytes + 1024 /*align*/ + 256 /*barriers*/;
 
@@ -488,6 +496,37 @@ __device__ __forceinline__ void pair_tile_origin(const EmulGemmParams& prm, int 
     n0 = (local / gsz) * kTN;
 }
 
+// The i-th segment of cluster `cid`: groups g_lo + 2 .. g_hi + 1 of a pair tile.
+// Its whole tiles come first; then its units, a unit being one group of one
+// tail tile: the units in descending order of their products (tiles innermost,
+// so that clusters side by side in time share digit slices in L2) are dealt out
+// in turns of alternating direction, which keeps the largest share within one
+// product of the mean (64 tiles of 8 slices on 76 pairs: 31 products for a mean
+// of 30.3, where a tile each made it 36).
+__device__ __forceinline__ bool pair_segment(const EmulGemmParams& prm, int cid, int i, int& tile,
+                                             int& g_lo, int& g_hi) {
+    const int whole = cid < prm.n_full ? (prm.n_full - cid + prm.stride - 1) / prm.stride : 0;
+    if (i < whole) {
+        tile = cid + i * prm.stride;
+        g_lo = 0;
+        g_hi = prm.s;
+        return true;
+    }
+    const int c = cid - prm.tail_first, j = i - whole;
+    if (c < 0 || c >= prm.parts) return false;
+    const int u = j * prm.parts + ((j & 1) ? prm.parts - 1 - c : c);
+    if (u >= prm.tail_tiles * prm.s) return false;
+    const int r = u / prm.tail_tiles;   // rank of the group by its products
+    tile = prm.n_full + u - r * prm.tail_tiles;
+    // group g + 2 holds g + 1 products; trimmed, the last one holds two and
+    // comes after group 3
+    const int s = prm.s;
+    if (prm.trim && s > 2) g_lo = r < s - 2 ? s - 2 - r : r == s - 2 ? s - 1 : 0;
+    else g_lo = s - 1 - r;
+    g_hi = g_lo + 1;
+    return true;
+}
+
 __global__ void __launch_bounds__(kPairThreads, 1)
     emul_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA,
                           const __grid_constant__ CUtensorMap tmB, EmulGemmParams prm) {
@@ -503,8 +542,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     uint64_t* agg = done + 1;   // block 1: its epilogue warps' hand-backs, gathered
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(agg + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    int* njobs_slot = const_cast<int*>(reinterpret_cast<volatile int*>(abort_flag + 1));
     uint32_t* jobs = reinterpret_cast<uint32_t*>(smem + kPairStages * kPairStageBytes + 256);
+    int* first = reinterpret_cast<int*>(jobs + kMaxJobs);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
@@ -522,17 +561,14 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
         mbar_init(done, 1);
         *abort_flag = 0;
-        // the tail split counts clusters: both blocks of a pair take the same piece
-        int t_lo = 2, t_hi = prm.s + 1;
-        const int cid = (int)blockIdx.x / 2;
-        if (cid >= prm.n_full) {
-            const int pc = (cid - prm.n_full) % prm.pieces;
-            const uint32_t r = (uint32_t)(prm.t_ranges >> (8 * pc)) & 0xffu;
-            t_lo = (int)(r & 15u) + 2;
-            t_hi = (int)(r >> 4) + 2;
+        // the jobs of a whole tile, group t's from first[t - 2] on
+        int n = 0;
+        for (int t = 2; t <= prm.s + 1; ++t) {
+            first[t - 2] = n;
+            n += build_jobs(prm.s, (int)prm.K, prm.digit_bits, prm.trim != 0, prm.modular != 0, t,
+                            t, jobs + n);
         }
-        *njobs_slot = build_jobs(prm.s, (int)prm.K, prm.digit_bits, prm.trim != 0, prm.modular != 0,
-                                 t_lo, t_hi, jobs);
+        first[prm.s] = n;
         fence_barrier_init();
     }
     if (warp == 1) {
@@ -544,14 +580,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     tc_fence_after();
     pdl_wait();           // the operands are written
     const uint32_t tmem_base = *tmem_slot;
-    const int njobs = *njobs_slot;
-
-    int m0, n0;
-    {
-        const int cid = (int)blockIdx.x / 2;
-        const int pid = cid < prm.n_full ? cid : prm.n_full + (cid - prm.n_full) / prm.pieces;
-        pair_tile_origin(prm, pid, rank, m0, n0);
-    }
+    const int cid = (int)blockIdx.x / 2;
     const uint64_t tmo = prm.timeout_ns;
     const uint32_t full0 = cluster_addr(full, 0);   // block 0's full barriers
     // each warpgroup changes its registers once, before its warps part: the
@@ -559,9 +588,14 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     const int wg = warp >> 2;
     if (wg == 1 || wg == 2) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPairEpiRegs));
-        epilogue_role(prm, jobs, njobs, tmem_base, accf, &acce[0],
-                      leader ? 0u : cluster_addr(acce, 0), agg, m0, n0, warp, lane, tmo,
-                      abort_flag, warp - 4);
+        const uint32_t acce_remote = leader ? 0u : cluster_addr(acce, 0);
+        int job = 0, tile, g_lo, g_hi, m0, n0;
+        for (int i = 0; pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
+            pair_tile_origin(prm, tile, rank, m0, n0);
+            if (!epilogue_jobs(prm, jobs, first[g_lo], first[g_hi], job, tmem_base, accf, &acce[0],
+                               acce_remote, agg, m0, n0, warp, lane, tmo, abort_flag, warp - 4))
+                break;
+        }
     } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPairLowRegs));
     if (warp == 0) {
@@ -571,7 +605,11 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             tma_prefetch_desc(&tmB);
             uint32_t it = 0;
             bool ok = true;
-            for (int j = 0; j < njobs && ok; ++j) {
+            int tile, g_lo, g_hi, m0, n0;
+            for (int i = 0; ok && pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
+            pair_tile_origin(prm, tile, rank, m0, n0);
+            const int j_end = first[g_hi];
+            for (int j = first[g_lo]; j < j_end && ok; ++j) {
                 const uint32_t jd = jobs[j];
                 for (int kb = job_kb(jd); kb < job_ke(jd); ++kb, ++it) {
                     const uint32_t st = it % kPairStages, round = it / kPairStages;
@@ -588,6 +626,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                     tma_load_3d_pair(a + kATile, &tmB, full0 + st * 8, kb * kTK,
                                      n0 + (int)rank * (kTN / 2), job_q(jd) - 1);
                 }
+            }
             }
             // The MMAs of every issued stage must have consumed it (so this
             // block's copies have landed, on block 0's barrier) and its
@@ -610,9 +649,12 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             // ---------------- MMA issuer (block 0) ----------------
             const uint32_t idesc = idesc_bf16_f32(2 * kTM, kTN);
             uint32_t it = 0;
+            int job = 0, tile, g_lo, g_hi;
             bool ok = true;
-            for (int job = 0; job < njobs && ok; ++job) {
-                const uint32_t jd = jobs[job];
+            for (int i = 0; ok && pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
+            const int j_end = first[g_hi];
+            for (int j = first[g_lo]; j < j_end && ok; ++j, ++job) {
+                const uint32_t jd = jobs[j];
                 const uint32_t b = job & 1;
                 if (job >= 2 &&
                     !mbar_wait_bounded(&acce[b], ((job >> 1) - 1) & 1, tmo, abort_flag, prm.err)) {
@@ -642,6 +684,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                 if (!ok) break;
                 umma_commit_pair(&accf[b], 3);
             }
+            }
             // all MMAs must have completed before TMEM and shared memory go away,
             // and both blocks' hand-backs of the last two chunks must have
             // arrived.  After an abort the epilogue warps leave without handing
@@ -649,8 +692,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             // arrival, which block 0 waits for before it exits.
             umma_commit_pair(done, 1);
             mbar_wait_bounded(done, 0, tmo, nullptr, prm.err, false);
-            for (int job = njobs > 2 ? njobs - 2 : 0; job < njobs && ok; ++job)
-                mbar_wait_bounded(&acce[job & 1], (job >> 1) & 1, tmo, nullptr, prm.err, false);
+            for (int j = job > 2 ? job - 2 : 0; j < job && ok; ++j)
+                mbar_wait_bounded(&acce[j & 1], (j >> 1) & 1, tmo, nullptr, prm.err, false);
         }
     }
     }   // warps 2, 3 and 12-15 have no role
@@ -1212,10 +1255,37 @@ TailSplit tail_split(int tiles, int s, int sms, bool trim, bool crt) {
     return ts;
 }
 
+// CTA-pair clusters that are resident at once (the persistent grids; the
+// fused kernel's footprint, which the product kernel's equals); half the SMs if the query fails.
+static int fused_active_clusters() {
+    static int c = 0;
+    if (c == 0) {
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3((unsigned)(2 * device_sm_count()));
+        lc.blockDim = dim3(kFusedThreads);
+        lc.dynamicSmemBytes = kFusedSmemBytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+        int nc = 0;
+        if (cudaOccupancyMaxActiveClusters(&nc, emul_crt_fused_pair_kernel, &lc) != cudaSuccess ||
+            nc < 1) {
+            (void)cudaGetLastError();
+            nc = device_sm_count() / 2;
+        }
+        c = nc > 0 ? nc : 1;
+    }
+    return c;
+}
+
 alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bfloat16* da,
                            const __nv_bfloat16* db, int64_t kpad, int32_t* G, int64_t ldg,
                            cudaStream_t stream, int group_m, int cluster, int digit_bits,
-                           bool trim, bool crt) {
+                           bool trim, bool crt, bool early, bool* paired) {
     if (crt) {
         if (s < kCrtMinModuli || s > kCrtMaxModuli || K > kCrtMaxK) return ALP_ERR_UNSUPPORTED;
     } else if (!emul_digit_bits_ok(digit_bits) || s > emul_max_slices(digit_bits) ||
@@ -1236,6 +1306,7 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     }
     const int arr = (cluster == kEmulSingle || cluster == kEmulPair) ? cluster : emul_cluster();
     const int cl = arr == kEmulSingle ? 1 : 2;   // blocks per cluster
+    if (paired) *paired = cl == 2;
     CUtensorMap ta, tb;
     alp_status st = make_tmap_3d_bf16(&ta, da, (uint64_t)kpad, (uint64_t)M, (uint64_t)s, kTK, kTM);
     if (st != ALP_OK) return st;
@@ -1285,16 +1356,28 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     }
     const int smem_bytes = kPairSmemBytes;
     const int64_t pair_tiles = ((tiles_m + 1) / 2) * tiles_n;
-    int64_t clusters = pair_tiles;
-    if (emul_tail_split_on()) {   // in units of pairs, half the SMs each
-        const TailSplit ts = tail_split((int)pair_tiles, s, device_sm_count() / 2, trim, crt);
-        p.n_full = ts.n_full;
-        p.pieces = ts.pieces;
-        p.t_ranges = 0;
-        for (int i = 0; i < ts.pieces; ++i)
-            p.t_ranges |= (uint64_t)((ts.t_lo[i] - 2) | (ts.t_hi[i] - 2) << 4) << (8 * i);
-        if (ts.n_full < pair_tiles) clusters = ts.n_full + (pair_tiles - ts.n_full) * ts.pieces;
-    }
+    if (pair_tiles * kCrtMaxModuli > 0x7fffffff) return ALP_ERR_UNSUPPORTED;
+    // P resident pairs; whole tiles fill whole waves, the units of the rest are
+    // shared by P clusters.  Up to kStaticWaves waves the clusters are resident
+    // and walk their tiles, so that the next tile's copies and products overlap
+    // the last drains and stores of a tile; beyond, each whole tile is a cluster
+    // of its own, which the hardware hands out as pairs become free (a fixed
+    // assignment lets fast and slow pairs drift apart, by 3 % over 13 waves).
+    constexpr int64_t kStaticWaves = 8;
+    const int64_t P = fused_active_clusters();
+    const int64_t waves = pair_tiles / P;
+    // (a rest of more than nine tenths of a wave stays whole: sharing it would
+    // gain less than its clusters lose by reading different slices, 526 us
+    // against 511 for 72 tiles of 8 slices)
+    const bool share = emul_tail_split_on() && 10 * (pair_tiles % P) <= 9 * P;
+    p.n_full = (int)(share ? waves * P : pair_tiles);
+    p.tail_tiles = (int)pair_tiles - p.n_full;
+    p.parts = (int)std::min<int64_t>(P, (int64_t)p.tail_tiles * s);
+    const bool resident = waves < kStaticWaves;
+    p.stride = (int)(resident ? P : pair_tiles);
+    p.tail_first = resident ? 0 : p.n_full;
+    const int64_t clusters = resident ? std::max<int64_t>(std::min<int64_t>(P, p.n_full), p.parts)
+                                      : (int64_t)p.n_full + p.parts;
     cudaError_t e = cudaFuncSetAttribute(emul_gemm_pair_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e != cudaSuccess) return cuda_status(e);
@@ -1305,42 +1388,17 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     lc.blockDim = dim3(kPairThreads);
     lc.dynamicSmemBytes = smem_bytes;
     lc.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
-    lc.numAttrs = 1;
+    lc.numAttrs = early ? 2 : 1;
     e = cudaLaunchKernelEx(&lc, emul_gemm_pair_kernel, ta, tb, p);
     return cuda_status(e);
-}
-
-// Clusters of the fused kernel that are resident at once (its persistent
-// grid); half the SMs if the query fails.
-static int fused_active_clusters() {
-    static int c = 0;
-    if (c == 0) {
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((unsigned)(2 * device_sm_count()));
-        lc.blockDim = dim3(kFusedThreads);
-        lc.dynamicSmemBytes = kFusedSmemBytes;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        lc.attrs = attr;
-        lc.numAttrs = 1;
-        int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, emul_crt_fused_pair_kernel, &lc) != cudaSuccess ||
-            nc < 1) {
-            (void)cudaGetLastError();
-            nc = device_sm_count() / 2;
-        }
-        c = nc > 0 ? nc : 1;
-    }
-    return c;
 }
 
 size_t emul_crt_sched_bytes(int64_t M, int64_t N) {
