@@ -2,6 +2,7 @@
 // count, tensor-map encoder) and config selection for alp_gemm_f64.
 #include <cudaTypedefs.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -34,12 +35,13 @@ bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* ou
 // ----------------------------------------------------------------------------
 namespace {
 constexpr int kMaxDevices = 64;
+// g_mu guards the set-up of what follows; once set, it is read without it.
 std::mutex g_mu;
-int* g_err_word[kMaxDevices];
-int g_sm_count[kMaxDevices];
-uint64_t g_timeout_ns = 0;
-int g_inject_skip_kt = -1;
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+std::atomic<int*> g_err_word[kMaxDevices];
+std::atomic<int> g_sm_count[kMaxDevices];
+std::atomic<uint64_t> g_timeout_ns{0};
+std::atomic<int> g_inject_skip_kt{-1};
+std::atomic<PFN_cuTensorMapEncodeTiled_v12000> g_encode{nullptr};
 
 int current_device() {
     int d = 0;
@@ -54,31 +56,51 @@ void init_device_locked(int d) {
     if (cudaMalloc(&w, sizeof(int)) == cudaSuccess) {
         cudaMemset(w, 0, sizeof(int));
         cudaDeviceSynchronize();
-        g_err_word[d] = w;
     }
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
     g_sm_count[d] = sms > 0 ? sms : 1;
+    g_err_word[d] = w;   // last: a set word means that all is set
+}
+void init_device(int d) {
+    if (d < 0 || d >= kMaxDevices || g_err_word[d].load()) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    init_device_locked(d);
+}
+// The tensor-map encoder, looked up once (null if the driver has none).
+PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
+    PFN_cuTensorMapEncodeTiled_v12000 f = g_encode.load();
+    if (f) return f;
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (!g_encode.load()) {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
+                                             cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess || !fn)
+            return nullptr;
+        g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    }
+    return g_encode.load();
 }
 }  // namespace
 
 int* device_error_word() {
     const int d = current_device();
-    std::lock_guard<std::mutex> lk(g_mu);
-    init_device_locked(d);
-    return (d >= 0 && d < kMaxDevices) ? g_err_word[d] : nullptr;
+    init_device(d);
+    return (d >= 0 && d < kMaxDevices) ? g_err_word[d].load() : nullptr;
 }
 
 int device_sm_count() {
     const int d = current_device();
-    std::lock_guard<std::mutex> lk(g_mu);
-    init_device_locked(d);
-    return (d >= 0 && d < kMaxDevices) ? g_sm_count[d] : 1;
+    init_device(d);
+    return (d >= 0 && d < kMaxDevices) ? g_sm_count[d].load() : 1;
 }
 
 uint64_t wait_timeout_ns() {
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (g_timeout_ns == 0) {
+    if (g_timeout_ns.load() == 0) {
+        std::lock_guard<std::mutex> lk(g_mu);
+        if (g_timeout_ns.load() != 0) return g_timeout_ns;
         double ms = 4000.0;   // default: 4 s per wait; no legitimate wait comes close
         if (const char* s = std::getenv("ALP_WAIT_TIMEOUT_MS")) {
             double v = std::atof(s);
@@ -94,24 +116,14 @@ alp_status cuda_status(cudaError_t e) { return e == cudaSuccess ? ALP_OK : ALP_E
 alp_status make_tmap_2d(CUtensorMap* map, CUtensorMapDataType dtype, int elem_bytes,
                         const void* base, uint64_t inner, uint64_t outer, uint64_t row_bytes,
                         uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz) {
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        if (!g_encode) {
-            void* fn = nullptr;
-            cudaDriverEntryPointQueryResult q;
-            if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                 cudaEnableDefault, &q) != cudaSuccess ||
-                q != cudaDriverEntryPointSuccess || !fn)
-                return ALP_ERR_CUDA;
-            g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-        }
-    }
+    const auto encode = tmap_encoder();
+    if (!encode) return ALP_ERR_CUDA;
     (void)elem_bytes;
     cuuint64_t dims[2] = {inner, outer};
     cuuint64_t strides[1] = {row_bytes};
     cuuint32_t box[2] = {box_inner, box_outer};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(map, dtype, 2, const_cast<void*>(base), dims, strides, box, estr,
+    CUresult r = encode(map, dtype, 2, const_cast<void*>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? ALP_OK : ALP_ERR_UNSUPPORTED;
@@ -121,23 +133,13 @@ alp_status make_tmap_2d(CUtensorMap* map, CUtensorMapDataType dtype, int elem_by
 // plane), 128-byte swizzle, box {box0, box1, 1}.
 alp_status make_tmap_3d_bf16(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1,
                              uint64_t d2, uint32_t box0, uint32_t box1) {
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        if (!g_encode) {
-            void* fn = nullptr;
-            cudaDriverEntryPointQueryResult q;
-            if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                 cudaEnableDefault, &q) != cudaSuccess ||
-                q != cudaDriverEntryPointSuccess || !fn)
-                return ALP_ERR_CUDA;
-            g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-        }
-    }
+    const auto encode = tmap_encoder();
+    if (!encode) return ALP_ERR_CUDA;
     cuuint64_t dims[3] = {d0, d1, d2};
     cuuint64_t strides[2] = {d0 * 2, d0 * d1 * 2};
     cuuint32_t box[3] = {box0, box1, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
+    CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
                           strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -160,10 +162,7 @@ bool default_config(alp_path path, alp_config* out) {
     return default_native_config(out);
 }
 
-int inject_skip_kt() {
-    std::lock_guard<std::mutex> lk(g_mu);
-    return g_inject_skip_kt;
-}
+int inject_skip_kt() { return g_inject_skip_kt.load(); }
 
 // Shared validation of one GEMM's arguments.
 alp_status validate_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* A,
@@ -367,13 +366,11 @@ int alp_config_threads(const alp_config* cfg) {
 
 alp_status alp_set_wait_timeout_ms(double ms) {
     if (!(ms > 0)) return ALP_ERR_INVALID_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
     g_timeout_ns = (uint64_t)(ms * 1e6);
     return ALP_OK;
 }
 
 alp_status alp_debug_inject_skip(int kt) {
-    std::lock_guard<std::mutex> lk(g_mu);
     g_inject_skip_kt = kt;
     return ALP_OK;
 }

@@ -20,6 +20,7 @@
 // (forward 130 -> 10, loss and deltas 676 -> 17, gradients 432 -> 18, Adam 4).
 // Parameters are one float array: W1[64][7], b1[64], W2[64][64], b2[64],
 // W3[C][64], b3[C].
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -474,8 +475,11 @@ struct Model {
 };
 std::mutex g_mmu;
 Model g_model;
+std::atomic<bool> g_loaded{false};   // g_model.loaded, read without the lock
 
 }  // namespace
+
+bool model_loaded() { return g_loaded.load(); }
 
 // Arg-min of the model's predicted log-time over the valid configs of `path`.
 bool model_predict(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
@@ -627,6 +631,7 @@ alp_status alp_tune_load_model(const float* host_params, int C, const float* hos
     std::memcpy(g_model.stdv, host_std, sizeof g_model.stdv);
     g_model.C = C;
     g_model.loaded = true;
+    g_loaded.store(true);
     g_model.dev = -1;    // re-upload on next use
     return ALP_OK;
 }
@@ -634,6 +639,7 @@ alp_status alp_tune_load_model(const float* host_params, int C, const float* hos
 alp_status alp_tune_unload_model(void) {
     std::lock_guard<std::mutex> lk(g_mmu);
     g_model.loaded = false;
+    g_loaded.store(false);
     return ALP_OK;
 }
 

@@ -15,6 +15,7 @@
 // pipe) and by K / K'.  Shapes that fit one wave with K <= kProxyK are timed
 // exactly.  The emulated path runs its full grid with K capped.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -38,6 +39,7 @@ alp_status native_launch(const alp_config& cfg, bool use_tma, int64_t M, int64_t
                          int inject_skip_kt, int64_t grid_limit);
 int native_occupancy(const alp_config& cfg, bool use_tma);
 bool default_config(alp_path path, alp_config* out);
+bool model_loaded();
 bool model_predict(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                    double* pred_tflops);
 
@@ -58,6 +60,7 @@ int64_t proxy_k_emul() {
 constexpr int kTimedRuns = 10;          // the paper keeps the best of ten runs
 
 std::mutex g_tmu;
+std::atomic<bool> g_cached{false};   // g_cache may have entries
 std::map<std::tuple<int64_t, int64_t, int64_t, int>, alp_config> g_cache;
 
 const int kBM[3] = {64, 128, 256};
@@ -237,6 +240,7 @@ std::vector<alp_config> configs_of(alp_path path) {
 void cache_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_config& c) {
     std::lock_guard<std::mutex> lk(g_tmu);
     g_cache[std::make_tuple(M, N, K, (int)path)] = c;
+    g_cached.store(true);
 }
 
 // Config of a GEMM issued with cfg == NULL: the tuned cache, else the cost
@@ -245,7 +249,7 @@ void cache_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_conf
 // neither has one.
 bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                    cudaStream_t stream) {
-    {
+    if (g_cached.load()) {
         std::lock_guard<std::mutex> lk(g_tmu);
         auto it = g_cache.find(std::make_tuple(M, N, K, (int)path));
         if (it != g_cache.end()) {
@@ -254,7 +258,8 @@ bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* ou
         }
     }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+    if (model_loaded() && cudaStreamIsCapturing(stream, &cs) == cudaSuccess &&
+        cs == cudaStreamCaptureStatusNone &&
         model_predict(M, N, K, path, out, nullptr)) {
         cache_config(M, N, K, path, *out);
         return true;
@@ -359,6 +364,7 @@ alp_status alp_tune_set_cached(int64_t M, int64_t N, int64_t K, alp_path path,
 alp_status alp_tune_clear_cache(void) {
     std::lock_guard<std::mutex> lk(g_tmu);
     g_cache.clear();
+    g_cached.store(false);
     return ALP_OK;
 }
 
