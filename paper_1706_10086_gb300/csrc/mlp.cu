@@ -16,8 +16,8 @@
 //   adam       elementwise Adam with bias correction (Kingma and Ba 2015).
 // All are small (0.23 GFLOP and 6 MB for 4000 samples and 78 outputs), so they
 // are bound by latency: what counts is the blocks in flight and the length of
-// each serial chain.  One training step of that size on GB300: 1061 -> 48.7 us
-// (forward 130 -> 10, loss and deltas 676 -> 17, gradients 432 -> 18, Adam 4).
+// each serial chain.  One training step of that size on GB300: 1061 -> 44.7 us
+// (forward 130 -> 10, loss and deltas 676 -> 13, gradients 432 -> 18, Adam 4).
 // Parameters are one float array: W1[64][7], b1[64], W2[64][64], b2[64],
 // W3[C][64], b3[C].
 #include <atomic>
@@ -173,26 +173,36 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// The block's sums of a and b, in warp 0's lanes (an FP64 addition holds a
-// sub-partition for 73 clocks, so no other warp repeats them); red: 2 *
-// kMlpThreads / 32 doubles.  Every thread passes its barrier.
+// The block's sums of a and b (b held by lane 0 of each warp only), in thread
+// 0; red: 2 * kMlpThreads / 32 doubles.  An FP64 addition holds a sub-partition
+// for 73 clocks, so only warp 0 adds the warps' sums, both at once in two
+// lanes.  Every thread passes its barrier.
 __device__ __forceinline__ void block_sums(double& a, double& b, double* red) {
     constexpr int kW = kMlpThreads / 32;
     a = warp_sum(a);
-    b = warp_sum(b);
     if ((threadIdx.x & 31) == 0) {
         red[threadIdx.x >> 5] = a;
         red[kW + (threadIdx.x >> 5)] = b;
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
-    a = red[0];
-    b = red[kW];
+    const double* r = red + (threadIdx.x & 1) * kW;
+    a = r[0];
 #pragma unroll
-    for (int i = 1; i < kW; ++i) {
-        a += red[i];
-        b += red[kW + i];
-    }
+    for (int i = 1; i < kW; ++i) a += r[i];
+    b = __shfl_sync(0xffffffffu, a, 1);
+}
+
+// The exact double of a float that is zero or normal, by its bits: a
+// conversion holds the FP64 unit for as long as an addition does.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), e = (u << 1) ? 896u << 20 : 0u;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + e)),
+                            (int)(u << 29));
+}
+__device__ __forceinline__ bool zero_or_normal(float x) {
+    const uint32_t e = (__float_as_uint(x) >> 23) & 255u;
+    return e - 1u < 254u || (__float_as_uint(x) << 1) == 0u;
 }
 
 // A double as two floats' bits in an array aligned to 4 bytes only.
@@ -208,8 +218,8 @@ __device__ __forceinline__ double load_double(const float* p) {
 // dy = 2 m (y - t), dz2 = (W3^T dy) * [z2 > 0], dz1 = (W2^T dz2) * [z1 > 0]
 // (dz[n] = dz1, dz2), 16 samples per block as in the forward, and the block's
 // sums of m (y - t)^2 and m in double: into part[4 * block] (the bits of
-// both doubles), or, from the only block of a launch, finished into lossc.  The loss and its count were a kernel of
-// one block, 657 us for 4000 x 78 elements.
+// both doubles), or, from the only block of a launch, finished into lossc.  The
+// loss and its count were a kernel of one block, 657 us for 4000 x 78 elements.
 __global__ void __launch_bounds__(kMlpThreads) delta_kernel(
     const float* __restrict__ P, int C, int64_t B, const float* __restrict__ cache,
     const float* __restrict__ Y, const float* __restrict__ T, const float* __restrict__ Mk,
@@ -239,7 +249,13 @@ __global__ void __launch_bounds__(kMlpThreads) delta_kernel(
         z2[u] = n < B ? __ldg(cache + n * 2 * kH + kH + j) : 0.f;
     }
     stage_weights<kH>(P + off_w2(), 0, kH, w2);
+    // A warp whose mask is zeros and ones and whose values are zero or normal
+    // (the tuner's own data) takes two FP64 operations per element, the others
+    // seven: the sums are the same, as products with 1 and counts are exact.
+    // (At 73 clocks each the seven took the step 48.9 us, the two 44.7.)
     double sum = 0.0, cnt = 0.0;
+    int ones = 0;           // elements counted by the first kind
+    bool others = false;    // cnt is in use (uniform in a warp)
     float v[4] = {0.f, 0.f, 0.f, 0.f};
     auto dot = [&](const float* w, int rows) {   // v += w^T d over the rows of w
 #pragma unroll 16
@@ -255,12 +271,28 @@ __global__ void __launch_bounds__(kMlpThreads) delta_kernel(
     for (int c0 = 0; c0 < C; c0 += kH) {
         if (c0) __syncthreads();
         stage_weights<kH>(P + off_w3(), c0, C, w3);
-        if (c0 + j < C) {   // whole warps past the last column skip the FP64 sums
+        if (c0 + (j & 32) < C) {   // whole warps past the last column skip the FP64 sums
+            bool plain = true;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const double e = (double)y[u] - (double)t[u];
-                sum += m[u] * e * e;
-                cnt += m[u];
+            for (int u = 0; u < 4; ++u)
+                plain = plain && (m[u] == 0.f || m[u] == 1.f) && zero_or_normal(y[u]) &&
+                        zero_or_normal(t[u]);
+            if (__all_sync(0xffffffffu, plain)) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool on = m[u] != 0.f;
+                    const double e = widen(on ? y[u] : 0.f) - widen(on ? t[u] : 0.f);
+                    sum = fma(e, e, sum);
+                    ones += on;
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const double e = (double)y[u] - (double)t[u];
+                    sum += m[u] * e * e;
+                    cnt += m[u];
+                }
+                others = true;
             }
         }
 #pragma unroll
@@ -278,6 +310,9 @@ __global__ void __launch_bounds__(kMlpThreads) delta_kernel(
         d[j][4 * g + u] = d2;
         v[u] = 0.f;
     }
+    ones = __reduce_add_sync(0xffffffffu, ones);
+    if (others) cnt = warp_sum(cnt);
+    if ((threadIdx.x & 31) == 0) cnt += ones;
     block_sums(sum, cnt, red);   // its barrier also makes d visible
     dot(w2, kH);
 #pragma unroll
