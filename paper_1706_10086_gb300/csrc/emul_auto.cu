@@ -38,11 +38,40 @@ __device__ __forceinline__ void atomic_max_pos(float* p, float v) {
     atomicMax(reinterpret_cast<int*>(p), __float_as_int(v));
 }
 
-__device__ __forceinline__ void record_stats(float s1, float s2, float* out) {
-    if (s1 > 0.0f && s2 > 0.0f) {
-        atomic_max_pos(out + 0, 1.0f / (s1 * s1));
-        atomic_max_pos(out + 1, s2 / (s1 * s1));
-        atomic_max_pos(out + 2, 1.0f / s2);
+// The three statistics of a line, or the largest of several lines'.
+struct LineStats {
+    float v[3] = {0.0f, 0.0f, 0.0f};
+    __device__ __forceinline__ void add(float s1, float s2) {
+        if (s1 > 0.0f && s2 > 0.0f) {
+            v[0] = fmaxf(v[0], 1.0f / (s1 * s1));
+            v[1] = fmaxf(v[1], s2 / (s1 * s1));
+            v[2] = fmaxf(v[2], 1.0f / s2);
+        }
+    }
+};
+
+__device__ __forceinline__ void record_stats(const LineStats& s, float* out) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (s.v[i] > 0.0f) atomic_max_pos(out + i, s.v[i]);
+}
+
+// The largest of the block's threads' statistics into out, one atomic for
+// each: those of every line, all to the same words, queue up in L2 (256^3 with
+// the automatic count: 41.7 -> 41.0 us).  All threads call it.
+__device__ __forceinline__ void record_block_stats(const LineStats& s, float* out,
+                                                   float (*red)[3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int m = __reduce_max_sync(0xffffffffu, __float_as_int(s.v[i]));
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = __int_as_float(m);
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        float m = red[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < kPrepWarps; ++w) m = fmaxf(m, red[w][threadIdx.x]);
+        if (m > 0.0f) atomic_max_pos(out + threadIdx.x, m);
     }
 }
 
@@ -83,7 +112,10 @@ __global__ void crt_stats_cols_kernel(const double* __restrict__ X, int64_t K, i
 __global__ void crt_stats_finish_kernel(int64_t N, const float* __restrict__ s1,
                                         const float* __restrict__ s2, float* out) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < N) record_stats(s1[j], s2[j], out);
+    if (j >= N) return;
+    LineStats s;
+    s.add(s1[j], s2[j]);
+    record_stats(s, out);
 }
 
 // Statistics of the R columns of a row-major L x R matrix X, scale exponents
@@ -131,8 +163,9 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 template <int TEAM>
 __device__ __forceinline__ void stat_rows(const PrepParams<double>& p,
-                                          const PrepOperand<double>& o, int block, float* out,
-                                          uint64_t (*red)[kPrepWarps], float2 (*sums)[kPrepWarps]) {
+                                          const PrepOperand<double>& o, int block,
+                                          LineStats& best, uint64_t (*red)[kPrepWarps],
+                                          float2 (*sums)[kPrepWarps]) {
     constexpr int kTeams = kPrepThreads / TEAM;
     const int t = threadIdx.x % TEAM;
     int par = 0;
@@ -160,14 +193,14 @@ __device__ __forceinline__ void stat_rows(const PrepParams<double>& p,
                 s2 += sums[par][w].y;
             }
         }
-        if (t == 0) record_stats(s1, s2, out);
+        if (t == 0) best.add(s1, s2);
     }
 }
 
 __device__ __forceinline__ void stat_cols(const PrepParams<double>& p,
                                           const PrepOperand<double>& o, int block, double* tile,
-                                          float* out, uint64_t* red, uint64_t* cmax, int* sexp,
-                                          float2* csum) {
+                                          LineStats& best, uint64_t* red, uint64_t* cmax,
+                                          int* sexp, float2* csum) {
     constexpr int W = kPrepStrip<double>;
     const uint32_t rank = cluster_ctarank(), size = cluster_nctarank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -209,7 +242,7 @@ __device__ __forceinline__ void stat_cols(const PrepParams<double>& p,
             s1 += a;
             s2 += b;
         }
-        record_stats(s1, s2, out);
+        best.add(s1, s2);
     }
     cluster_sync_all();   // csum and cmax read by the whole cluster
 }
@@ -224,14 +257,16 @@ __global__ void __launch_bounds__(kPrepThreads, 3)
     const bool second = (int)blockIdx.x >= p.op[0].blocks;
     const PrepOperand<double>& o = p.op[second ? 1 : 0];
     const int block = (int)blockIdx.x - (second ? p.op[0].blocks : 0);
-    float* st = out + (second ? 3 : 0);
+    __shared__ float stats[kPrepWarps][3];
+    LineStats best;
     if (o.cols)
-        stat_cols(p, o, block, reinterpret_cast<double*>(smem_raw), st, red, cmax, sexp, sums[0]);
+        stat_cols(p, o, block, reinterpret_cast<double*>(smem_raw), best, red, cmax, sexp, sums[0]);
     else if (p.K <= kPrepWarpRowK)
-        stat_rows<32>(p, o, block, st, reinterpret_cast<uint64_t(*)[kPrepWarps]>(red), sums);
+        stat_rows<32>(p, o, block, best, reinterpret_cast<uint64_t(*)[kPrepWarps]>(red), sums);
     else
-        stat_rows<kPrepThreads>(p, o, block, st, reinterpret_cast<uint64_t(*)[kPrepWarps]>(red),
-                                sums);
+        stat_rows<kPrepThreads>(p, o, block, best,
+                                reinterpret_cast<uint64_t(*)[kPrepWarps]>(red), sums);
+    record_block_stats(best, out + (second ? 3 : 0), stats);
 }
 
 }  // namespace
