@@ -16,8 +16,8 @@
 //   adam       elementwise Adam with bias correction (Kingma and Ba 2015).
 // All are small (0.23 GFLOP and 6 MB for 4000 samples and 78 outputs), so they
 // are bound by latency: what counts is the blocks in flight and the length of
-// each serial chain.  One training step of that size on GB300: 1061 -> 44.7 us
-// (forward 130 -> 10, loss and deltas 676 -> 13, gradients 432 -> 18, Adam 4).
+// each serial chain.  One training step of that size on GB300: 1061 -> 43.1 us
+// (forward 130 -> 10, loss and deltas 676 -> 12, gradients 432 -> 15, Adam 4).
 // Parameters are one float array: W1[64][7], b1[64], W2[64][64], b2[64],
 // W3[C][64], b3[C].
 #include <atomic>
@@ -89,11 +89,13 @@ constexpr int kWPad = kH + 1;        // row stride of a staged 64 x 64 weight ti
 template <int LD>
 __device__ __forceinline__ void stage_weights(const float* __restrict__ W, int row0, int rows,
                                               float* w) {
+    constexpr int kStep = kMlpThreads / kH;   // rows per pass
+    const int r = threadIdx.x / kH, left = rows - row0 - r;
+    const float* p = W + (int64_t)row0 * kH + threadIdx.x;
+    float* o = w + r * LD + threadIdx.x % kH;
 #pragma unroll
-    for (int i = 0; i < kH * kH / kMlpThreads; ++i) {
-        const int e = threadIdx.x + i * kMlpThreads, r = e / kH, c = e % kH;
-        w[r * LD + c] = row0 + r < rows ? __ldg(W + (int64_t)(row0 + r) * kH + c) : 0.f;
-    }
+    for (int i = 0; i < kH / kStep; ++i)
+        o[i * kStep * LD] = i * kStep < left ? __ldg(p + i * kMlpThreads) : 0.f;
 }
 
 // z[0..3] += sum_k w[j][k] h[k][4 g .. 4 g + 3]
@@ -231,11 +233,13 @@ __global__ void __launch_bounds__(kMlpThreads) delta_kernel(
     const int j = threadIdx.x & 63, g = threadIdx.x >> 6;
     // every load of a chunk in flight before the first use
     float m[4], y[4], t[4], z1[4], z2[4];
+    const int64_t at = (n0 + 4 * g) * C + j;
+    const int rows = (int)(B - n0 - 4 * g < 4 ? B - n0 - 4 * g : 4);
     auto load = [&](int c0) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int64_t n = n0 + 4 * g + u, i = n * C + c0 + j;
-            const bool in = c0 + j < C && n < B;
+            const int64_t i = at + c0 + (int64_t)u * C;
+            const bool in = c0 + j < C && u < rows;
             m[u] = in ? __ldg(Mk + i) : 0.f;
             y[u] = in ? __ldg(Y + i) : 0.f;
             t[u] = in ? __ldg(T + i) : 0.f;
@@ -368,28 +372,39 @@ __global__ void __launch_bounds__(kMlpThreads) grad_kernel(
     const int64_t dld = w3 ? C : 2 * kH, hld = seg == 1 ? kF : 2 * kH;
     const int dcols = w3 ? min(C - r0, kGradRows) : kGradRows, hcols = seg == 1 ? kF : kH;
     constexpr int kD = kGradChunk * kGradRows / kMlpThreads, kHn = kGradChunk * kH / kMlpThreads;
+    constexpr int kDStep = kMlpThreads / kGradRows, kHStep = kMlpThreads / kH;   // samples
+    const int dn = tid / kGradRows, dr = tid % kGradRows, hn = tid / kH, hc = tid % kH;
+    const bool din = dr < dcols, hin = hc < hcols;
+    // this thread's first elements of the next chunk to load, which advance by
+    // chunks (with indices formed anew for each load a training step took 44.7
+    // us, 43.1 this way)
+    const float* dp = dsrc + (lo + dn) * dld + dr;
+    const float* tp = T + (lo + dn) * C + r0 + dr;
+    const float* mp = Mk + (lo + dn) * C + r0 + dr;
+    const float* hp = hsrc + (lo + hn) * hld + hc;
+    int left = (int)(hi - lo);   // samples not loaded yet
     float rd[kD], rt[kD], rm[kD], rh[kHn];
-    auto load = [&](int64_t n0) {
+    auto load = [&]() {
 #pragma unroll
         for (int i = 0; i < kD; ++i) {
-            const int e = tid + i * kMlpThreads, r = e % kGradRows;
-            const int64_t n = n0 + e / kGradRows;
-            const bool in = n < hi && r < dcols;
-            rd[i] = in ? dsrc[n * dld + r] : 0.f;
-            rt[i] = in && w3 ? __ldg(T + n * C + r0 + r) : 0.f;
-            rm[i] = in && w3 ? __ldg(Mk + n * C + r0 + r) : 0.5f;   // 2 m (y - t) = dz below
+            const bool in = din && dn + i * kDStep < left;
+            rd[i] = in ? dp[i * kDStep * dld] : 0.f;
+            rt[i] = in && w3 ? __ldg(tp + i * kDStep * (int64_t)C) : 0.f;
+            rm[i] = in && w3 ? __ldg(mp + i * kDStep * (int64_t)C) : 0.5f;   // 2 m (y - t) = dz below
         }
 #pragma unroll
-        for (int i = 0; i < kHn; ++i) {
-            const int e = tid + i * kMlpThreads, c = e % kH;
-            const int64_t n = n0 + e / kH;
-            rh[i] = n < hi && c < hcols ? __ldg(hsrc + n * hld + c) : 0.f;
-        }
+        for (int i = 0; i < kHn; ++i)
+            rh[i] = hin && hn + i * kHStep < left ? __ldg(hp + i * kHStep * hld) : 0.f;
+        dp += kGradChunk * dld;
+        tp += kGradChunk * (int64_t)C;
+        mp += kGradChunk * (int64_t)C;
+        hp += kGradChunk * hld;
+        left -= kGradChunk;
     };
     float acc[kGradRows][2], bias = 0.f;
 #pragma unroll
     for (int r = 0; r < kGradRows; ++r) acc[r][0] = acc[r][1] = 0.f;
-    if (lo < hi) load(lo);
+    if (left > 0) load();
     // while those arrive, one warp adds the delta blocks' mask counts (and, in
     // the first block, their losses): the same sum in every block
     if (warp == kWarps - 1) {
@@ -421,7 +436,7 @@ __global__ void __launch_bounds__(kMlpThreads) grad_kernel(
         for (int i = 0; i < kHn; ++i)
             (&sh[0][0])[tid + i * kMlpThreads] = seg == 1 || rh[i] > 0.f ? rh[i] : 0.f;
         __syncthreads();
-        if (n0 + kGradChunk < hi) load(n0 + kGradChunk);
+        if (left > 0) load();
 #pragma unroll
         for (int s = 0; s < kGradChunk / kWarps; ++s) {
             const int n = warp + s * kWarps;
