@@ -171,7 +171,8 @@ alp_status alp_gemm_batched_varsize_noalloc(int64_t count, const int64_t* dM, co
 
 /* Host-only query (no GPU needed): how alp_emul_slice_products cuts a launch
  * of `tiles` tiles with `nslices` slices on `sms` SMs in the one-block
- * arrangement (CTA pairs share the groups of the last tiles one by one).  Blocks [0, *n_full) take whole tiles; each remaining
+ * arrangement (CTA pairs share the groups of the last tiles one by one).
+ * Blocks [0, *n_full) take whole tiles; each remaining
  * tile (the last, partial wave) is taken by *pieces blocks, piece i computing
  * the group sums S^t for t = t_lo[i]..t_hi[i] (arrays of 8).  The cut is the
  * contiguous one whose largest piece (in digit pairs of the kind's scheme:

@@ -3,8 +3,10 @@
 // Arrangements (emul_arrangement_of): by default a CTA pair (2-block cluster)
 // per 256 x 256 tile of C, its tcgen05 MMAs (.cta_group::2, M = 256) spanning
 // both SMs; otherwise one block per 128 x 256 tile.  In the last, partial wave
-// each tile is cut into up to 8 blocks (or pairs) by ranges of groups t
-// (tail_split below) so that the wave ends sooner.  Per block:
+// the tiles' groups (moduli) are shared: one by one by all pairs (pair_segment,
+// fused_item), or, with one block per tile, in up to 8 ranges (tail_split below).
+// Where even that leaves pairs idle, their tiles are narrower (narrow_tiles).
+// Per block:
 //
 //   warp 0      TMA producer: 128x64 A and 256x64 (pair: 128x64) B tiles
 //               (128-byte swizzle) into a shared-memory ring of stages
@@ -724,8 +726,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
 //
 // A persistent launch of CTA pairs (P clusters, all resident) that take
 // items from a counter as they go, an item being a whole 256 x 256 tile (all
-// n moduli; items 0..n_full-1 in raster order) or one piece of a tail tile (a
-// range of moduli; tail_split).  Block 0's producer takes the cluster's next
+// n moduli; items 0..n_full-1 in raster order) or a share of the units (tile,
+// modulus) of the tail tiles (fused_item).  Block 0's producer takes the cluster's next
 // item when it has issued the copies of the current one and publishes it in
 // the cluster's list in global memory; every other role of both blocks reads
 // the list (bounded waits), so that a pair that runs faster takes more items

@@ -360,10 +360,9 @@ def tune_batched_classes(M, N, K, pA, pB, pC, alpha=1.5, beta=0.5, runs=3,
         if log:
             log(f"class {c}: {n} problems, default {old} {times.get(tuple(old), float('nan')):.3f} ms"
                 f" -> {win} {times[win]:.3f} ms")
-    # Each class was timed alone; in one batch the largest tile of any class
-    # decides the persistent kernel's variant (128: one block per SM, 64: two,
-    # 32: three).  Time the whole batch with the per-class winners and with the
-    # best tiles of at most 64 and of at most 32, and keep the fastest table.
+    # Each class was timed alone; in one batch the classes' raster strips share
+    # L2.  Time the whole batch with the per-class winners and with the best
+    # tiles of at most 64 and of at most 32, and keep the fastest table.
     def capped(cap):
         return {c: min((k for k in v[2] if max(k[0], k[1]) <= cap), key=lambda k: (v[2][k], k))
                 for c, v in out.items()}
