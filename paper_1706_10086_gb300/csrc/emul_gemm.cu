@@ -962,9 +962,14 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
                 tc_fence_after();
                 const uint32_t taddr =
                     tmem_base + ((uint32_t)(quarter * 32) << 16) + b * kTN + half * hcols;
+                if (hcols == 128) {   // (a branch at each of the four costs 0.5 % at 8192^3)
 #pragma unroll
-                for (int cc = 0; cc < 4; ++cc)
-                    if (cc * 32 < hcols) tmem_drain32_cvt(taddr + cc * 32, &acc[cc * 32]);
+                    for (int cc = 0; cc < 4; ++cc)
+                        tmem_drain32_cvt(taddr + cc * 32, &acc[cc * 32]);
+                } else {
+                    tmem_drain32_cvt(taddr, &acc[0]);
+                    if (hcols == 64) tmem_drain32_cvt(taddr + 32, &acc[32]);
+                }
                 tc_fence_before();
                 __syncwarp();
                 // the first epilogue warp forwards block 1's hand-backs

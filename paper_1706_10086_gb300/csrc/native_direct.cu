@@ -5,9 +5,10 @@
 //
 // Measured on GB300 through alp_gemm_f64 (us; the shared-memory kernel's
 // default config before, this file after; floor 2MNK / 1.098 TFLOP/s):
-//   64^3      151.6 ->   9.9          512^3    1168 ->   262 (floor 244)
+//   64^3      151.6 ->   6.2          512^3    1168 ->   262 (floor 244)
 //   2048^3    18575 -> 15694 (15646)  1021 x 771 x 1333, A^T: 3154 -> 1960 (1911)
-// 8192 x 8192 x 2048 runs 249,700 (250,340).
+// 8192 x 8192 x 2048 runs 249,700 (250,340).  The 64^3 call is bound by its issue;
+// its kernel takes 4.7.
 #include <algorithm>
 
 #include "native_direct.cuh"
