@@ -136,7 +136,6 @@ struct EmulGemmParams {
     // test hook: block 0's producer arms pipeline stage inject_skip_it (its
     // running stage count) without issuing the copies (-1: off)
     int64_t inject_skip_it;
-    int narrow;   // pairs: tiles of kTN >> narrow columns (narrow_tiles)
     // modular scheme: the weighted reduction of modulus l's sums
     CrtByte crt[kCrtMaxModuli];
 };
@@ -243,13 +242,9 @@ __device__ __forceinline__ bool epilogue_jobs(const EmulGemmParams& prm, const u
     // forwards block 1's hand-backs); warp: its index in the block, whose
     // value modulo 4 fixes the TMEM lanes it may access
     const int quarter = warp & 3;
-    const int hcols = 128 >> prm.narrow;
-    const int half = ew >> 2;              // columns [hcols*half, hcols*half + hcols)
+    const int half = ew >> 2;              // columns [128*half, 128*half + 128)
     const int row = quarter * 32 + lane;
     const int gm = m0 + row;
-    // whether columns 0.., 32.. and 64.. of this thread's are stored
-    const uint32_t stored[3] = {gm < prm.M ? 1u : 0u, gm < prm.M && hcols > 32 ? 1u : 0u,
-                                gm < prm.M && hcols > 64 ? 1u : 0u};
     uint32_t acc[128];
     const uint32_t zero = prm.modular ? kCrtSumZero : 0u;
 #pragma unroll
@@ -260,14 +255,9 @@ __device__ __forceinline__ bool epilogue_jobs(const EmulGemmParams& prm, const u
         if (!mbar_wait_bounded(&accf[b], (job >> 1) & 1, tmo, abort_flag, prm.err)) return false;
         tc_fence_after();
         const uint32_t taddr =
-            tmem_base + ((uint32_t)(quarter * 32) << 16) + b * kTN + half * hcols;
-        if (hcols == 128) {   // (a branch at each of the four: f32 4096^3 665 -> 675 us)
+            tmem_base + ((uint32_t)(quarter * 32) << 16) + b * kTN + half * 128;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_drain32_cvt(taddr + c * 32, &acc[c * 32]);
-        } else {
-            tmem_drain32_cvt(taddr, &acc[0]);
-            if (hcols == 64) tmem_drain32_cvt(taddr + 32, &acc[32]);
-        }
+        for (int c = 0; c < 4; ++c) tmem_drain32_cvt(taddr + c * 32, &acc[c * 32]);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) hand_back(acce, acce_remote, agg, b, job, ew + 2, tmo, abort_flag, prm.err);
@@ -278,14 +268,15 @@ __device__ __forceinline__ bool epilogue_jobs(const EmulGemmParams& prm, const u
             const int l = job_p(jd) - 1;
             const CrtByte k = prm.crt[l];
             uint8_t* g = reinterpret_cast<uint8_t*>(prm.G) + (int64_t)l * prm.gplane +
-                         (int64_t)gm * prm.ldg + n0 + half * hcols;
+                         (int64_t)gm * prm.ldg + n0 + half * 128;
+            const uint32_t do_store = gm < prm.M ? 1u : 0u;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 uint32_t w[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) w[x] = crt_bytes4(acc + 16 * i + 4 * x, k);
-                store4_and_zero(reinterpret_cast<int32_t*>(g + 16 * i), stored[i < 2 ? 0 : i < 4 ? 1 : 2],
-                                w[0], w[1], w[2], w[3]);
+                store4_and_zero(reinterpret_cast<int32_t*>(g + 16 * i), do_store, w[0], w[1],
+                                w[2], w[3]);
             }
 #pragma unroll
             for (int i = 0; i < 128; ++i) acc[i] = zero;
@@ -296,11 +287,12 @@ __device__ __forceinline__ bool epilogue_jobs(const EmulGemmParams& prm, const u
             // bounds; rows past M are not stored.  Each asm block stores acc
             // and zeroes it in place.
             int32_t* g = prm.G + (int64_t)(t_group - 2) * prm.gplane + (int64_t)gm * prm.ldg +
-                         n0 + half * hcols;
+                         n0 + half * 128;
+            const uint32_t do_store = gm < prm.M ? 1u : 0u;
 #pragma unroll
             for (int i = 0; i < 32; ++i)
-                store4_and_zero(g + 4 * i, stored[i < 8 ? 0 : i < 16 ? 1 : 2], acc[4 * i], acc[4 * i + 1],
-                                acc[4 * i + 2], acc[4 * i + 3]);
+                store4_and_zero(g + 4 * i, do_store, acc[4 * i], acc[4 * i + 1], acc[4 * i + 2],
+                                acc[4 * i + 3]);
         }
     }
     return true;
@@ -602,7 +594,6 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         int job = 0, tile, g_lo, g_hi, m0, n0;
         for (int i = 0; pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
             pair_tile_origin(prm, tile, rank, m0, n0);
-            n0 >>= prm.narrow;
             if (!epilogue_jobs(prm, jobs, first[g_lo], first[g_hi], job, tmem_base, accf, &acce[0],
                                acce_remote, agg, m0, n0, warp, lane, tmo, abort_flag, warp - 4))
                 break;
@@ -619,7 +610,6 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             int tile, g_lo, g_hi, m0, n0;
             for (int i = 0; ok && pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
             pair_tile_origin(prm, tile, rank, m0, n0);
-            n0 >>= prm.narrow;
             const int j_end = first[g_hi];
             for (int j = first[g_lo]; j < j_end && ok; ++j) {
                 const uint32_t jd = jobs[j];
@@ -630,14 +620,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                         ok = false;
                         break;
                     }
-                    if (leader)
-                        mbar_arrive_expect_tx(&full[st], 2 * (kATile + (kPairBTile >> prm.narrow)));
+                    if (leader) mbar_arrive_expect_tx(&full[st], 2 * kPairStageBytes);
                     // fault injection: block 0 issues no copy, the stage never fills
                     if ((int64_t)it == prm.inject_skip_it && blockIdx.x == 0) continue;
                     unsigned char* a = tiles + st * kPairStageBytes;
                     tma_load_3d_pair(a, &tmA, full0 + st * 8, kb * kTK, m0, job_p(jd) - 1);
                     tma_load_3d_pair(a + kATile, &tmB, full0 + st * 8, kb * kTK,
-                                     n0 + (int)rank * ((kTN / 2) >> prm.narrow), job_q(jd) - 1);
+                                     n0 + (int)rank * (kTN / 2), job_q(jd) - 1);
                 }
             }
             }
@@ -660,7 +649,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     } else if (warp == 1) {
         if (lane == 0 && leader) {
             // ---------------- MMA issuer (block 0) ----------------
-            const uint32_t idesc = idesc_bf16_f32(2 * kTM, kTN >> prm.narrow);
+            const uint32_t idesc = idesc_bf16_f32(2 * kTM, kTN);
             uint32_t it = 0;
             int job = 0, tile, g_lo, g_hi;
             bool ok = true;
@@ -759,6 +748,7 @@ struct CrtFuse {
     int n_items;        // whole tiles n_full, then the parts of the tail tiles
     int parts;
     int tail_tiles;     // pair tiles - n_full
+    int narrow;         // tiles of kTN >> narrow columns (fused_narrow)
     int rec;            // whole tiles are reconstructed in the launch
     // the schedule (workspace, all bytes 0xff before the launch): sched[0] the
     // item counter, sched[1 + c * stride + k] the k-th item of cluster c
@@ -935,7 +925,7 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
                                                volatile int* abort_flag) {
     const int quarter = warp & 3;                      // TMEM lanes this warp may access
     const int half = (warp - kFusedEpiWarp0) >> 2;     // columns [hcols*half, hcols*half + hcols)
-    const int hcols = 128 >> prm.narrow;
+    const int hcols = 128 >> fz.narrow;
     const int row = quarter * 32 + lane;
     const int kblocks = (int)((prm.K + kTK - 1) / kTK), cpm = (kblocks + 15) / 16;
     uint32_t acc[128];
@@ -949,7 +939,7 @@ __device__ __forceinline__ void fused_epilogue(const EmulGemmParams& prm, const 
             int pid, q, m0, n0;
             fused_unit(prm, fz, fu, pid, q);
             pair_tile_origin(prm, pid, rank, m0, n0);
-            n0 >>= prm.narrow;
+            n0 >>= fz.narrow;
             const int gm = m0 + row;
 #pragma unroll
             for (int x = 0; x < 128; ++x) acc[x] = kCrtSumZero;
@@ -1119,7 +1109,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                     int pid, q, m0, n0;
                     fused_unit(prm, fz, fu, pid, q);
                     pair_tile_origin(prm, pid, rank, m0, n0);
-                    n0 >>= prm.narrow;
+                    n0 >>= fz.narrow;
                     for (int kb = 0; kb < kblocks; ++kb, ++it) {
                         const uint32_t st = it % kPairStages, round = it / kPairStages;
                         if (it >= (uint32_t)kPairStages &&
@@ -1128,13 +1118,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                             ok = false;
                             break;
                         }
-                        if (leader) mbar_arrive_expect_tx(&full[st], 2 * (kATile + (kPairBTile >> prm.narrow)));
+                        if (leader) mbar_arrive_expect_tx(&full[st], 2 * (kATile + (kPairBTile >> fz.narrow)));
                         // fault injection: block 0 issues no copy, the stage never fills
                         if ((int64_t)it == prm.inject_skip_it && blockIdx.x == 0) continue;
                         unsigned char* a = tiles + st * kPairStageBytes;
                         tma_load_3d_pair(a, &tmA, full0 + st * 8, kb * kTK, m0, q);
                         tma_load_3d_pair(a + kATile, &tmB, full0 + st * 8, kb * kTK,
-                                         n0 + (int)rank * ((kTN / 2) >> prm.narrow), q);
+                                         n0 + (int)rank * ((kTN / 2) >> fz.narrow), q);
                     }
                 }
             }
@@ -1153,7 +1143,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     } else if (warp == 1) {
         if (lane == 0 && leader) {
             // ---------------- MMA issuer (block 0) ----------------
-            const uint32_t idesc = idesc_bf16_f32(2 * kTM, kTN >> prm.narrow);
+            const uint32_t idesc = idesc_bf16_f32(2 * kTM, kTN >> fz.narrow);
             uint32_t it = 0;
             int job = 0;
             bool ok = true;
@@ -1317,20 +1307,6 @@ static int fused_active_clusters() {
     return c;
 }
 
-// Tiles of 128 or 64 columns (1 or 2) where all units of a launch on CTA pairs
-// (a modulus or a group of one tile) still have one of the P clusters each: a
-// unit's products, drains and stores are that much shorter (256^3 with 15 moduli
-// 20.8 -> 19.0 us, 64^3 18.9 -> 16.4; eight 7-bit slices at 256^3 37.4 -> 28.7,
-// three FP32 slices at 512^3 27.2 -> 21.0).  A fused launch then needs no
-// schedule, and its planes are rebuilt by the kernel that follows.
-static int narrow_tiles(int64_t M, int64_t N, int n, int64_t P) {
-    if (!emul_tail_split_on()) return 0;
-    const int64_t rows = (M + 2 * kTM - 1) / (2 * kTM);
-    int s = 0;
-    while (s < 2 && rows * ((N + (kTN >> (s + 1)) - 1) / (kTN >> (s + 1))) * n <= P) ++s;
-    return s;
-}
-
 alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bfloat16* da,
                            const __nv_bfloat16* db, int64_t kpad, int32_t* G, int64_t ldg,
                            cudaStream_t stream, int group_m, int cluster, int digit_bits,
@@ -1356,13 +1332,10 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     const int arr = (cluster == kEmulSingle || cluster == kEmulPair) ? cluster : emul_cluster();
     const int cl = arr == kEmulSingle ? 1 : 2;   // blocks per cluster
     if (paired) *paired = cl == 2;
-    const int64_t P = cl == 2 ? fused_active_clusters() : 0;
-    const int narrow = cl == 2 ? narrow_tiles(M, N, s, P) : 0;
     CUtensorMap ta, tb;
     alp_status st = make_tmap_3d_bf16(&ta, da, (uint64_t)kpad, (uint64_t)M, (uint64_t)s, kTK, kTM);
     if (st != ALP_OK) return st;
-    st = make_tmap_3d_bf16(&tb, db, (uint64_t)kpad, (uint64_t)N, (uint64_t)s, kTK,
-                           (kTN / cl) >> narrow);
+    st = make_tmap_3d_bf16(&tb, db, (uint64_t)kpad, (uint64_t)N, (uint64_t)s, kTK, kTN / cl);
     if (st != ALP_OK) return st;
     EmulGemmParams p;
     p.M = M;
@@ -1376,9 +1349,7 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     p.G = G;
     p.ldg = ldg;
     p.gplane = M * ldg;
-    p.narrow = narrow;
-    const int64_t tiles_m = (M + kTM - 1) / kTM;
-    const int64_t tiles_n = (N + (kTN >> narrow) - 1) / (kTN >> narrow);
+    const int64_t tiles_m = (M + kTM - 1) / kTM, tiles_n = (N + kTN - 1) / kTN;
     if (tiles_m * tiles_n > 0x7fffffff) return ALP_ERR_UNSUPPORTED;
     p.tiles_m = (int)tiles_m;
     p.tiles_n = (int)tiles_n;
@@ -1418,6 +1389,7 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     // of its own, which the hardware hands out as pairs become free (a fixed
     // assignment lets fast and slow pairs drift apart, by 3 % over 13 waves).
     constexpr int64_t kStaticWaves = 8;
+    const int64_t P = fused_active_clusters();
     const int64_t waves = pair_tiles / P;
     // (a rest of more than nine tenths of a wave stays whole: sharing it would
     // gain less than its clusters lose by reading different slices, 526 us
@@ -1505,6 +1477,18 @@ static FusedCut fused_cut(int64_t tiles, int n, int64_t kblocks, int P) {
     return c;
 }
 
+// Tiles of 128 or 64 columns (1 or 2) where all units of a launch still have a
+// cluster of their own: a unit's products, drains and stores are that much
+// shorter (256^3 with 15 moduli: 20.8 -> 19.0 us, 64^3: 18.9 -> 16.4).  Every unit is then the only one of its cluster, so no
+// schedule is used, and the planes are rebuilt by the kernel that follows.
+static int fused_narrow(int64_t M, int64_t N, int n, int P) {
+    if (!emul_tail_split_on()) return 0;
+    const int64_t rows = (M + 2 * kTM - 1) / (2 * kTM);
+    int s = 0;
+    while (s < 2 && rows * ((N + (kTN >> (s + 1)) - 1) / (kTN >> (s + 1))) * n <= P) ++s;
+    return s;
+}
+
 alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
                                        const __nv_bfloat16* da, const __nv_bfloat16* db,
                                        int64_t kpad, uint8_t* G, int64_t ldg, const int32_t* e,
@@ -1529,7 +1513,7 @@ alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
     if (st != ALP_OK) return st;
     const int P = fused_active_clusters() < kMaxFusedClusters ? fused_active_clusters()
                                                                : kMaxFusedClusters;
-    const int narrow = narrow_tiles(M, N, n, P);
+    const int narrow = fused_narrow(M, N, n, P);
     st = make_tmap_3d_bf16(&tb, db, (uint64_t)kpad, (uint64_t)N, (uint64_t)n, kTK,
                            (kTN / 2) >> narrow);
     if (st != ALP_OK) return st;
@@ -1562,7 +1546,7 @@ alp_status emul_crt_products_recombine(int64_t M, int64_t N, int64_t K, int n,
     p.pieces = 1;
     p.t_ranges = 0;
     CrtFuse fz;
-    p.narrow = narrow;
+    fz.narrow = narrow;
     const FusedCut cut = fused_cut(pair_tiles, n, (K + kTK - 1) / kTK, P);
     p.n_full = (int)cut.n_full;
     fz.parts = cut.parts;

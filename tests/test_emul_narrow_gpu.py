@@ -40,31 +40,3 @@ def test_narrow_tiles_match_the_stages(alp, M, N, K, n, alpha, beta):
     torch.cuda.synchronize()
     assert alp.alp_get_device_error() == alp.ALP_OK
     assert np.array_equal(got.cpu().numpy(), want.cpu().numpy())
-
-
-@pytest.mark.parametrize("M,N,K,kind,s", [
-    (1, 1, 1, "BF16", 3), (256, 64, 64, "BF16", 8), (257, 65, 1025, "BF16", 8),
-    (255, 129, 300, "BF16_B8", 7), (512, 512, 130, "BF16_B8_TRIM", 5), (200, 257, 2049, "BF16", 3),
-    (256, 608, 100, "BF16", 8), (256, 609, 100, "BF16", 8)])
-def test_narrow_digit_tiles_match_single_blocks(alp, M, N, K, kind, s):
-    """Digit schemes: the pairs' narrow tiles against the single-block
-    arrangement's 128 x 256 ones, chosen by a tuned config."""
-    import torch
-    A, B, C = inputs.gemm_operands(7400 + M + N + K, M, N, K, kind="scaled", phi=3)
-    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
-    sk = getattr(alp, "ALP_SLICE_" + kind)
-    ws = alp.alp_gemm_f64_emul_workspace(M, N, K, s, sk)
-    out = []
-    for cfg in (None, (128, 256, 64, 1, 0, 8)):
-        work = torch.full((ws,), 255, dtype=torch.uint8, device="cuda")
-        got = torch.from_numpy(C.copy()).cuda()
-        if cfg is not None:
-            alp.alp_tune_set_cached(M, N, K, alp.ALP_PATH_EMUL, cfg)
-        try:
-            alp.alp_gemm_f64_emul(M, N, K, -0.75, dA, K, dB, N, 0.5, got, N, s, sk, work, ws)
-        finally:
-            alp.alp_tune_clear_cache()
-        torch.cuda.synchronize()
-        assert alp.alp_get_device_error() == alp.ALP_OK
-        out.append(got.cpu().numpy())
-    assert np.array_equal(out[0], out[1])
