@@ -5,7 +5,8 @@
 // both SMs; otherwise one block per 128 x 256 tile.  In the last, partial wave
 // the tiles' groups (moduli) are shared: one by one by all pairs (pair_segment,
 // fused_item), or, with one block per tile, in up to 8 ranges (tail_split below).
-// Where even that leaves pairs idle, their tiles are narrower (narrow_tiles).
+// Where even that leaves pairs of the fused kernel idle, tiles are narrower
+// (fused_narrow).
 // Per block:
 //
 //   warp 0      TMA producer: 128x64 A and 256x64 (pair: 128x64) B tiles
