@@ -166,11 +166,20 @@ class Trainer:
                 self.std.cpu().numpy().copy())
 
 
+# Decoupled weight decay of a training step, times its learning rate (Loshchilov
+# and Hutter 2019).  Without it the choice on held-out shapes depends on the
+# initial weights: 400 shapes, both paths, four seeds: mean regret 1.0-3.1 %
+# (single cases 100 %), 0.9-1.0 % with it.
+WEIGHT_DECAY = 1.0
+
+
 def train(ds, epochs=3000, lr=3e-3, seed=1706 + 4, log_every=0):
     tr = Trainer(ds, seed)
     hist = [tr.current_loss()]
     for e in range(epochs):
-        tr.epoch(lr if e < epochs * 0.7 else lr * 0.1)
+        step = lr if e < epochs * 0.7 else lr * 0.1
+        tr.epoch(step)
+        tr.params.mul_(1.0 - step * WEIGHT_DECAY)
         if log_every and (e + 1) % log_every == 0:
             hist.append(tr.current_loss())
     hist.append(tr.current_loss())
