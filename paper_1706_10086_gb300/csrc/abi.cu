@@ -98,17 +98,16 @@ int device_sm_count() {
 }
 
 uint64_t wait_timeout_ns() {
-    if (g_timeout_ns.load() == 0) {
-        std::lock_guard<std::mutex> lk(g_mu);
-        if (g_timeout_ns.load() != 0) return g_timeout_ns;
-        double ms = 4000.0;   // default: 4 s per wait; no legitimate wait comes close
-        if (const char* s = std::getenv("ALP_WAIT_TIMEOUT_MS")) {
-            double v = std::atof(s);
-            if (v > 0) ms = v;
-        }
-        g_timeout_ns = (uint64_t)(ms * 1e6);
+    uint64_t ns = g_timeout_ns.load();
+    if (ns) return ns;
+    double ms = 4000.0;   // default: 4 s per wait; no legitimate wait comes close
+    if (const char* s = std::getenv("ALP_WAIT_TIMEOUT_MS")) {
+        double v = std::atof(s);
+        if (v > 0) ms = v;
     }
-    return g_timeout_ns;
+    // a limit set since the load stays
+    const uint64_t first = (uint64_t)(ms * 1e6);
+    return g_timeout_ns.compare_exchange_strong(ns, first) ? first : ns;
 }
 
 alp_status cuda_status(cudaError_t e) { return e == cudaSuccess ? ALP_OK : ALP_ERR_CUDA; }
