@@ -37,6 +37,7 @@
 // the block writes S^t to G[t-2] (int32), or, for the modular scheme, the byte
 // (Q_l y_l) mod m_l to plane l-1 of G.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 
 #include "crt.cuh"
@@ -1281,31 +1282,41 @@ TailSplit tail_split(int tiles, int s, int sms, bool trim, bool crt) {
     return ts;
 }
 
-// CTA-pair clusters that are resident at once (the persistent grids; the
-// fused kernel's footprint, which the product kernel's equals); half the SMs if the query fails.
+// CTA-pair clusters that are resident at once (the persistent grids), asked once
+// per device for the fused kernel; the product kernel also runs one block of as
+// many threads per SM, with a little more shared memory.  The kernel's limit is
+// raised before the query, which else refuses its shared memory.  Half the SMs
+// if it fails; kept either way, since the schedule's words and the launch that
+// uses them must agree on it.
 static int fused_active_clusters() {
-    static int c = 0;
-    if (c == 0) {
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((unsigned)(2 * device_sm_count()));
-        lc.blockDim = dim3(kFusedThreads);
-        lc.dynamicSmemBytes = kFusedSmemBytes;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        lc.attrs = attr;
-        lc.numAttrs = 1;
-        int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, emul_crt_fused_pair_kernel, &lc) != cudaSuccess ||
-            nc < 1) {
-            (void)cudaGetLastError();
-            nc = device_sm_count() / 2;
-        }
-        c = nc > 0 ? nc : 1;
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const bool keep = dev >= 0 && dev < kDevices;
+    if (keep && known[dev].load() > 0) return known[dev].load();
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)(2 * device_sm_count()));
+    lc.blockDim = dim3(kFusedThreads);
+    lc.dynamicSmemBytes = kFusedSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(emul_crt_fused_pair_kernel,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kFusedSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, emul_crt_fused_pair_kernel, &lc) != cudaSuccess ||
+        n < 1) {
+        (void)cudaGetLastError();
+        n = std::max(device_sm_count() / 2, 1);
     }
-    return c;
+    if (keep) known[dev].store(n);
+    return n;
 }
 
 alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bfloat16* da,
