@@ -801,8 +801,8 @@ def batched_leg(args, torch, alp, dev, stream, tune=True):
     tiles autotuned first, outside the timed region), against loops of
     single-problem native launches: with the default config on one stream, the
     same captured in a CUDA graph, and a fairer loop whose problems take the
-    best of LOOP_CANDIDATES for their size class (timed per class) and run
-    round-robin on four streams."""
+    best of LOOP_CANDIDATES or no config for their size class (timed per class)
+    and run round-robin on four streams."""
     import numpy as np
 
     from paper_1706_10086_gb300 import inputs
@@ -853,7 +853,7 @@ def batched_leg(args, torch, alp, dev, stream, tune=True):
     stream.wait_stream(side)
     ms_loop_graph = timed(gl.replay, 1, 1)
     del gl
-    # fairer loop: per size class the fastest candidate config, four streams
+    # fairer loop: per size class the fastest candidate (None: no config), four streams
     cls = np.array([alp.alp_batched_class_of(int(m), int(q)) for m, q in zip(M, N)])
     best = {}
     for c in sorted(set(cls.tolist())):
@@ -864,8 +864,9 @@ def batched_leg(args, torch, alp, dev, stream, tune=True):
                 alp.alp_gemm_f64(int(M[p]), int(N[p]), int(K[p]), 1.5, int(pA[p]), int(K[p]),
                                  int(pB[p]), int(N[p]), 0.5, int(pC[p]), int(N[p]), cfg=cfg,
                                  stream=stream)
-        times = {cfg: timed(lambda cfg=cfg: run_class(cfg), 1, 1) for cfg in LOOP_CANDIDATES}
-        best[c] = min(times, key=lambda k: (times[k], k))
+        times = {cfg: timed(lambda cfg=cfg: run_class(cfg), 1, 1)
+                 for cfg in (None,) + LOOP_CANDIDATES}
+        best[c] = min(times, key=times.get)
     cfgs = [best[c] for c in cls]
     streams = [torch.cuda.Stream(dev) for _ in range(4)]
 
@@ -890,7 +891,7 @@ def batched_leg(args, torch, alp, dev, stream, tune=True):
             "loop_of_launches_graph": {"ms": round(ms_loop_graph, 3), "tflops": tf(ms_loop_graph)},
             "loop_tuned_per_class_4_streams": {
                 "ms": round(ms_fair, 3), "tflops": tf(ms_fair),
-                "configs": {str(c): list(v) for c, v in best.items()}},
+                "configs": {str(c): list(v) if v else None for c, v in best.items()}},
             "speedup_vs_loop": round(ms_loop / ms_graph, 3),
             "speedup_vs_tuned_loop_4_streams": round(ms_fair / ms_graph, 3)}
 

@@ -94,11 +94,11 @@ const char* alp_status_string(alp_status s);
 /*
  * Native FP64 GEMM, Eq. 1 (Sect. 2, Fig. 2): TMA-staged A and B tiles in a
  * multi-stage mbarrier ring, FP64 DMMA tensor-core MMAs into per-thread
- * register tiles, alpha/beta epilogue.  cfg == NULL selects the config from the
- * tuned cache, else the loaded cost model; without either the call runs the
- * register-direct kernels, which cut the work evenly over the SMs for any
- * shape, alignment and leading dimension (a k range may be shared by a
- * cluster's blocks, its partial sums added in a fixed order).
+ * register tiles, alpha/beta epilogue.  cfg == NULL runs the register-direct
+ * kernels, which cut the work evenly over the SMs for any shape, alignment and
+ * leading dimension (a k range may be shared by a cluster's blocks, its partial
+ * sums added in a fixed order), unless the tuned cache has a config for
+ * (M, N, K) that was set by hand or that the sweep timed faster than them.
  * With a config, operands whose base address is not 16-byte aligned, or whose
  * lda/ldb is odd, run through a non-TMA variant of the same kernel.
  * Returns ALP_ERR_INVALID_ARG for negative sizes, ld < row width, NULL
@@ -416,7 +416,9 @@ size_t alp_gemm_batched_workspace(int64_t count, const int64_t* hM, const int64_
  * at N = 10240 and keeps the best).  EXHAUSTIVE: times every valid config of
  * `path` on the current GPU (10 CUDA-event-timed runs after warm-up, best
  * kept), appends each timing to the JSONL database (env ALP_TUNE_DB, if set),
- * and caches the winner for (M,N,K,path).  PREDICT: the cost model's argmin
+ * and caches the winner for (M,N,K,path); on the native path it times the
+ * register-direct kernels too, and calls with cfg == NULL keep running those
+ * where no config is faster.  PREDICT: the cost model's argmin
  * over valid configs (ALP_ERR_NOT_TUNED without a loaded model).  LOOKUP:
  * cached winner only.  out: the chosen config; out_tflops: its measured (or
  * for PREDICT, predicted) TFLOP/s, may be NULL.  Allocates its own scratch.

@@ -66,8 +66,9 @@ alp_status alp_debug_inject_skip(int kt);
  * tensor-core stage).  Allocates its own scratch. */
 alp_status alp_tune_time_config(int64_t M, int64_t N, int64_t K, alp_path path,
                                 const alp_config* cfg, int use_proxy, int runs, double* est_ms);
-/* Puts cfg into the tuned cache for (M, N, K, path) (what alp_tune(EXHAUSTIVE)
- * does with its winner), and empties the cache. */
+/* Puts cfg into the tuned cache for (M, N, K, path), for every later call with
+ * cfg == NULL (alp_tune(EXHAUSTIVE) does the same with its winner where that is
+ * the fastest there is), and empties the cache. */
 alp_status alp_tune_set_cached(int64_t M, int64_t N, int64_t K, alp_path path,
                                const alp_config* cfg);
 alp_status alp_tune_clear_cache(void);
@@ -102,9 +103,10 @@ alp_status alp_mlp_backward(const float* params, int C, const float* X, int64_t 
 alp_status alp_mlp_adam(float* params, const float* grads, float* m, float* v, int64_t n,
                         int step, float lr, float beta1, float beta2, float eps, void* stream);
 /* Installs a trained model (HOST arrays: params, 7-float mean and std) for
- * alp_tune(PREDICT) and for GEMM calls with cfg == NULL that miss the tuned
- * cache (the prediction runs the forward kernel once per new shape, then it
- * is cached); unload removes it. */
+ * alp_tune(PREDICT) and for emulated GEMM calls that miss the tuned cache (the
+ * prediction runs the forward kernel once per new shape, then it is cached);
+ * unload removes it.  Native calls with cfg == NULL do not ask it: the
+ * register-direct kernels they run are no slower than any config. */
 alp_status alp_tune_load_model(const float* host_params, int C, const float* host_mean,
                                const float* host_std);
 alp_status alp_tune_unload_model(void);

@@ -25,8 +25,9 @@ alp_status native_scale(int64_t M, int64_t N, double beta, double* C, int64_t ld
                         cudaStream_t stream);
 alp_status native_direct(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
                          const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
-                         double* C, int64_t ldc, cudaStream_t stream);
-// tune.cu: tuned cache, then cost model; false when neither has a config.
+                         double* C, int64_t ldc, cudaStream_t stream, int cut = -1,
+                         int64_t tile_limit = 0);
+// tune.cu: the config a call without one runs with; false when there is none.
 bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                   cudaStream_t stream);
 
@@ -198,8 +199,9 @@ const char* alp_status_string(alp_status s) {
     return "unknown alp_status";
 }
 
-// The tile config of a native call: the caller's, a tuned one, or the default
-// while the fault-injection hook is on.  False: none, native_direct runs.
+// The tile config of a native call: the caller's, a cached one that was set or
+// timed faster than the register-direct kernels, or the default while the
+// fault-injection hook is on.  False: none, native_direct runs.
 static bool pick_config(int64_t M, int64_t N, int64_t K, const alp_config* cfg, alp_config* c,
                         cudaStream_t s) {
     if (cfg) {

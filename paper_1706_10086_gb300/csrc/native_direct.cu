@@ -148,10 +148,13 @@ int native_direct_cut(int64_t M, int64_t N, int64_t K, int sms) {
 }
 
 // C = alpha op(A) op(B) + beta C for M, N, K > 0 and alpha != 0, every size
-// below 2^31; any alignment and leading dimensions.
+// below 2^31; any alignment and leading dimensions.  cut: as native_direct_cut
+// gives it (-1: asked here); tile_limit > 0: only the first that many tiles or
+// fragments of C (the tuner's timing proxy).
 alp_status native_direct(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
                          const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
-                         double* C, int64_t ldc, cudaStream_t stream) {
+                         double* C, int64_t ldc, cudaStream_t stream, int cut,
+                         int64_t tile_limit) {
     DirectParams p;
     p.A = ta ? DirectOperand{A, 1, lda} : DirectOperand{A, lda, 1};
     p.B = tb ? DirectOperand{B, ldb, 1} : DirectOperand{B, 1, ldb};
@@ -163,10 +166,12 @@ alp_status native_direct(int ta, int tb, int64_t M, int64_t N, int64_t K, double
     p.alpha = alpha;
     p.beta = beta;
     p.vec2 = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && ldc % 2 == 0;
-    const int cut = native_direct_cut(M, N, K, device_sm_count());
+    if (cut < 0) cut = native_direct_cut(M, N, K, device_sm_count());
     p.tiles_m = cut ? (M + 15) / 16 : (M + 31) / 32;
     p.tiles_n = cut ? (N + 7) / 8 : (N + 15) / 16;
-    const int64_t blocks = p.tiles_m * p.tiles_n * std::max(cut, 1);
+    int64_t tiles = p.tiles_m * p.tiles_n;
+    if (tile_limit > 0) tiles = std::min(tiles, tile_limit);
+    const int64_t blocks = tiles * std::max(cut, 1);
     if (blocks > 0x7fffffff) return ALP_ERR_UNSUPPORTED;
     if (cut <= 1) {
         auto kernel = cut ? dgemm_direct_split_kernel : dgemm_direct_kernel;

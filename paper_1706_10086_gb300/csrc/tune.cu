@@ -38,6 +38,10 @@ alp_status native_launch(const alp_config& cfg, bool use_tma, int64_t M, int64_t
                          int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t stream,
                          int inject_skip_kt, int64_t grid_limit);
 int native_occupancy(const alp_config& cfg, bool use_tma);
+int native_direct_cut(int64_t M, int64_t N, int64_t K, int sms);
+alp_status native_direct(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
+                         const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
+                         double* C, int64_t ldc, cudaStream_t stream, int cut, int64_t tile_limit);
 bool default_config(alp_path path, alp_config* out);
 bool model_loaded();
 bool model_predict(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
@@ -61,7 +65,11 @@ constexpr int kTimedRuns = 10;          // the paper keeps the best of ten runs
 
 std::mutex g_tmu;
 std::atomic<bool> g_cached{false};   // g_cache may have entries
-std::map<std::tuple<int64_t, int64_t, int64_t, int>, alp_config> g_cache;
+struct Tuned {
+    alp_config cfg;
+    bool direct;   // timed no faster than the register-direct kernels (native path)
+};
+std::map<std::tuple<int64_t, int64_t, int64_t, int>, Tuned> g_cache;
 
 const int kBM[3] = {64, 128, 256};
 const int kBK[3] = {16, 32, 64};
@@ -197,9 +205,36 @@ bool time_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_confi
     return true;
 }
 
+// Estimated time (ms) of the register-direct kernels on the whole problem, as
+// the configs' proxy takes it: at most kDirectWaves waves of blocks and kProxyK
+// k per warp, in the cut the whole problem takes.
+constexpr int64_t kDirectWaves = 16;
+bool time_direct(int64_t M, int64_t N, int64_t K, Scratch& sc, cudaStream_t st, int runs,
+                 double* est_ms) {
+    const int64_t sms = device_sm_count();
+    const int cut = native_direct_cut(M, N, K, (int)sms), size = std::max(cut, 1);
+    const int64_t tiles = cut ? ((M + 15) / 16) * ((N + 7) / 8) : ((M + 31) / 32) * ((N + 15) / 16);
+    const int64_t Kp = std::min(K, kProxyK * (cut ? 4 * cut : 1));
+    const int64_t run_tiles = std::min(tiles, std::max<int64_t>(kDirectWaves * sms / size, 1));
+    const size_t ba = up256((size_t)M * Kp * 8), bb = up256((size_t)Kp * N * 8);
+    if (!sc.get(ba + bb + up256((size_t)M * N * 8))) return false;
+    char* base = static_cast<char*>(sc.p);
+    const double* A = reinterpret_cast<const double*>(base);
+    const double* B = reinterpret_cast<const double*>(base + ba);
+    double* C = reinterpret_cast<double*>(base + ba + bb);
+    auto launch = [&]() {
+        return native_direct(0, 0, M, N, Kp, 1.0, A, Kp, B, N, 0.0, C, N, st, cut, run_tiles);
+    };
+    double best, median;
+    if (!time_launch(launch, st, runs, &best, &median)) return false;
+    auto waves = [&](int64_t t) { return std::ceil((double)(t * size) / (double)sms); };
+    *est_ms = best * (waves(tiles) / waves(run_tiles)) * ((double)K / (double)Kp);
+    return true;
+}
+
 void db_append(int64_t M, int64_t N, int64_t K, alp_path path, const std::vector<alp_config>& cs,
                const std::vector<double>& est, const std::vector<double>& best,
-               const std::vector<double>& med, int winner, bool proxy) {
+               const std::vector<double>& med, int winner, bool proxy, double direct) {
     const char* path_env = std::getenv("ALP_TUNE_DB");
     if (!path_env || !*path_env) return;
     FILE* f = std::fopen(path_env, "a");
@@ -224,7 +259,12 @@ void db_append(int64_t M, int64_t N, int64_t K, alp_path path, const std::vector
                       est[i], best[i], med[i]);
         line += buf;
     }
-    line += "]}\n";
+    line += "]";
+    if (std::isfinite(direct)) {   // ms of the register-direct kernels
+        std::snprintf(buf, sizeof buf, ", \"direct\": %.6g", direct);
+        line += buf;
+    }
+    line += "}\n";
     std::fputs(line.c_str(), f);
     std::fclose(f);
 }
@@ -237,26 +277,33 @@ std::vector<alp_config> configs_of(alp_path path) {
     return {};
 }
 
-void cache_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_config& c) {
+void cache_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_config& c,
+                  bool direct = false) {
     std::lock_guard<std::mutex> lk(g_tmu);
-    g_cache[std::make_tuple(M, N, K, (int)path)] = c;
+    g_cache[std::make_tuple(M, N, K, (int)path)] = {c, direct};
     g_cached.store(true);
 }
 
-// Config of a GEMM issued with cfg == NULL: the tuned cache, else the cost
-// model's prediction (made once per shape and then cached; skipped while
-// `stream` is being captured, since the prediction synchronises).  False when
-// neither has one.
+// Config of a GEMM issued with cfg == NULL: the tuned cache's, else, on the
+// emulated path, the cost model's prediction (made once per shape and then
+// cached; skipped while `stream` is being captured, since the prediction
+// synchronises).  False when there is none, and on the native path also where
+// the sweep timed its best config no faster than the register-direct kernels
+// (64^3: 73 us with the best config, 6.2 without).  The model, which only knows
+// configs, is not asked there: a config's tiles are made of the direct kernels'
+// 32 x 16 ones, so its busiest sub-partition never has fewer MMAs (4096^3: 125.1
+// ms without a config, 125.6 with the tuned one).
 bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                    cudaStream_t stream) {
     if (g_cached.load()) {
         std::lock_guard<std::mutex> lk(g_tmu);
         auto it = g_cache.find(std::make_tuple(M, N, K, (int)path));
         if (it != g_cache.end()) {
-            *out = it->second;
-            return true;
+            *out = it->second.cfg;
+            return !it->second.direct;
         }
     }
+    if (path == ALP_PATH_NATIVE) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (model_loaded() && cudaStreamIsCapturing(stream, &cs) == cudaSuccess &&
         cs == cudaStreamCaptureStatusNone &&
@@ -315,7 +362,7 @@ alp_status alp_tune(int64_t M, int64_t N, int64_t K, alp_path path, alp_tune_mod
         std::lock_guard<std::mutex> lk(g_tmu);
         auto it = g_cache.find(std::make_tuple(M, N, K, (int)path));
         if (it == g_cache.end()) return ALP_ERR_NOT_TUNED;
-        *out = it->second;
+        *out = it->second.cfg;
         if (out_tflops) *out_tflops = 0.0;
         return ALP_OK;
     }
@@ -343,12 +390,14 @@ alp_status alp_tune(int64_t M, int64_t N, int64_t K, alp_path path, alp_tune_mod
              alp_config_smem_bytes(&cs[i]) < alp_config_smem_bytes(&cs[winner])))
             winner = (int)i;
     }
+    double direct = INFINITY;   // a failure leaves the sweep's winner
+    if (path == ALP_PATH_NATIVE && !time_direct(M, N, K, sc, st, runs, &direct)) direct = INFINITY;
     cudaStreamSynchronize(st);
     cudaStreamDestroy(st);
     if (winner < 0) return ALP_ERR_CUDA;
     const bool proxy = path == ALP_PATH_NATIVE ? (K > kProxyK) : (K > proxy_k_emul());
-    db_append(M, N, K, path, cs, est, best, med, winner, proxy);
-    cache_config(M, N, K, path, cs[winner]);
+    db_append(M, N, K, path, cs, est, best, med, winner, proxy, direct);
+    cache_config(M, N, K, path, cs[winner], direct <= est[winner]);
     *out = cs[winner];
     if (out_tflops) *out_tflops = flops / (est[winner] * 1e-3) / 1e12;
     return ALP_OK;
