@@ -99,6 +99,9 @@ const char* alp_status_string(alp_status s);
  * leading dimension (a k range may be shared by a cluster's blocks, its partial
  * sums added in a fixed order), unless the tuned cache has a config for
  * (M, N, K) that was set by hand or that the sweep timed faster than them.
+ * Every config gives the same bits, and so does the batched call; the
+ * register-direct kernels give others where they share a k range, which depends
+ * on the shape and the GPU's SM count (alp_native_cut in alp_ext.h).
  * With a config, operands whose base address is not 16-byte aligned, or whose
  * lda/ldb is odd, run through a non-TMA variant of the same kernel.
  * Returns ALP_ERR_INVALID_ARG for negative sizes, ld < row width, NULL

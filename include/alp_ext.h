@@ -169,6 +169,16 @@ alp_status alp_gemm_batched_varsize_noalloc(int64_t count, const int64_t* dM, co
                                             const int64_t* dldc, const int64_t* hM,
                                             const int64_t* hN, const int64_t* hK, void* stream);
 
+/* ---- native path: launch shape ------------------------------------------------ */
+
+/* Host-only query (no GPU needed): how a native call without a config cuts
+ * M x N x K on a GPU of `sms` SMs: 0 whole 32 x 16 tiles of C over their k range,
+ * else 16 x 8 fragments whose k range is shared by the four warps of each of 1,
+ * 2, 4 or 8 blocks (the value), whose partial sums are added in a fixed order.
+ * The results' bits depend on it, and so on the GPU's SM count.  -1 for sizes or
+ * sms below 1. */
+int alp_native_cut(int64_t M, int64_t N, int64_t K, int sms);
+
 /* ---- emulated path: launch shape -------------------------------------------- */
 
 /* Host-only query (no GPU needed): how alp_emul_slice_products cuts a launch

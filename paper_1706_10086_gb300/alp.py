@@ -126,6 +126,7 @@ _SIGS = {
     "alp_set_wait_timeout_ms": ([_f64], _int),
     "alp_debug_inject_skip": ([_int], _int),
     "alp_probe_fp64_peak": ([_int, _i64, _int, _int, ctypes.POINTER(_f64), _vp], _int),
+    "alp_native_cut": ([_i64, _i64, _i64, _int], _int),
     "alp_emul_tail_split": ([_int, _int, _int, _int, ctypes.POINTER(_int), ctypes.POINTER(_int),
                              ctypes.POINTER(_int), ctypes.POINTER(_int)], _int),
     "alp_tune_time_config": ([_i64, _i64, _i64, _int, ctypes.POINTER(alp_config), _int, _int,
@@ -517,6 +518,10 @@ def alp_probe_fp64_peak(kind=0, iters=20000, blocks_per_sm=2, threads=256, strea
     _check(lib().alp_probe_fp64_peak(int(kind), int(iters), int(blocks_per_sm), int(threads),
                                      ctypes.byref(out), _s(stream)), "alp_probe_fp64_peak", True)
     return out.value
+
+
+def alp_native_cut(M, N, K, sms) -> int:
+    return int(lib().alp_native_cut(M, N, K, int(sms)))
 
 
 def alp_emul_tail_split(tiles, nslices, kind, sms):

@@ -11,6 +11,7 @@
 // its kernel takes 4.7.
 #include <algorithm>
 
+#include "alp_ext.h"
 #include "native_direct.cuh"
 #include "tc.cuh"
 
@@ -193,3 +194,8 @@ alp_status native_direct(int ta, int tb, int64_t M, int64_t N, int64_t K, double
 }
 
 }  // namespace alp
+
+extern "C" int alp_native_cut(int64_t M, int64_t N, int64_t K, int sms) {
+    if (M <= 0 || N <= 0 || K <= 0 || sms <= 0) return -1;
+    return alp::native_direct_cut(M, N, K, sms);
+}
