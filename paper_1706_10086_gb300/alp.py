@@ -192,20 +192,23 @@ def _p(x):
     return x.data_ptr()
 
 
-_torch_c = None   # torch._C, once CUDA is initialised
+_raw = None   # torch's (raw stream of a device, current device); () if it lacks them
 
 
 def _current_stream():
     """Handle of the current torch stream, without building a Stream object
-    (with the C side's locks gone, a 64^3 call is issued in 5.6 us, not 9.9)."""
-    global _torch_c
-    c = _torch_c
-    if c is None:
-        import torch
-        handle = torch.cuda.current_stream().cuda_stream   # initialises CUDA
-        _torch_c = torch._C
-        return handle
-    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+    (with the C side's locks gone, a 64^3 call is issued in 5.6 us, not 9.9)
+    where this torch has the two functions, private ones, that this takes."""
+    global _raw
+    if _raw:
+        stream_of, device = _raw
+        return stream_of(device())
+    import torch
+    handle = torch.cuda.current_stream().cuda_stream   # initialises CUDA
+    if _raw is None:
+        fs = [getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice")]
+        _raw = tuple(fs) if all(fs) else ()
+    return handle
 
 
 def _s(stream):
