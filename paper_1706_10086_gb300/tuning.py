@@ -323,13 +323,14 @@ def validate_full_runs(model, train_ds, test_ds, tuning_ds=None, count=50, max_f
 
 def tune_batched_classes(M, N, K, pA, pB, pC, alpha=1.5, beta=0.5, runs=3,
                          tiles=(32, 64, 128), bks=(16, 32), log=None):
-    """Autotunes the batched GEMM's tile per size class: for every class
+    """Autotunes the batched GEMM's raster strip per size class: for every class
     present in the batch, times the class's own problems (alp_gemm_batched_varsize
     on that sub-batch, CUDA events, best of ``runs`` after a warm-up) with each
-    candidate (bm, bn, bk) and installs the fastest with
-    alp_batched_set_class_config.  M, N, K, pA, pB, pC are host arrays (sizes and
-    device addresses of row-major operands with tight leading dimensions).
-    Returns {class: ((bm, bn, bk), ms, {candidate: ms})}."""
+    bm of ``tiles`` and installs the fastest with alp_batched_set_class_config.
+    bn and bk change nothing that the kernel runs: candidates carry the class's
+    own, kept within ``tiles`` and ``bks``.  M, N, K, pA, pB, pC are host arrays
+    (sizes and device addresses of row-major operands with tight leading
+    dimensions).  Returns {class: ((bm, bn, bk), ms, {candidate: ms})}."""
     import torch
     dev = torch.device("cuda")
     M, N, K = (np.ascontiguousarray(a, dtype=np.int64) for a in (M, N, K))
@@ -347,22 +348,22 @@ def tune_batched_classes(M, N, K, pA, pB, pC, alpha=1.5, beta=0.5, runs=3,
         ws = alp.alp_gemm_batched_workspace(n, hM, hN, hK)
         work = torch.empty(max(ws, 1), dtype=torch.uint8, device=dev)
         old = alp.alp_batched_get_class_config(c)
+        bn = old[1] if old[1] in tiles else tiles[0]
+        bk = old[2] if old[2] in bks else bks[0]
         times = {}
         for bm in tiles:
-            for bn in tiles:
-                for bk in bks:
-                    alp.alp_batched_set_class_config(c, bm, bn, bk)
-                    alp.alp_gemm_batched_varsize(*args, work, ws, stream=stream)
-                    best = float("inf")
-                    for _ in range(runs):
-                        e0 = torch.cuda.Event(enable_timing=True)
-                        e1 = torch.cuda.Event(enable_timing=True)
-                        e0.record(stream)
-                        alp.alp_gemm_batched_varsize(*args, work, ws, stream=stream)
-                        e1.record(stream)
-                        e1.synchronize()
-                        best = min(best, e0.elapsed_time(e1))
-                    times[(bm, bn, bk)] = best
+            alp.alp_batched_set_class_config(c, bm, bn, bk)
+            alp.alp_gemm_batched_varsize(*args, work, ws, stream=stream)
+            best = float("inf")
+            for _ in range(runs):
+                e0 = torch.cuda.Event(enable_timing=True)
+                e1 = torch.cuda.Event(enable_timing=True)
+                e0.record(stream)
+                alp.alp_gemm_batched_varsize(*args, work, ws, stream=stream)
+                e1.record(stream)
+                e1.synchronize()
+                best = min(best, e0.elapsed_time(e1))
+            times[(bm, bn, bk)] = best
         win = min(times, key=lambda k: (times[k], k))
         alp.alp_batched_set_class_config(c, *win)
         out[c] = (win, times[win], times)
@@ -371,9 +372,9 @@ def tune_batched_classes(M, N, K, pA, pB, pC, alpha=1.5, beta=0.5, runs=3,
                 f" -> {win} {times[win]:.3f} ms")
     # Each class was timed alone; in one batch the classes' raster strips share
     # L2.  Time the whole batch with the per-class winners and with the best
-    # tiles of at most 64 and of at most 32, and keep the fastest table.
+    # strips of at most 64 and of at most 32 rows, and keep the fastest table.
     def capped(cap):
-        return {c: min((k for k in v[2] if max(k[0], k[1]) <= cap), key=lambda k: (v[2][k], k))
+        return {c: min((k for k in v[2] if k[0] <= cap), key=lambda k: (v[2][k], k))
                 for c, v in out.items()}
     tables = [{c: v[0] for c, v in out.items()}]
     for cap in (64, 32):
@@ -404,7 +405,7 @@ def tune_batched_classes(M, N, K, pA, pB, pC, alpha=1.5, beta=0.5, runs=3,
             return best
         ts = [whole(tb) for tb in tables]
         if log:
-            log("whole batch: " + ", ".join(f"{max(max(k[0], k[1]) for k in tb.values())}-wide "
+            log("whole batch: " + ", ".join(f"strips to {max(k[0] for k in tb.values())} "
                                             f"{t:.3f} ms" for tb, t in zip(tables, ts)))
         chosen = tables[int(np.argmin(ts))]
         for c, cfg in chosen.items():
