@@ -108,9 +108,10 @@ void crt_weights(int n, CrtByte (&b)[kCrtMaxModuli]) {
 // float minus 1.5 2^23 and kSplitBias mod m is an integer x = A' (mod m); q =
 // RN(x / m) by RN(1/m) and 1.5 2^23, and r = x - q m by one fma, exact.
 // x RN(1/m) is off by at most 2^-13, so q is RN(x / m) or one off it next to a
-// half-integer, and |r| <= m / 2 + 0.04, an integer at most 128.  Six instructions per modulus and none to cut A' up (three 13-bit
-// chunks turned into floats and three fmas each before, six and some 14 per
-// value, and eleven integer ones for k >= 52: 2048 x 2048 with 15 moduli, k = 52).
+// half-integer, and |r| <= m / 2 + 0.04, an integer at most 128.  Six
+// instructions per modulus and none to cut A' up (three 13-bit chunks turned
+// into floats and three fmas each before, six and some 14 per value, and eleven
+// integer ones for k >= 52: 2048 x 2048 with 15 moduli, k = 52).
 constexpr uint64_t kSplitBias = 0x4338000000000000ull;   // the encoding of 1.5 2^52
 
 // The constants of modulus l, as literals: kept in the constant bank, the

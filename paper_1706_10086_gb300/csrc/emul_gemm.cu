@@ -611,26 +611,26 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             bool ok = true;
             int tile, g_lo, g_hi, m0, n0;
             for (int i = 0; ok && pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
-            pair_tile_origin(prm, tile, rank, m0, n0);
-            const int j_end = first[g_hi];
-            for (int j = first[g_lo]; j < j_end && ok; ++j) {
-                const uint32_t jd = jobs[j];
-                for (int kb = job_kb(jd); kb < job_ke(jd); ++kb, ++it) {
-                    const uint32_t st = it % kPairStages, round = it / kPairStages;
-                    if (it >= (uint32_t)kPairStages &&
-                        !mbar_wait_bounded(&empty[st], (round - 1) & 1, tmo, abort_flag, prm.err)) {
-                        ok = false;
-                        break;
+                pair_tile_origin(prm, tile, rank, m0, n0);
+                const int j_end = first[g_hi];
+                for (int j = first[g_lo]; j < j_end && ok; ++j) {
+                    const uint32_t jd = jobs[j];
+                    for (int kb = job_kb(jd); kb < job_ke(jd); ++kb, ++it) {
+                        const uint32_t st = it % kPairStages, round = it / kPairStages;
+                        if (it >= (uint32_t)kPairStages &&
+                            !mbar_wait_bounded(&empty[st], (round - 1) & 1, tmo, abort_flag, prm.err)) {
+                            ok = false;
+                            break;
+                        }
+                        if (leader) mbar_arrive_expect_tx(&full[st], 2 * kPairStageBytes);
+                        // fault injection: block 0 issues no copy, the stage never fills
+                        if ((int64_t)it == prm.inject_skip_it && blockIdx.x == 0) continue;
+                        unsigned char* a = tiles + st * kPairStageBytes;
+                        tma_load_3d_pair(a, &tmA, full0 + st * 8, kb * kTK, m0, job_p(jd) - 1);
+                        tma_load_3d_pair(a + kATile, &tmB, full0 + st * 8, kb * kTK,
+                                         n0 + (int)rank * (kTN / 2), job_q(jd) - 1);
                     }
-                    if (leader) mbar_arrive_expect_tx(&full[st], 2 * kPairStageBytes);
-                    // fault injection: block 0 issues no copy, the stage never fills
-                    if ((int64_t)it == prm.inject_skip_it && blockIdx.x == 0) continue;
-                    unsigned char* a = tiles + st * kPairStageBytes;
-                    tma_load_3d_pair(a, &tmA, full0 + st * 8, kb * kTK, m0, job_p(jd) - 1);
-                    tma_load_3d_pair(a + kATile, &tmB, full0 + st * 8, kb * kTK,
-                                     n0 + (int)rank * (kTN / 2), job_q(jd) - 1);
                 }
-            }
             }
             // The MMAs of every issued stage must have consumed it (so this
             // block's copies have landed, on block 0's barrier) and its
@@ -656,38 +656,38 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             int job = 0, tile, g_lo, g_hi;
             bool ok = true;
             for (int i = 0; ok && pair_segment(prm, cid, i, tile, g_lo, g_hi); ++i) {
-            const int j_end = first[g_hi];
-            for (int j = first[g_lo]; j < j_end && ok; ++j, ++job) {
-                const uint32_t jd = jobs[j];
-                const uint32_t b = job & 1;
-                if (job >= 2 &&
-                    !mbar_wait_bounded(&acce[b], ((job >> 1) - 1) & 1, tmo, abort_flag, prm.err)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + b * kTN;
-                uint32_t accumulate = 0;
-                for (int kb = job_kb(jd); kb < job_ke(jd); ++kb, ++it) {
-                    const uint32_t st = it % kPairStages, round = it / kPairStages;
-                    if (!mbar_wait_bounded(&full[st], round & 1, tmo, abort_flag, prm.err)) {
+                const int j_end = first[g_hi];
+                for (int j = first[g_lo]; j < j_end && ok; ++j, ++job) {
+                    const uint32_t jd = jobs[j];
+                    const uint32_t b = job & 1;
+                    if (job >= 2 &&
+                        !mbar_wait_bounded(&acce[b], ((job >> 1) - 1) & 1, tmo, abort_flag, prm.err)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t a_addr = smem_u32(tiles + st * kPairStageBytes);
-                    const uint64_t adesc = sw128_kmajor_desc(a_addr);
-                    const uint64_t bdesc = sw128_kmajor_desc(a_addr + kATile);
+                    const uint32_t d_tmem = tmem_base + b * kTN;
+                    uint32_t accumulate = 0;
+                    for (int kb = job_kb(jd); kb < job_ke(jd); ++kb, ++it) {
+                        const uint32_t st = it % kPairStages, round = it / kPairStages;
+                        if (!mbar_wait_bounded(&full[st], round & 1, tmo, abort_flag, prm.err)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t a_addr = smem_u32(tiles + st * kPairStageBytes);
+                        const uint64_t adesc = sw128_kmajor_desc(a_addr);
+                        const uint64_t bdesc = sw128_kmajor_desc(a_addr + kATile);
 #pragma unroll
-                    for (int kk = 0; kk < kTK / 16; ++kk) {
-                        umma_bf16_pair(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, accumulate);
-                        accumulate = 1;
+                        for (int kk = 0; kk < kTK / 16; ++kk) {
+                            umma_bf16_pair(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, accumulate);
+                            accumulate = 1;
+                        }
+                        umma_commit_pair(&empty[st], 3);
                     }
-                    umma_commit_pair(&empty[st], 3);
+                    if (!ok) break;
+                    umma_commit_pair(&accf[b], 3);
                 }
-                if (!ok) break;
-                umma_commit_pair(&accf[b], 3);
-            }
             }
             // all MMAs must have completed before TMEM and shared memory go away,
             // and both blocks' hand-backs of the last two chunks must have
@@ -1120,7 +1120,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                             ok = false;
                             break;
                         }
-                        if (leader) mbar_arrive_expect_tx(&full[st], 2 * (kATile + (kPairBTile >> fz.narrow)));
+                        if (leader)
+                            mbar_arrive_expect_tx(&full[st],
+                                                  2 * (kATile + (kPairBTile >> fz.narrow)));
                         // fault injection: block 0 issues no copy, the stage never fills
                         if ((int64_t)it == prm.inject_skip_it && blockIdx.x == 0) continue;
                         unsigned char* a = tiles + st * kPairStageBytes;
@@ -1491,8 +1493,9 @@ static FusedCut fused_cut(int64_t tiles, int n, int64_t kblocks, int P) {
 
 // Tiles of 128 or 64 columns (1 or 2) where all units of a launch still have a
 // cluster of their own: a unit's products, drains and stores are that much
-// shorter (256^3 with 15 moduli: 20.8 -> 19.0 us, 64^3: 18.9 -> 16.4).  Every unit is then the only one of its cluster, so no
-// schedule is used, and the planes are rebuilt by the kernel that follows.
+// shorter (256^3 with 15 moduli: 20.8 -> 19.0 us, 64^3: 18.9 -> 16.4).  Every
+// unit is then the only one of its cluster, so no schedule is used, and the
+// planes are rebuilt by the kernel that follows.
 static int fused_narrow(int64_t M, int64_t N, int n, int P) {
     if (!emul_tail_split_on()) return 0;
     const int64_t rows = (M + 2 * kTM - 1) / (2 * kTM);

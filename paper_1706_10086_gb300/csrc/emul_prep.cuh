@@ -293,7 +293,8 @@ __device__ __forceinline__ void prep_cols(const PrepParams<T>& p, const PrepOper
     typename ScanKey<T>::type mx[kPrepV<T>];
     prep_fill(o, p.K, j0, kb0, rows, p.block_k, tile, mx);
     if (p.known) {
-        if (threadIdx.x < W) sexp[threadIdx.x] = j0 + threadIdx.x < o.R ? __ldg(o.exps + j0 + threadIdx.x) : 0;
+        if (threadIdx.x < W)
+            sexp[threadIdx.x] = j0 + threadIdx.x < o.R ? __ldg(o.exps + j0 + threadIdx.x) : 0;
     } else {
         const auto m = prep_column_max<T>(mx, red, cmax, size);
         if (threadIdx.x < W) {
@@ -315,7 +316,8 @@ __device__ __forceinline__ void prep_cols(const PrepParams<T>& p, const PrepOper
         const int e = sexp[c];
         const T* col = tile + c * ld;
 #pragma unroll 1
-        for (int k = 4 * lane + 128 * (warp / W); k < rows; k += 128 * (kPrepWarps > W ? kPrepWarps / W : 1)) {
+        for (int k = 4 * lane + 128 * (warp / W); k < rows;
+             k += 128 * (kPrepWarps > W ? kPrepWarps / W : 1)) {
             const int q = k >> 2;
             const T a[4] = {col[q], col[Q + q], col[2 * Q + q], col[3 * Q + q]};
             split4<S>(sp, a, e, o.out + j * p.kpad + kb0 + k, plane);
