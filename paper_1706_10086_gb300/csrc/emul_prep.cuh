@@ -390,10 +390,19 @@ inline int prep_cut(PrepParams<T>& p, int sms) {
 // maxima and its split follow one another in each block, so that at 4096^2 a
 // scan and a split kernel of their own, each at the HBM rate, take 128 us
 // against 145 (2048^2: 41 and three launches against 35; float, with 6 bytes
-// written per element instead of 30, the strips win up to 5000^2).
+// written per element instead of 30, the strips win up to 5000^2).  Short lines
+// leave a block little to overlap that chain with, so that many of them are too
+// large as well (whole calls with M = 64, strips and separate, us; N x K is the
+// strided operand): 8 digits 24576 x 64 166 and 168, 32768 x 64 204 and 201, 131072
+// x 64 748 and 678; 32768 x 192 241 and 242, 61000 x 136 434 and 424; float, 3 digits
+// 49152 x 64 94 and 96, 65536 x 64 107.5 and 106.5, 131072 x 64 206 and 187, but 131072
+// x 256 255 and 268.
 template <typename T>
 inline bool prep_in_strips(int64_t R, int64_t K) {
-    return K <= kPrepMaxColK && R * K <= (sizeof(T) == 8 ? int64_t(1) << 23 : int64_t(1) << 25);
+    const int64_t strips = (R + kPrepStrip<T> - 1) / kPrepStrip<T>;
+    return K <= kPrepMaxColK &&
+           R * K <= (sizeof(T) == 8 ? int64_t(1) << 23 : int64_t(1) << 25) &&
+           strips <= (K <= 128 ? 6144 : sizeof(T) == 8 ? 8192 : int64_t(1) << 22);
 }
 
 // Launches `kernel` (of these roles) with the cut of p's operands.

@@ -1,0 +1,135 @@
+"""Which launches an emulated GEMM call makes: its strided operands prepared in
+strips together with the others, or by a scan and a split of their own.  A C
+program stands in for the runtime and records the launches, so no GPU is needed;
+the GPU tests compare the routes with the stages bit for bit."""
+import subprocess
+
+import pytest
+
+from paper_1706_10086_gb300 import alp as lib
+
+from .test_emul_prep_gpu import check
+
+PROGRAM = r"""
+#define _GNU_SOURCE
+#include <cuda_runtime_api.h>
+#include <dlfcn.h>
+#include <stdint.h>
+#include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
+static int word, launches, last_attrs;
+cudaError_t cudaGetDevice(int* d) { *d = 0; return 0; }
+cudaError_t cudaDeviceGetAttribute(int* v, enum cudaDeviceAttr a, int d) { *v = 152; return 0; }
+cudaError_t cudaMalloc(void** p, size_t n) { *p = &word; return 0; }
+cudaError_t cudaMemset(void* p, int v, size_t n) { return 0; }
+cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) { return 0; }
+cudaError_t cudaDeviceSynchronize(void) { return 0; }
+cudaError_t cudaGetLastError(void) { return 0; }
+cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) { return 0; }
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaunchConfig_t* c) {
+    *n = 76;
+    return 0;
+}
+cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void** a, size_t m, cudaStream_t s) {
+    ++launches;
+    last_attrs = 0;
+    return 0;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) { return 0; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t f, dim3 g, dim3 b, void** a, size_t m, cudaStream_t s) {
+    return cudaLaunchKernel(0, g, b, a, m, s);
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** a) {
+    ++launches;
+    last_attrs = (int)c->numAttrs;
+    return 0;
+}
+static int encode() { return 0; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** fn, unsigned v,
+                                             unsigned long long flags,
+                                             enum cudaDriverEntryPointQueryResult* r) {
+    *fn = (void*)encode;
+    *r = cudaDriverEntryPointSuccess;
+    return 0;
+}
+
+typedef int (*gemm64)(int, int, int64_t, int64_t, int64_t, double, const void*, int64_t,
+                      const void*, int64_t, double, void*, int64_t, int, int, void*, size_t, void*);
+typedef int (*gemm32)(int, int, int64_t, int64_t, int64_t, float, const void*, int64_t,
+                      const void*, int64_t, float, void*, int64_t, int, int, void*, size_t, void*);
+
+int main(int argc, char** argv) {
+    void* so = dlopen(argv[1], RTLD_NOW);
+    if (!so) return fprintf(stderr, "%s\n", dlerror()), 2;
+    gemm64 f64 = (gemm64)dlsym(so, "alp_gemm_f64_emul_ex");
+    gemm32 f32 = (gemm32)dlsym(so, "alp_gemm_f32_emul_ex");
+    char* p = (char*)0x10000000;   /* never read: nothing is launched */
+    int64_t M, N, K;
+    int is32, kind, n;
+    while (scanf("%d %d %d %ld %ld %ld", &is32, &kind, &n, &M, &N, &K) == 6) {
+        launches = 0;
+        const int rc =
+            is32 ? f32(0, 0, M, N, K, 1, p, K, p, N, 0, p, N, n, kind, p, (size_t)1 << 60, 0)
+                 : f64(0, 0, M, N, K, 1, p, K, p, N, 0, p, N, n, kind, p, (size_t)1 << 60, 0);
+        printf("%d %d %d\n", rc, launches, last_attrs);
+    }
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def routes(alp, tmp_path_factory):
+    """calls -> (launches, whether the last one may start early) of each."""
+    d = tmp_path_factory.mktemp("routes")
+    src, exe = d / "routes.c", d / "routes"
+    src.write_text(PROGRAM)
+    subprocess.run(["gcc", "-O1", "-w", "-rdynamic", "-I/usr/local/cuda/include", "-o", str(exe),
+                    str(src), "-ldl"], check=True)
+
+    def run(calls):
+        text = "\n".join(" ".join(str(int(v)) for v in c) for c in calls)
+        r = subprocess.run([str(exe), alp.LIB_PATH], input=text, capture_output=True, text=True,
+                           timeout=120)
+        assert r.returncode == 0, r.stderr
+        rows = [[int(v) for v in l.split()] for l in r.stdout.splitlines()]
+        assert len(rows) == len(calls) and all(row[0] == 0 for row in rows)
+        return [(row[1], row[2] > 0) for row in rows]
+    return run
+
+
+B7, B8, CRT = lib.ALP_SLICE_BF16, lib.ALP_SLICE_BF16_B8, lib.ALP_SLICE_BF16_CRT
+# (float, kind, slices, M, N, K): whether B is prepared in strips
+STRIPS = {
+    (0, B7, 8, 64, 64, 64): True, (0, CRT, 15, 64, 16384, 64): True,
+    (0, B7, 8, 64, 24576, 128): True, (0, B7, 8, 64, 24577, 128): False,
+    (0, CRT, 15, 64, 24576, 64): True, (0, CRT, 15, 64, 24580, 1): False,
+    (0, B7, 8, 64, 131072, 64): False, (0, CRT, 15, 64, 131072, 16): False,
+    (0, B7, 8, 64, 32768, 129): True, (0, B7, 8, 64, 32769, 129): False,
+    (0, B7, 8, 64, 32768, 256): True, (0, CRT, 15, 64, 1024, 8192): True,
+    (0, CRT, 15, 64, 1024, 8193): False, (0, CRT, 15, 64, 4097, 2048): False,
+    (1, B8, 3, 64, 49152, 128): True, (1, B8, 3, 64, 49153, 128): False,
+    (1, B8, 3, 64, 262144, 64): False, (1, B8, 3, 64, 131072, 129): True,
+    (1, B8, 3, 64, 131072, 256): True, (1, B8, 3, 64, 131073, 256): False}
+
+
+def test_strips_or_separate(routes):
+    """In strips: one preparation launch, then products and sums.  Separate:
+    the scan's two or three launches and the split before the other operand's."""
+    got = routes(STRIPS)
+    assert {c: n == 3 for c, (n, _) in zip(STRIPS, got)} == STRIPS
+    assert all(n in (3, 6) for n, _ in got), got
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", [(0, B7, 8, 3, 24576, 70), (0, B7, 8, 3, 24577, 70),
+                                  (0, CRT, 15, 5, 24579, 33), (0, B7, 3, 2, 32769, 130),
+                                  (1, B8, 3, 3, 49152, 70), (1, B8, 3, 3, 49157, 70)])
+@pytest.mark.parametrize("ta,pad,shift", [(0, 0, 0), (1, 1, 1)])
+def test_routes_agree_with_the_stages(alp, call, ta, pad, shift):
+    """Both sides of each line; with ta the long operand is A, stored K x M."""
+    f32, kind, n, M, N, K = call
+    if ta:
+        M, N = N, M
+    check(alp, M, N, K, kind, n, f32=bool(f32), ta=ta, pad=pad, shift=shift)
