@@ -310,6 +310,16 @@ __global__ void __launch_bounds__(256) recombine4_kernel(
     }
 }
 
+// Up to this many group sums a recombination starts while the products drain.
+// That saves the gap between the two launches, but started so the kernel runs
+// slower on sums that no longer come from L2 (whole calls, us, started early and
+// after the products: 8 digits 256^3 39.6 and 41.5, 1024^3 87 and 87, 2048^3 415 and
+// 411, 4096 x 4096 x 64 577 and 546, 8192 x 8192 x 64 2326 and 2225; float, 3 digits
+// 724 x 724 x 64 26.3 and 29.3, 2048^3 124 and 125, 4096^3 672 and 662, 8192 x 8192 x
+// 256 782 and 722).  Lines of equal cost: 8 sums of 1450^2, 7 of 1700^2, more than 4
+// of 2048^2.
+constexpr int64_t kEarlySumWords = int64_t(20) << 20;
+
 // Launch of a recombination kernel; early: the kernel before it on the stream
 // lets it start while that one drains.
 template <typename... P, typename... A>
@@ -724,6 +734,7 @@ alp_status emul_gemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, T alp
                               have ? cfg.stages : 0, have ? emul_arrangement_of(cfg) : 0, b,
                               sc.trim, sc.crt, prepared, &paired)) != ALP_OK)
         return st;
+    paired = paired && (int64_t)nslices * M * L.ldg <= kEarlySumWords;
     if constexpr (kF32)
         return launch_recombine_f32(nslices, b, recombine_grid(M, N), s, G, M * L.ldg, L.ldg, e,
                                     f, M, N, alpha, beta, C, ldc, paired);

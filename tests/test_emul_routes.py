@@ -1,5 +1,6 @@
 """Which launches an emulated GEMM call makes: its strided operands prepared in
-strips together with the others, or by a scan and a split of their own.  A C
+strips together with the others, or by a scan and a split of their own; the sums
+recombined by a kernel that starts while the products drain, or after them.  A C
 program stands in for the runtime and records the launches, so no GPU is needed;
 the GPU tests compare the routes with the stages bit for bit."""
 import subprocess
@@ -122,6 +123,21 @@ def test_strips_or_separate(routes):
     assert all(n in (3, 6) for n, _ in got), got
 
 
+# whether the kernel that makes C of the sums starts while the products drain
+EARLY = {
+    (0, B7, 8, 256, 256, 256): True, (0, B7, 8, 1280, 2048, 64): True,
+    (0, B7, 8, 1281, 2048, 64): False, (0, B7, 8, 1281, 2048, 2048): False,
+    (0, B7, 4, 2048, 2048, 64): True, (0, B7, 8, 8192, 8192, 64): False,
+    (1, B8, 3, 724, 724, 64): True, (1, B8, 3, 2048, 2048, 64): True,
+    (1, B8, 3, 4096, 4096, 64): False, (1, B8, 2, 3072, 3072, 64): True,
+    (1, B8, 3, 8192, 8192, 256): False, (0, CRT, 15, 4096, 4096, 64): True}
+
+
+def test_recombination_early_or_after(routes):
+    got = routes(EARLY)
+    assert {c: early for c, (_, early) in zip(EARLY, got)} == EARLY
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("call", [(0, B7, 8, 3, 24576, 70), (0, B7, 8, 3, 24577, 70),
                                   (0, CRT, 15, 5, 24579, 33), (0, B7, 3, 2, 32769, 130),
@@ -133,3 +149,11 @@ def test_routes_agree_with_the_stages(alp, call, ta, pad, shift):
     if ta:
         M, N = N, M
     check(alp, M, N, K, kind, n, f32=bool(f32), ta=ta, pad=pad, shift=shift)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", [(0, B7, 8, 1280, 2048, 40), (0, B7, 8, 1281, 2047, 40),
+                                  (1, B8, 3, 3300, 2048, 100), (0, B7, 3, 3000, 2600, 33)])
+def test_sums_agree_with_the_stages(alp, call):
+    f32, kind, n, M, N, K = call
+    check(alp, M, N, K, kind, n, f32=bool(f32))
