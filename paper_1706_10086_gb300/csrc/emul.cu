@@ -436,19 +436,24 @@ static alp_status emul_split_b(int64_t R, int64_t K, const T* X, int64_t ldx, in
                                const int32_t* exps, int s, __nv_bfloat16* out, int64_t kpad,
                                cudaStream_t st) {
     const bool vec = (reinterpret_cast<uintptr_t>(out) & 7) == 0 && kpad % 4 == 0;
+    const int sms = device_sm_count();
+    // rows: four k per thread, blocks no wider than a row needs (four digits of
+    // 262144 x 64 468 us with 256 threads, 115 with 32; 65536 x 256 132 and 62)
+    const int threads = kpad <= 128 ? 32 : kpad <= 256 ? 64 : kpad <= 512 ? 128 : 256;
     const int64_t bx = (kpad + 1023) / 1024;
-    int64_t by = (int64_t)device_sm_count() * 8 / bx;
+    int64_t by = (int64_t)sms * (2048 / threads) / bx;
     by = by < 1 ? 1 : by > R ? R : by > 65535 ? 65535 : by;
     const dim3 grid4((unsigned)bx, (unsigned)by);
+    const bool by_128 = vec && split_cols_by_128(R, kpad, sms);
 #define ALP_SPLIT_CASE(x)                                                                        \
     case x:                                                                                      \
         if (!trans && vec)                                                                       \
-            split_rows4_kernel<T, x, DigitSplit<B>><<<grid4, 256, 0, st>>>(X, R, K, ldx, exps,  \
-                                                                           out, kpad, {});    \
+            split_rows4_kernel<T, x, DigitSplit<B>><<<grid4, threads, 0, st>>>(                  \
+                X, R, K, ldx, exps, out, kpad, {});                                              \
         else if (!trans)                                                                         \
             split_rows_kernel<T, x, DigitSplit<B>><<<grid_for(R * (kpad / 2), 256), 256, 0, st>>>( \
                 X, R, K, ldx, exps, out, kpad, {});                                              \
-        else if (vec)                                                                            \
+        else if (by_128)                                                                         \
             split_cols4_kernel<T, x, DigitSplit<B>><<<dim3((unsigned)((R + 31) / 32),             \
                                                            (unsigned)((kpad + 127) / 128)),      \
                                                       256, 0, st>>>(X, K, R, ldx, exps, out,     \

@@ -205,6 +205,7 @@ alp_status emul_split_crt(int64_t R, int64_t K, const T* X, int64_t ldx, int tra
     int64_t blocks = (R * (kpad / 2) + 255) / 256;
     const int64_t cap = (int64_t)device_sm_count() * 16;
     blocks = blocks > cap ? cap : blocks < 1 ? 1 : blocks;
+    const bool by_128 = vec && split_cols_by_128(R, kpad, device_sm_count());
 #define ALP_CRT_SPLIT_CASE(x)                                                                    \
     case x:                                                                                      \
         if (!trans && vec)                                                                       \
@@ -213,7 +214,7 @@ alp_status emul_split_crt(int64_t R, int64_t K, const T* X, int64_t ldx, int tra
         else if (!trans)                                                                         \
             split_rows_kernel<T, x, CrtSplit><<<(unsigned)blocks, 256, 0, st>>>(                  \
                 X, R, K, ldx, exps, out, kpad, sp);                                              \
-        else if (vec)                                                                            \
+        else if (by_128)                                                                         \
             split_cols4_kernel<T, x, CrtSplit><<<dim3((unsigned)((R + 31) / 32),                  \
                                                       (unsigned)((kpad + 127) / 128)),           \
                                                  256, 0, st>>>(X, K, R, ldx, exps, out, kpad, sp); \

@@ -402,6 +402,18 @@ __global__ void __launch_bounds__(256, 4) split_cols4_kernel(
     }
 }
 
+// Whether the columns of an R-line operand go through split_cols4_kernel's 128-k
+// tiles rather than split_cols_kernel's of 64: not where a half empty last tile
+// is a fifteenth or more of them, nor where they leave SMs idle (us, 128 and 64;
+// lines x kpad).  Eight 7-bit digits: 65536 x 64 43.6 and 29.3, x 192 82.7 and 72.3,
+// x 320 122 and 113, x 256 86.7 and 90.8, 8192^2 298 and 320, 512^2 10.9 and 8.8; 15
+// moduli: 65536 x 64 51.8 and 35.5, x 256 107 and 115; float, 3 digits: 65536 x 64 19.1
+// and 15.0, x 128 23.2 and 25.2.
+inline bool split_cols_by_128(int64_t R, int64_t kpad, int sms) {
+    if (kpad % 128 != 0 && kpad < 1024) return false;
+    return (R + 31) / 32 * ((kpad + 127) / 128) >= 4 * (int64_t)sms;
+}
+
 // Nearest double (ties to even) of the 128-bit two's-complement integer
 // hi:lo, multiplied by 2^E: built from 32-bit integer operations on the IEEE
 // encoding (FP64 arithmetic is slow on this GPU).  The magnitude's top 64 bits

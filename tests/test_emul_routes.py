@@ -1,6 +1,7 @@
 """Which launches an emulated GEMM call makes: its strided operands prepared in
 strips together with the others, or by a scan and a split of their own; the sums
-recombined by a kernel that starts while the products drain, or after them.  A C
+recombined by a kernel that starts while the products drain, or after them; and
+the tiles and blocks of the splits.  A C
 program stands in for the runtime and records the launches, so no GPU is needed;
 the GPU tests compare the routes with the stages bit for bit."""
 import subprocess
@@ -20,6 +21,8 @@ PROGRAM = r"""
 #include <stdlib.h>
 #include <string.h>
 static int word, launches, last_attrs;
+static const void* last_kernel;
+static dim3 last_grid, last_block;
 cudaError_t cudaGetDevice(int* d) { *d = 0; return 0; }
 cudaError_t cudaDeviceGetAttribute(int* v, enum cudaDeviceAttr a, int d) { *v = 152; return 0; }
 cudaError_t cudaMalloc(void** p, size_t n) { *p = &word; return 0; }
@@ -35,11 +38,17 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaun
 cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void** a, size_t m, cudaStream_t s) {
     ++launches;
     last_attrs = 0;
+    last_kernel = f;
+    last_grid = g;
+    last_block = b;
     return 0;
 }
-cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) { return 0; }
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
+    *k = (cudaKernel_t)f;
+    return 0;
+}
 cudaError_t __cudaLaunchKernel(cudaKernel_t f, dim3 g, dim3 b, void** a, size_t m, cudaStream_t s) {
-    return cudaLaunchKernel(0, g, b, a, m, s);
+    return cudaLaunchKernel((const void*)f, g, b, a, m, s);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** a) {
     ++launches;
@@ -60,6 +69,9 @@ typedef int (*gemm64)(int, int, int64_t, int64_t, int64_t, double, const void*, 
 typedef int (*gemm32)(int, int, int64_t, int64_t, int64_t, float, const void*, int64_t,
                       const void*, int64_t, float, void*, int64_t, int, int, void*, size_t, void*);
 
+typedef int (*split)(int64_t, int64_t, const void*, int64_t, int, const void*, int, int, void*,
+                     int64_t, void*);
+
 int main(int argc, char** argv) {
     void* so = dlopen(argv[1], RTLD_NOW);
     if (!so) return fprintf(stderr, "%s\n", dlerror()), 2;
@@ -68,6 +80,17 @@ int main(int argc, char** argv) {
     char* p = (char*)0x10000000;   /* never read: nothing is launched */
     int64_t M, N, K;
     int is32, kind, n;
+    if (argc > 2) {   /* the split of R lines of K: which kernel, its grid and block */
+        split s64 = (split)dlsym(so, "alp_emul_split"), s32 = (split)dlsym(so, "alp_emul_split_f32");
+        int trans, shift;
+        while (scanf("%d %d %d %ld %ld %d %d", &is32, &kind, &n, &M, &K, &trans, &shift) == 7) {
+            const int rc = (is32 ? s32 : s64)(M, K, p, trans ? M : K, trans, p, n, kind, p + shift,
+                                              (K + 63) / 64 * 64, 0);
+            printf("%d %ld %u %u %u\n", rc, (long)last_kernel, last_grid.x, last_grid.y,
+                   last_block.x);
+        }
+        return 0;
+    }
     while (scanf("%d %d %d %ld %ld %ld", &is32, &kind, &n, &M, &N, &K) == 6) {
         launches = 0;
         const int rc =
@@ -81,23 +104,28 @@ int main(int argc, char** argv) {
 
 
 @pytest.fixture(scope="module")
-def routes(alp, tmp_path_factory):
-    """calls -> (launches, whether the last one may start early) of each."""
+def recorded(alp, tmp_path_factory):
     d = tmp_path_factory.mktemp("routes")
     src, exe = d / "routes.c", d / "routes"
     src.write_text(PROGRAM)
     subprocess.run(["gcc", "-O1", "-w", "-rdynamic", "-I/usr/local/cuda/include", "-o", str(exe),
                     str(src), "-ldl"], check=True)
 
-    def run(calls):
+    def run(calls, *args):
         text = "\n".join(" ".join(str(int(v)) for v in c) for c in calls)
-        r = subprocess.run([str(exe), alp.LIB_PATH], input=text, capture_output=True, text=True,
-                           timeout=120)
+        r = subprocess.run([str(exe), alp.LIB_PATH, *args], input=text, capture_output=True,
+                           text=True, timeout=120)
         assert r.returncode == 0, r.stderr
         rows = [[int(v) for v in l.split()] for l in r.stdout.splitlines()]
         assert len(rows) == len(calls) and all(row[0] == 0 for row in rows)
-        return [(row[1], row[2] > 0) for row in rows]
+        return [row[1:] for row in rows]
     return run
+
+
+@pytest.fixture(scope="module")
+def routes(recorded):
+    """calls -> (launches, whether the last one may start early) of each."""
+    return lambda calls: [(n, attrs > 0) for n, attrs in recorded(calls)]
 
 
 B7, B8, CRT = lib.ALP_SLICE_BF16, lib.ALP_SLICE_BF16_B8, lib.ALP_SLICE_BF16_CRT
@@ -138,6 +166,40 @@ def test_recombination_early_or_after(routes):
     assert {c: early for c, (_, early) in zip(EARLY, got)} == EARLY
 
 
+# (float, kind, slices, lines, K): whether the columns are split by 128-k tiles
+BY_128 = {
+    (0, B7, 8, 65536, 64): False, (0, B7, 8, 65536, 65): True, (0, B7, 8, 65536, 128): True,
+    (0, B7, 8, 65536, 129): False, (0, B7, 4, 65536, 192): False, (0, B7, 4, 32768, 448): False,
+    (0, B8, 7, 4096, 960): False, (0, B8, 7, 4096, 1088): True, (0, B7, 8, 8192, 8192): True,
+    (0, B7, 8, 512, 512): False, (0, B7, 8, 19424, 128): False, (0, B7, 8, 19425, 128): True,
+    (1, B8, 3, 262144, 64): False, (1, B8, 3, 65536, 128): True, (0, CRT, 15, 65536, 64): False,
+    (0, CRT, 15, 4096, 4096): True}
+
+
+def test_column_split_tiles(recorded):
+    """Told apart by the kernel: output off 8 bytes always takes the 64-k tiles."""
+    both = recorded([c + (1, shift) for shift in (0, 4) for c in BY_128], "split")
+    got, by_64 = both[:len(BY_128)], both[len(BY_128):]
+    assert {c: g[0] != h[0] for c, g, h in zip(BY_128, got, by_64)} == BY_128
+    for (_, _, _, R, K), g, h in zip(BY_128, got, by_64):
+        kpad = (K + 63) // 64 * 64
+        assert h[1:] == [(R + 31) // 32, kpad // 64, 256]
+        assert g == h or g[1:] == [(R + 31) // 32, (kpad + 127) // 128, 256]
+
+
+def test_row_split_blocks(recorded):
+    """Digit rows: no more threads than a row of four k each needs, and as many
+    on an SM as with the widest blocks."""
+    calls = [(f, k, n, R, K) for f, k, n in ((0, B7, 4), (0, B8, 7), (1, B8, 3))
+             for R in (5, 1000, 262144) for K in (1, 64, 128, 129, 256, 300, 512, 513, 1024, 4097)]
+    for (_, _, _, R, K), (_, gx, gy, threads) in zip(
+            calls, recorded([c + (0, 0) for c in calls], "split")):
+        kpad = (K + 63) // 64 * 64
+        assert threads == (32 if kpad <= 128 else 64 if kpad <= 256 else 128 if kpad <= 512 else 256)
+        assert gx == (kpad + 1023) // 1024 and gx * threads * 4 >= min(kpad, 1024)
+        assert gy == min(R, 152 * (2048 // threads) // gx)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("call", [(0, B7, 8, 3, 24576, 70), (0, B7, 8, 3, 24577, 70),
                                   (0, CRT, 15, 5, 24579, 33), (0, B7, 3, 2, 32769, 130),
@@ -157,3 +219,33 @@ def test_routes_agree_with_the_stages(alp, call, ta, pad, shift):
 def test_sums_agree_with_the_stages(alp, call):
     f32, kind, n, M, N, K = call
     check(alp, M, N, K, kind, n, f32=bool(f32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("f32,kind,n", [(0, B7, 4), (0, B7, 8), (0, CRT, 15), (1, B8, 3)])
+@pytest.mark.parametrize("R,K", [(19425, 65), (19424, 128), (20001, 129), (700, 1088), (700, 301),
+                                 (3, 64), (33, 1), (2500, 513)])
+@pytest.mark.parametrize("trans", [0, 1])
+def test_split_agrees_with_the_general_kernels(alp, f32, kind, n, R, K, trans):
+    """Output 8-byte aligned, and off it, where the kernels of two k per thread
+    and 64-k tiles run."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(R + K)
+    X = torch.rand((K, R) if trans else (R, K), dtype=torch.float32 if f32 else torch.float64,
+                   device="cuda", generator=g) - 0.5
+    kpad = (K + 63) // 64 * 64
+    e = torch.empty(R, dtype=torch.int32, device="cuda")
+    exps = alp.alp_emul_exponents_f32 if f32 else alp.alp_emul_exponents
+    split = alp.alp_emul_split_f32 if f32 else alp.alp_emul_split
+    exps(R, K, X, X.shape[1], trans, e)
+    bufs = [torch.full((n * R * kpad + 64,), 7.0, dtype=torch.bfloat16, device="cuda")
+            for _ in range(2)]
+    for buf, shift in zip(bufs, (0, 2)):
+        split(R, K, X, X.shape[1], trans, e, n, kind, buf[shift:], kpad)
+    torch.cuda.synchronize()
+    assert alp.alp_get_device_error() == alp.ALP_OK
+    size = n * R * kpad
+    assert torch.equal(bufs[0][:size], bufs[1][2:2 + size])
+    assert (bufs[0][size:] == 7.0).all() and (bufs[1][size + 2:] == 7.0).all()
+    assert (bufs[1][:2] == 7.0).all()
