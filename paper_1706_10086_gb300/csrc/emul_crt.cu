@@ -195,11 +195,14 @@ alp_status emul_split_crt(int64_t R, int64_t K, const T* X, int64_t ldx, int tra
     if (k < 1 || k > 60) return ALP_ERR_UNSUPPORTED;
     const CrtSplit sp{k};
     const bool vec = (reinterpret_cast<uintptr_t>(out) & 7) == 0 && kpad % 4 == 0;
-    // 128-thread blocks (4 k per thread), registers capped for 6 blocks per
+    // 128-thread blocks (4 k per thread), registers capped for 8 blocks per
     // SM (measured faster than 256 threads, than 5 blocks and than 2 k per
-    // thread at 8 blocks)
+    // thread at 8 blocks); 16 blocks per SM, and 64 once each of those would
+    // walk four rows or more (8192^2 with 15 moduli 431 -> 394 us, 4096^2 113 ->
+    // 103; 2048^2 33 and 31 either way)
     const int64_t bx = (kpad + 511) / 512;
     int64_t by = (int64_t)device_sm_count() * 16 / bx;
+    if (R >= 4 * by) by *= 4;
     by = by < 1 ? 1 : by > R ? R : by > 65535 ? 65535 : by;
     const dim3 grid4((unsigned)bx, (unsigned)by);
     int64_t blocks = (R * (kpad / 2) + 255) / 256;

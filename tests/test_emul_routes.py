@@ -200,6 +200,17 @@ def test_row_split_blocks(recorded):
         assert gy == min(R, 152 * (2048 // threads) // gx)
 
 
+def test_residue_row_blocks(recorded):
+    """16 blocks per SM, 64 where each would walk four rows or more."""
+    shapes = [(8192, 8192), (4096, 4096), (2048, 2048), (16384, 8192), (9728, 512), (9727, 512),
+              (262144, 64), (5, 64), (1, 60000)]
+    for (R, K), (_, gx, gy, threads) in zip(
+            shapes, recorded([(0, CRT, 15, R, K, 0, 0) for R, K in shapes], "split")):
+        by = 152 * 16 // gx
+        assert threads == 128 and gx == ((K + 63) // 64 * 64 + 511) // 512
+        assert gy == min(max(by * (4 if R >= 4 * by else 1), 1), R)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("call", [(0, B7, 8, 3, 24576, 70), (0, B7, 8, 3, 24577, 70),
                                   (0, CRT, 15, 5, 24579, 33), (0, B7, 3, 2, 32769, 130),
