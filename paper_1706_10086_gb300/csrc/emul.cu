@@ -266,9 +266,11 @@ __global__ void recombine_kernel(const int32_t* __restrict__ G, int64_t gplane, 
 // Four columns per thread: the S group sums of four adjacent columns arrive
 // as one 16-byte load per plane (G rows are 256-column padded, so the vector
 // never leaves the row), and C is written as two 16-byte stores when the row
-// of C is 16-byte aligned.  Needs G 16-byte aligned (the launch checks).
+// of C is 16-byte aligned.  Needs G 16-byte aligned (the launch checks).  Seven
+// sums take 70 registers if left alone, which is three blocks per SM: held to the
+// 64 of four (8 bytes spilled), 8192^2 with beta takes 515 us, not 565.
 template <int S, int B>
-__global__ void __launch_bounds__(256) recombine4_kernel(
+__global__ void __launch_bounds__(256, S == 7 ? 4 : 0) recombine4_kernel(
     const int32_t* __restrict__ G, int64_t gplane, int64_t ldg, const int32_t* __restrict__ e,
     const int32_t* __restrict__ f, int64_t M, int64_t N, double alpha, double beta,
     double* __restrict__ C, int64_t ldc) {
