@@ -1321,6 +1321,29 @@ static int fused_active_clusters() {
     return n;
 }
 
+// Products of the cluster that pair_segment deals most of `tiles` shared tiles to
+// (of a whole tile: one tile on one cluster).
+static int largest_share(int tiles, int s, bool trim, bool crt, int P) {
+    const int units = tiles * s, parts = std::min(P, units);
+    auto products = [&](int u) {   // by rank, as pair_segment orders the groups
+        const int r = u / tiles;
+        if (crt) return 1;
+        if (trim && s > 2) return r < s - 2 ? s - 1 - r : r == s - 2 ? 2 : 1;
+        return s - r;
+    };
+    int most = 0;
+    for (int c = 0; c < parts; ++c) {
+        int sum = 0;
+        for (int j = 0;; ++j) {
+            const int u = j * parts + ((j & 1) ? parts - 1 - c : c);
+            if (u >= units) break;
+            sum += products(u);
+        }
+        most = std::max(most, sum);
+    }
+    return most;
+}
+
 alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bfloat16* da,
                            const __nv_bfloat16* db, int64_t kpad, int32_t* G, int64_t ldg,
                            cudaStream_t stream, int group_m, int cluster, int digit_bits,
@@ -1407,8 +1430,12 @@ alp_status emul_slice_gemm(int64_t M, int64_t N, int64_t K, int s, const __nv_bf
     const int64_t waves = pair_tiles / P;
     // (a rest of more than nine tenths of a wave stays whole: sharing it would
     // gain less than its clusters lose by reading different slices, 526 us
-    // against 511 for 72 tiles of 8 slices)
-    const bool share = emul_tail_split_on() && 10 * (pair_tiles % P) <= 9 * P;
+    // against 511 for 72 tiles of 8 slices; so does one whose largest share is no
+    // shorter than a tile: 64 tiles of three slices 90 us whole, 99 shared)
+    const int64_t rest = pair_tiles % P;
+    const bool share = emul_tail_split_on() && rest > 0 && 10 * rest <= 9 * P &&
+                       largest_share((int)rest, s, trim, crt, (int)P) <
+                           largest_share(1, s, trim, crt, 1);
     p.n_full = (int)(share ? waves * P : pair_tiles);
     p.tail_tiles = (int)pair_tiles - p.n_full;
     p.parts = (int)std::min<int64_t>(P, (int64_t)p.tail_tiles * s);

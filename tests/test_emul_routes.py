@@ -1,9 +1,9 @@
 """Which launches an emulated GEMM call makes: its strided operands prepared in
 strips together with the others, or by a scan and a split of their own; the sums
-recombined by a kernel that starts while the products drain, or after them; and
-the tiles and blocks of the splits.  A C
-program stands in for the runtime and records the launches, so no GPU is needed;
-the GPU tests compare the routes with the stages bit for bit."""
+recombined by a kernel that starts while the products drain, or after them; the
+tiles that the products share; the tiles and blocks of the splits.  A C program
+stands in for the runtime and records the launches, so no GPU is needed; the GPU
+tests compare the routes with the stages bit for bit."""
 import subprocess
 
 import pytest
@@ -21,6 +21,7 @@ PROGRAM = r"""
 #include <stdlib.h>
 #include <string.h>
 static int word, launches, last_attrs;
+static unsigned grids[16];   /* x, by launch */
 static const void* last_kernel;
 static dim3 last_grid, last_block;
 cudaError_t cudaGetDevice(int* d) { *d = 0; return 0; }
@@ -36,7 +37,7 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaun
     return 0;
 }
 cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void** a, size_t m, cudaStream_t s) {
-    ++launches;
+    grids[launches++ % 16] = g.x;
     last_attrs = 0;
     last_kernel = f;
     last_grid = g;
@@ -51,7 +52,7 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t f, dim3 g, dim3 b, void** a, size_t 
     return cudaLaunchKernel((const void*)f, g, b, a, m, s);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** a) {
-    ++launches;
+    grids[launches++ % 16] = c->gridDim.x;
     last_attrs = (int)c->numAttrs;
     return 0;
 }
@@ -96,7 +97,7 @@ int main(int argc, char** argv) {
         const int rc =
             is32 ? f32(0, 0, M, N, K, 1, p, K, p, N, 0, p, N, n, kind, p, (size_t)1 << 60, 0)
                  : f64(0, 0, M, N, K, 1, p, K, p, N, 0, p, N, n, kind, p, (size_t)1 << 60, 0);
-        printf("%d %d %d\n", rc, launches, last_attrs);
+        printf("%d %d %d %u\n", rc, launches, last_attrs, grids[(launches - 2) % 16]);
     }
     return 0;
 }
@@ -125,7 +126,7 @@ def recorded(alp, tmp_path_factory):
 @pytest.fixture(scope="module")
 def routes(recorded):
     """calls -> (launches, whether the last one may start early) of each."""
-    return lambda calls: [(n, attrs > 0) for n, attrs in recorded(calls)]
+    return lambda calls: [(n, attrs > 0) for n, attrs, _ in recorded(calls)]
 
 
 B7, B8, CRT = lib.ALP_SLICE_BF16, lib.ALP_SLICE_BF16_B8, lib.ALP_SLICE_BF16_CRT
@@ -164,6 +165,43 @@ EARLY = {
 def test_recombination_early_or_after(routes):
     got = routes(EARLY)
     assert {c: early for c, (_, early) in zip(EARLY, got)} == EARLY
+
+
+# whether the tiles of the last wave are shared by all 76 CTA pairs of the products
+# (digit schemes; tiles of 256 x 256): not where the pair that gets most of them
+# would get a whole tile's products
+SHARED = {
+    (1, B8, 3, 2048, 2048, 512): False, (1, B8, 3, 60 * 256, 256, 512): True,
+    (1, B8, 3, 61 * 256, 256, 512): False, (1, B8, 2, 50 * 256, 256, 64): True,
+    (1, B8, 2, 51 * 256, 256, 64): False, (0, B7, 4, 65 * 256, 256, 64): True,
+    (0, B7, 4, 66 * 256, 256, 64): False, (0, B7, 8, 2048, 2048, 64): True,
+    (0, B7, 8, 68 * 256, 256, 64): True, (0, B7, 8, 69 * 256, 256, 64): False,
+    (0, lib.ALP_SLICE_BF16_B8_TRIM, 4, 66 * 256, 256, 64): False,
+    (0, lib.ALP_SLICE_BF16_B8_TRIM, 7, 64 * 256, 256, 64): True, (1, B8, 3, 256, 256, 64): True}
+
+
+def largest_share(tiles, s, trim, pairs):
+    """The units (groups of `tiles` tiles) in descending order of their products,
+    dealt out to the pairs in turns of alternating direction."""
+    groups = [s - r for r in range(s)] if not trim else list(range(s - 1, 0, -1)) + [2]
+    units = [g for g in sorted(groups, reverse=True) for _ in range(tiles)]
+    shares = [0] * min(pairs, len(units))
+    for i in range(0, len(units), len(shares)):
+        turn = units[i:i + len(shares)]
+        order = range(len(shares)) if i // len(shares) % 2 == 0 else reversed(range(len(shares)))
+        for c, u in zip(order, turn + [0] * (len(shares) - len(turn))):
+            shares[c] += u
+    return max(shares), sum(groups)
+
+
+def test_shared_tiles_pay(recorded):
+    got = recorded(SHARED)
+    for call, (_, _, grid) in zip(SHARED, got):
+        _, kind, s, M, N, _ = call
+        tiles = M // 256 * (N // 256)
+        most, whole = largest_share(tiles, s, kind == lib.ALP_SLICE_BF16_B8_TRIM, 76)
+        assert SHARED[call] == (10 * tiles <= 9 * 76 and most < whole), call
+        assert grid == 2 * (min(76, tiles * s) if SHARED[call] else tiles), call
 
 
 # (float, kind, slices, lines, K): whether the columns are split by 128-k tiles
