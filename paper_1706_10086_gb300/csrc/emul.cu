@@ -707,7 +707,7 @@ alp_status emul_gemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, T alp
     bool prepared = false;
     for (int i = 0; i < 2; ++i) {
         const auto& o = ops[i];
-        if (!o.cols || prep_in_strips<T>(o.R, K)) {
+        if (!o.cols || prep_in_strips<T>(o.R, K, auto_n)) {
             p.op[i] = {o.X, o.R, o.ldx, o.exps, o.out, o.cols, 0};
             prepared = true;
             continue;

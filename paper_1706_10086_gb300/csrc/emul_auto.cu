@@ -340,7 +340,7 @@ alp_status crt_choose_moduli(int ta, int tb, int64_t M, int64_t N, int64_t K, co
     } ops[2] = {{A, M, lda, ta, e}, {B, N, ldb, 1 - tb, f}};
     for (int i = 0; i < 2; ++i) {
         const auto& o = ops[i];
-        if (!o.cols || prep_in_strips<double>(o.R, K))
+        if (!o.cols || prep_in_strips<double>(o.R, K, true))
             p.op[i] = {o.X, o.R, o.ldx, o.exps, nullptr, o.cols, 0};
         else if ((st = emul_exponents<double>(o.R, K, o.X, o.ldx, 1, o.exps, stream)) != ALP_OK ||
                  (st = column_stats(o.X, o.R, K, o.ldx, o.exps, out + 3 * i, s1, s2, stream)) !=

@@ -396,9 +396,13 @@ inline int prep_cut(PrepParams<T>& p, int sms) {
 // strided operand): 8 digits 24576 x 64 166 and 168, 32768 x 64 204 and 201, 131072
 // x 64 748 and 678; 32768 x 192 241 and 242, 61000 x 136 434 and 424; float, 3 digits
 // 49152 x 64 94 and 96, 65536 x 64 107.5 and 106.5, 131072 x 64 206 and 187, but 131072
-// x 256 255 and 268.
+// x 256 255 and 268.  With the automatic count's statistics in the strips as well
+// (stats), clusters of eight blocks cost more than launches from a smaller size on:
+// 1024 x 1024 x 8192, A and B strided, 456 and 412, 800 x 800 x 8190 394 and 378, 700 x
+// 700 x 8190 301 and 306.
 template <typename T>
-inline bool prep_in_strips(int64_t R, int64_t K) {
+inline bool prep_in_strips(int64_t R, int64_t K, bool stats = false) {
+    if (stats && K > 4 * kPrepBlockK && R * K > int64_t(6) << 20) return false;
     const int64_t strips = (R + kPrepStrip<T> - 1) / kPrepStrip<T>;
     return K <= kPrepMaxColK &&
            R * K <= (sizeof(T) == 8 ? int64_t(1) << 23 : int64_t(1) << 25) &&

@@ -29,6 +29,12 @@ cudaError_t cudaDeviceGetAttribute(int* v, enum cudaDeviceAttr a, int d) { *v = 
 cudaError_t cudaMalloc(void** p, size_t n) { *p = &word; return 0; }
 cudaError_t cudaMemset(void* p, int v, size_t n) { return 0; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) { return 0; }
+cudaError_t cudaMemcpyAsync(void* d, const void* x, size_t n, enum cudaMemcpyKind k,
+                            cudaStream_t s) {
+    if (k == cudaMemcpyDeviceToHost) memset(d, 0, n);   /* no statistics: fewest moduli */
+    return 0;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) { return 0; }
 cudaError_t cudaDeviceSynchronize(void) { return 0; }
 cudaError_t cudaGetLastError(void) { return 0; }
 cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) { return 0; }
@@ -152,6 +158,22 @@ def test_strips_or_separate(routes):
     assert all(n in (3, 6) for n, _ in got), got
 
 
+# the automatic count (float, kind, 0, M, N, K): whether B's statistics come in strips
+AUTO = {
+    (0, CRT, 0, 64, 256, 256): True, (0, CRT, 0, 64, 700, 8190): True,
+    (0, CRT, 0, 64, 768, 8192): True, (0, CRT, 0, 64, 769, 8192): False,
+    (0, CRT, 0, 64, 1024, 8192): False, (0, CRT, 0, 64, 2048, 4096): True,
+    (0, CRT, 0, 64, 1535, 4097): True, (0, CRT, 0, 64, 1536, 4097): False,
+    (0, CRT, 0, 64, 24576, 64): True, (0, CRT, 0, 64, 24577, 64): False}
+
+
+def test_statistics_in_strips_or_separate(routes):
+    """In strips: statistics, preparation, products, reconstruction."""
+    got = routes(AUTO)
+    assert {c: n == 4 for c, (n, _) in zip(AUTO, got)} == AUTO
+    assert all(n == 4 or n >= 8 for n, _ in got), got
+
+
 # whether the kernel that makes C of the sums starts while the products drain
 EARLY = {
     (0, B7, 8, 256, 256, 256): True, (0, B7, 8, 1280, 2048, 64): True,
@@ -260,6 +282,33 @@ def test_routes_agree_with_the_stages(alp, call, ta, pad, shift):
     if ta:
         M, N = N, M
     check(alp, M, N, K, kind, n, f32=bool(f32), ta=ta, pad=pad, shift=shift)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K", [(70, 768, 8192), (70, 769, 8192), (800, 90, 8000),
+                                   (10, 24577, 40)])
+@pytest.mark.parametrize("ta,tb", [(0, 0), (1, 0), (1, 1)])
+def test_automatic_count_is_the_given_count(alp, M, N, K, ta, tb):
+    """The count and C of nslices = 0, on either route, against the same call
+    with that count given."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N + K)
+    rand = lambda r, c: torch.rand((r, c), dtype=torch.float64, device="cuda", generator=g) - 0.5
+    A = rand(K, M) if ta else rand(M, K)
+    B = rand(N, K) if tb else rand(K, N)
+    ws = alp.alp_gemm_f64_emul_workspace(M, N, K, 0, CRT)
+    work = torch.empty(ws, dtype=torch.uint8, device="cuda")
+    n, _ = alp.alp_emul_crt_choose(ta, tb, M, N, K, A, A.shape[1], B, B.shape[1], work, ws)
+    out = []
+    for count in (0, n):
+        C = torch.full((M, N), float("nan"), dtype=torch.float64, device="cuda")
+        alp.alp_gemm_f64_emul_ex(ta, tb, M, N, K, 1.0, A, A.shape[1], B, B.shape[1], 0.0, C, N,
+                                 count, CRT, work, ws)
+        out.append(C)
+    torch.cuda.synchronize()
+    assert alp.alp_get_device_error() == alp.ALP_OK
+    assert torch.equal(out[0], out[1]) and n >= 4
 
 
 @pytest.mark.gpu
