@@ -206,16 +206,21 @@ bool time_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_confi
 }
 
 // Estimated time (ms) of the register-direct kernels on the whole problem, as
-// the configs' proxy takes it: at most kDirectWaves waves of blocks and kProxyK
-// k per warp, in the cut the whole problem takes.
+// the configs' proxy takes it: at most kProxyK k per warp, in the cut the whole
+// problem takes, and kDirectWaves waves of blocks of that length (0.6 ms), so as
+// many more of shorter ones: with 16 of any length the start and the end of 16
+// short ones counted for all (232 x 15888 x 80, 20 k per warp: 0.72 ms for the 0.61
+// of the call, and a config of 0.66 was taken instead).
 constexpr int64_t kDirectWaves = 16;
 bool time_direct(int64_t M, int64_t N, int64_t K, Scratch& sc, cudaStream_t st, int runs,
                  double* est_ms) {
     const int64_t sms = device_sm_count();
     const int cut = native_direct_cut(M, N, K, (int)sms), size = std::max(cut, 1);
     const int64_t tiles = cut ? ((M + 15) / 16) * ((N + 7) / 8) : ((M + 31) / 32) * ((N + 15) / 16);
-    const int64_t Kp = std::min(K, kProxyK * (cut ? 4 * cut : 1));
-    const int64_t run_tiles = std::min(tiles, std::max<int64_t>(kDirectWaves * sms / size, 1));
+    const int64_t warps = cut ? 4 * cut : 1;   // that share a k range
+    const int64_t Kp = std::min(K, kProxyK * warps);
+    const int64_t most = kDirectWaves * (kProxyK * warps / Kp) * sms / size;
+    const int64_t run_tiles = std::min(tiles, std::max<int64_t>(most, 1));
     const size_t ba = up256((size_t)M * Kp * 8), bb = up256((size_t)Kp * N * 8);
     if (!sc.get(ba + bb + up256((size_t)M * N * 8))) return false;
     char* base = static_cast<char*>(sc.p);
@@ -292,7 +297,8 @@ void cache_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_conf
 // (64^3: 73 us with the best config, 6.2 without).  The model, which only knows
 // configs, is not asked there: a config's tiles are made of the direct kernels'
 // 32 x 16 ones, so its busiest sub-partition never has fewer MMAs (4096^3: 125.1
-// ms without a config, 125.6 with the tuned one).
+// ms without a config, 125.6 with the tuned one; 8192 x 8192 x 32, where the ends
+// of tiles count most, 4.10 and 4.07).
 bool tuned_config(int64_t M, int64_t N, int64_t K, alp_path path, alp_config* out,
                    cudaStream_t stream) {
     if (g_cached.load()) {

@@ -111,3 +111,29 @@ def test_the_sweep_records_the_direct_kernels(alp, clean, monkeypatch, tmp_path)
             ts.append(e0.elapsed_time(e1))
         assert abs(rec["direct"] / min(ts) - 1) < 0.15, (rec["direct"], ts)
     os.environ.pop("ALP_TUNE_DB", None)
+
+
+@pytest.mark.parametrize("shape", [(232, 15888, 80), (173, 9398, 79), (3000, 4000, 77),
+                                   (1000, 1000, 33), (5000, 3000, 126)])
+def test_tuned_calls_of_short_k_are_no_slower(alp, clean, shape):
+    """The sweep's proxies at short K: the call that it leaves behind is within 3 %
+    (the runs' own spread, and what a proxy may be off between near equals) of the
+    call without it.  The two are timed in turn, best of four."""
+    import torch
+    M, N, K = shape
+    call = Calls(alp, M, N, K)
+    ts = {True: [], False: []}
+    for _ in range(4):
+        for tuned in (True, False):
+            if tuned:
+                alp.alp_tune(M, N, K, alp.ALP_PATH_NATIVE, alp.ALP_TUNE_EXHAUSTIVE)
+            else:
+                alp.alp_tune_clear_cache()
+            alp.alp_gemm_f64(M, N, K, 1.0, call.A, K, call.B, N, 0.0, call.C, N)
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            alp.alp_gemm_f64(M, N, K, 1.0, call.A, K, call.B, N, 0.0, call.C, N)
+            e1.record()
+            e1.synchronize()
+            ts[tuned].append(e0.elapsed_time(e1))
+    assert min(ts[True]) <= 1.03 * min(ts[False]) + 0.002, ts
