@@ -206,11 +206,14 @@ bool time_config(int64_t M, int64_t N, int64_t K, alp_path path, const alp_confi
 }
 
 // Estimated time (ms) of the register-direct kernels on the whole problem, as
-// the configs' proxy takes it: at most kProxyK k per warp, in the cut the whole
-// problem takes, and kDirectWaves waves of blocks of that length (0.6 ms), so as
-// many more of shorter ones: with 16 of any length the start and the end of 16
-// short ones counted for all (232 x 15888 x 80, 20 k per warp: 0.72 ms for the 0.61
-// of the call, and a config of 0.66 was taken instead).
+// the configs' proxy takes it, in the cut the whole problem takes: at most kProxyK
+// k per warp (four times that where warps share a k range and exchange their sums,
+// which must not count several times over), and kDirectWaves waves of blocks, twice
+// as many of clusters, whose last ones end less evenly (629 x 937 x 11136, clusters
+// of four: 13.2 ms by 16 waves, 12.8 by 32, 12.7 the call), and more where they are
+// shorter than kProxyK k (0.6 ms).  With 16 waves of any length the start and the
+// end of the launch counted for all: 232 x 15888 x 80, 20 k per warp, 0.72 ms for
+// the 0.61 of the call, and a config of 0.66 was taken instead.
 constexpr int64_t kDirectWaves = 16;
 bool time_direct(int64_t M, int64_t N, int64_t K, Scratch& sc, cudaStream_t st, int runs,
                  double* est_ms) {
@@ -218,8 +221,9 @@ bool time_direct(int64_t M, int64_t N, int64_t K, Scratch& sc, cudaStream_t st, 
     const int cut = native_direct_cut(M, N, K, (int)sms), size = std::max(cut, 1);
     const int64_t tiles = cut ? ((M + 15) / 16) * ((N + 7) / 8) : ((M + 31) / 32) * ((N + 15) / 16);
     const int64_t warps = cut ? 4 * cut : 1;   // that share a k range
-    const int64_t Kp = std::min(K, kProxyK * warps);
-    const int64_t most = kDirectWaves * (kProxyK * warps / Kp) * sms / size;
+    const int64_t Kp = std::min(K, (cut ? 4 : 1) * kProxyK * warps);
+    const int64_t least = cut > 1 ? 2 * kDirectWaves : kDirectWaves;
+    const int64_t most = std::max(kDirectWaves * kProxyK * warps, least * Kp) * sms / (Kp * size);
     const int64_t run_tiles = std::min(tiles, std::max<int64_t>(most, 1));
     const size_t ba = up256((size_t)M * Kp * 8), bb = up256((size_t)Kp * N * 8);
     if (!sc.get(ba + bb + up256((size_t)M * N * 8))) return false;
